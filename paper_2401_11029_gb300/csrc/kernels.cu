@@ -2103,6 +2103,91 @@ __global__ void k_fill_u64(unsigned long long *p, unsigned long long count,
         p[s] = v;
 }
 
+// Empty every slot's pair set in one launch.  Bound by the write bandwidth
+// for large sets and by the launch for small ones: a fill per set cost 4 us
+// each on the host (1539 sets of the 100k-vertex value-flow graph: with this
+// and k_clear_rows its reset-solve-read pass went from 14.7 to 8.6 ms, the
+// field-sensitive alias pass from 13.7 to 12.2 ms).  The sets are cut into chunks of CLEAR_CHUNK entries, numbered over
+// all sets; every block finds the sets of its chunks itself, from a scan of
+// CLEAR_SEG slots' chunk counts at a time, so the host prepares no table.
+constexpr uint32_t CLEAR_CHUNK = 4096;   // 32 KB: 128 bytes a thread
+constexpr uint32_t CLEAR_SEG = 2048;     // slots scanned at a time, 8 a thread
+
+__global__ void __launch_bounds__(256) k_clear_sets(SlotTab S, uint32_t n_slots) {
+    __shared__ unsigned long long first[CLEAR_SEG + 1];   // first chunk of each slot
+    __shared__ unsigned long long sh[16];
+    const uint4 empty = make_uint4(EMPTY32, EMPTY32, EMPTY32, EMPTY32);
+    unsigned long long done = 0;                          // chunks of the segments before
+    for (uint32_t s0 = 0; s0 < n_slots; s0 += CLEAR_SEG) {
+        const uint32_t ns = min(CLEAR_SEG, n_slots - s0);
+        unsigned long long c[8], sum = 0, total;
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const uint32_t s = threadIdx.x * 8 + q;
+            c[q] = s < ns ? S.hmask[s0 + s] / CLEAR_CHUNK + 1 : 0;
+            sum += c[q];
+        }
+        unsigned long long at = block_excl_scan256(sum, sh, total);
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            first[threadIdx.x * 8 + q] = at;
+            at += c[q];
+        }
+        if (threadIdx.x == 0) first[CLEAR_SEG] = total;
+        __syncthreads();
+        // the chunks take the blocks in turn over all segments
+        unsigned long long k = (blockIdx.x + gridDim.x - done % gridDim.x) % gridDim.x;
+        uint32_t lo = 0;
+        for (; k < total; k += gridDim.x) {
+            uint32_t hi = ns;                             // first[lo] <= k < first[hi]
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (first[mid] <= k) lo = mid;
+                else hi = mid;
+            }
+            const unsigned long long e0 = (k - first[lo]) * CLEAR_CHUNK;
+            const unsigned long long cap = S.hmask[s0 + lo] + 1;
+            const uint32_t n2 = (uint32_t)(min((unsigned long long)CLEAR_CHUNK, cap - e0) / 2);
+            uint4 *p = reinterpret_cast<uint4 *>(S.htab[s0 + lo] + e0);
+            for (uint32_t q = threadIdx.x; q < n2; q += 256) p[q] = empty;
+        }
+        done += total;
+        __syncthreads();
+    }
+}
+
+// Back to empty rows before a solve is repeated: the descriptors and delta
+// counts of the rows whose occupancy bit is set (all others are zero), then
+// the bits.  A lane per vertex and a turn per bit, so that a non-terminal
+// with a row at every vertex is written like a plain fill, and one with few
+// rows costs the read of its occupancy words only (500k points-to graph, 644
+// non-terminals: 15.5 GB of descriptors and counts, of which few are in use;
+// its pass went from 148.4 to 144.6 ms).
+__global__ void __launch_bounds__(256) k_clear_rows(uint4 *desc, uint2 *dn, uint32_t *occ,
+                                                    uint32_t n, uint32_t occ_w) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t per_o = (n + 31) / 32;                 // warps' vertex blocks per orientation
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    for (uint32_t t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < 2 * per_o;
+         t += warps) {
+        const uint32_t o = t >= per_o;
+        const uint32_t v = (t - o * per_o) * 32 + lane;
+        uint32_t *ow = occ + ((size_t)o * n + v) * occ_w;
+        for (uint32_t w = 0; w < occ_w; w++) {
+            const uint32_t bits = v < n ? ow[w] : 0u;
+            for (uint32_t any = __reduce_or_sync(FULL_MASK, bits); any; any &= any - 1) {
+                const uint32_t b = __ffs(any) - 1;
+                if ((bits >> b) & 1u) {
+                    const size_t r = ((size_t)(32 * w + b) * 2 + o) * n + v;
+                    desc[r] = make_uint4(0, 0, 0, 0);
+                    dn[r] = make_uint2(0, 0);
+                }
+            }
+            if (bits) ow[w] = 0;
+        }
+    }
+}
+
 // Split a batch's touched list back into per-instance lists with local
 // slot ids: first count the entries of every instance, then scatter.
 // (Lanes of one instance add their entries with one atomic per warp: the
@@ -2774,6 +2859,19 @@ void launch_fill_u64(unsigned long long *p, unsigned long long count, unsigned l
                      int sms, cudaStream_t st) {
     if (!count) return;
     k_fill_u64<<<grid_for(count, 256, sms, 8), 256, 0, st>>>(p, count, v);
+}
+
+void launch_clear_sets(const SlotTab &S, uint32_t n_slots, unsigned long long entries, int sms,
+                       cudaStream_t st) {
+    if (!n_slots) return;
+    // at least a chunk per set, and no more blocks than chunks
+    k_clear_sets<<<grid_for(entries / CLEAR_CHUNK + n_slots, 1, sms, 8), 256, 0, st>>>(S, n_slots);
+}
+
+void launch_clear_rows(uint4 *desc, uint2 *dn, uint32_t *occ, uint32_t n, uint32_t occ_w, int sms,
+                       cudaStream_t st) {
+    if (!n) return;
+    k_clear_rows<<<grid_for((n + 31) / 32 * 2, 8, sms, 8), 256, 0, st>>>(desc, dn, occ, n, occ_w);
 }
 
 void launch_remap_touched(const uint2 *in, unsigned long long n, uint32_t slot_base,

@@ -253,6 +253,14 @@ void launch_witness_lookup(const unsigned long long *tab, const uint2 *val,
                            cudaStream_t st);
 void launch_fill_u64(unsigned long long *p, unsigned long long count, unsigned long long v,
                      int sms, cudaStream_t st);
+// Empty the pair sets of every slot (entries: the sum of their capacities,
+// each a power of two of at least two entries).
+void launch_clear_sets(const SlotTab &S, uint32_t n_slots, unsigned long long entries, int sms,
+                       cudaStream_t st);
+// Zero the descriptors and delta counts of every row with its occupancy bit
+// set (the only ones that are not zero), and the occupancy bits.
+void launch_clear_rows(uint4 *desc, uint2 *dn, uint32_t *occ, uint32_t n, uint32_t occ_w, int sms,
+                       cudaStream_t st);
 void launch_remap_touched(const uint2 *in, unsigned long long n, uint32_t slot_base,
                           uint2 *out, cudaStream_t st);
 // Per-instance split of a batch touched list (counts, then scatter with

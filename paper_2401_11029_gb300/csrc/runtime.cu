@@ -119,6 +119,7 @@ struct cflr_ctx {
     uint2 *dn = nullptr;                // n_nt * 2 * n delta counts / append cursors
     uint32_t *occ = nullptr;            // occupancy bits: 2 * n * occ_w words
     uint32_t occ_w = 0;
+    bool rows_set = false;              // desc, dn and occ hold a (possibly empty) graph's rows
     uint32_t *pool = nullptr;
     uint64_t pool_cap = 0;
     uint64_t pool_top = 0;              // host mirror between solves
@@ -250,6 +251,7 @@ struct cflr_ctx {
         if (occ) dfree(occ, (size_t)2 * n * occ_w * 4);
         occ = nullptr;
         occ_w = 0;
+        rows_set = false;
         if (pool) dfree(pool, pool_cap * 4);
         pool = nullptr;
         pool_cap = pool_top = 0;
@@ -1493,17 +1495,25 @@ void reset_matrices(cflr_ctx *c) {
     const uint32_t nt = (uint32_t)g.nts.size(), nterm = (uint32_t)g.terms.size();
     const uint32_t n = c->n;
     cudaStream_t st = c->stream;
-    ck(cudaMemsetAsync(c->desc, 0, (size_t)nt * 2 * n * sizeof(uint4), st), "memset");
-    ck(cudaMemsetAsync(c->dn, 0, (size_t)nt * 2 * n * sizeof(uint2), st), "memset");
-    ck(cudaMemsetAsync(c->occ, 0, (size_t)2 * n * c->occ_w * 4, st), "memset");
-    for (uint32_t A = 0; A < nt; A++)
-        ck(cudaMemsetAsync(c->htab[A], 0xFF, c->hcap[A] * 8, st), "memset");
+    if (c->rows_set) {
+        launch_clear_rows(c->desc, c->dn, c->occ, n, c->occ_w, c->sms, st);
+        ck(cudaGetLastError(), "clear rows");
+    } else {
+        ck(cudaMemsetAsync(c->desc, 0, (size_t)nt * 2 * n * sizeof(uint4), st), "memset");
+        ck(cudaMemsetAsync(c->dn, 0, (size_t)nt * 2 * n * sizeof(uint2), st), "memset");
+        ck(cudaMemsetAsync(c->occ, 0, (size_t)2 * n * c->occ_w * 4, st), "memset");
+        c->rows_set = true;
+    }
     c->pool_top = 0;
     std::fill(c->nnz.begin(), c->nnz.end(), 0);
     c->iterations = 0;
     c->touched_n = 0;
     Runner &r = runner_of(c);
     r.bind({c});
+    uint64_t entries = 0;
+    for (uint64_t h : c->hcap) entries += h;
+    launch_clear_sets(r.slots(), r.n_slots, entries, c->sms, st);
+    ck(cudaGetLastError(), "clear pair sets");
     r.init_buffers(std::max<uint64_t>(c->n_init, 1), 0);
     if (r.cand_cap < c->n_init) {      // the initial pairs are counted exactly
         r.size_cand(c->n_init);
