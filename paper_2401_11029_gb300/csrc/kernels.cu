@@ -2493,7 +2493,91 @@ __device__ __forceinline__ uint32_t unit_rows(const ExtractList &L, unsigned lon
     return lo;
 }
 
-// Pairs of every unit (a warp per unit, its lanes over the rows).
+// Which rows of the listed non-terminals are non-empty, in caller order: bit
+// i % 32 of map[k * row_words(n) + i / 32] for row i of the k-th listed one.  A
+// warp takes 32 rows, reads their vertices' occupancy words and turns the bit
+// of every listed non-terminal into a word by a ballot.  The read-out then
+// reads the descriptors of non-empty rows only: the 386 named non-terminals of
+// the 500k points-to graph have 193 M rows of which few hold pairs, and two
+// passes over their descriptors were most of its 10.7 ms (now 4.2 ms).
+__device__ __forceinline__ uint32_t row_words(uint32_t n) { return (n + 31) / 32; }
+
+__global__ void __launch_bounds__(256) k_row_map(ExtractList L, const uint32_t *occ,
+                                                 uint32_t occ_w, uint32_t *map) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t words = row_words(L.n);
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    for (uint32_t t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < words; t += warps) {
+        const uint32_t i = t * 32 + lane;
+        const uint32_t *ov = occ + (size_t)(i < L.n ? stored_row(L.perm, i) : 0) * occ_w;
+        uint32_t have = EMPTY32, bits = 0, mine = 0;      // `bits`: occupancy word `have`
+        for (uint32_t k = 0; k < L.count; k++) {
+            const uint32_t x = L.nts[k];
+            if (x >> 5 != have) {                         // uniform
+                have = x >> 5;
+                bits = i < L.n ? ov[have] : 0u;
+            }
+            const uint32_t rows = __ballot_sync(FULL_MASK, (bits >> (x & 31)) & 1u);
+            if ((k & 31) == (uint32_t)lane) mine = rows;
+            // 32 entries' words are written together, one a lane
+            if ((k & 31) == 31 || k + 1 == L.count) {
+                const uint32_t k0 = k & ~31u;
+                if (k0 + lane <= k) map[(size_t)(k0 + lane) * words + t] = mine;
+            }
+        }
+    }
+}
+
+// Non-empty rows among rb + 32 * lane .. rb + 32 * lane + 31 (warp-collective),
+// as bits, rows from r1 on left out; dk: the non-terminal's row descriptors,
+// read when there is no map (no room for one under the memory budget).
+__device__ __forceinline__ uint32_t row_bits(const ExtractList &L, uint32_t k, const uint4 *dk,
+                                             uint32_t rb, uint32_t r1, int lane) {
+    const uint32_t r = rb + 32 * lane;
+    uint32_t bits = 0;
+    if (L.map) {
+        if (r < r1) {
+            const uint32_t *mk = L.map + (size_t)k * row_words(L.n);
+            const uint32_t w = r >> 5, sh = r & 31;
+            bits = mk[w] >> sh;
+            if (sh && w + 1 < row_words(L.n)) bits |= mk[w + 1] << (32 - sh);
+        }
+    } else {
+        for (uint32_t j = 0; j < 32 && rb + 32 * j < r1; j++) {
+            const uint32_t i = rb + 32 * j + lane;
+            const uint32_t m =
+                __ballot_sync(FULL_MASK, i < r1 && dk[stored_row(L.perm, i)].y != 0);
+            if (j == (uint32_t)lane) bits = m;
+        }
+    }
+    if (r >= r1) return 0;
+    return r1 - r < 32 ? bits & ((1u << (r1 - r)) - 1) : bits;
+}
+
+// Pairs of a row of few tiles, by one lane (16-byte loads of tile pairs; a
+// tile section holds an even number of tiles).
+constexpr uint32_t LANE_TILES = 16;
+
+__device__ __forceinline__ uint32_t lane_row_len(const uint32_t *tl, uint32_t nt) {
+    uint32_t c = 0;
+#pragma unroll 4
+    for (uint32_t q = 0; q < nt; q += 2) {
+        const uint4 t = *reinterpret_cast<const uint4 *>(tl + 2 * q);
+        c += __popc(t.y) + (q + 1 < nt ? __popc(t.w) : 0);
+    }
+    return c;
+}
+
+// Pairs of a row by the whole warp (the sum in every lane).
+__device__ __forceinline__ uint32_t warp_row_len(const uint32_t *tl, uint32_t nt, int lane) {
+    uint32_t c = 0;
+    for (uint32_t q = lane; q < nt; q += 32) c += __popc(tl[2 * q + 1]);
+    return __reduce_add_sync(FULL_MASK, c);
+}
+
+// Pairs of every unit (a warp per unit): 1024 rows' bits at once, then the
+// non-empty rows 32 at a time, rows of up to LANE_TILES tiles by a lane each,
+// longer ones by the warp.
 __global__ void __launch_bounds__(256) k_unit_lengths(ExtractList L,
                                                       unsigned long long *unit_len) {
     const int lane = threadIdx.x & 31;
@@ -2502,23 +2586,37 @@ __global__ void __launch_bounds__(256) k_unit_lengths(ExtractList L,
                                 (threadIdx.x >> 5);
          u < L.units; u += warps) {
         uint32_t r0, r1;
-        const uint4 *dk = list_desc(L, unit_rows(L, u, r0, r1));
-        unsigned long long len = 0;
-        for (uint32_t i = r0 + lane; i < r1; i += 32) {
-            const uint4 d = dk[stored_row(L.perm, i)];
-            const uint32_t *tl = L.pool + d.x;
-            uint32_t c32 = 0;
-            for (uint32_t q = 0; q < d.y; q++) c32 += __popc(tl[2 * q + 1]);
-            len += c32;
+        const uint32_t k = unit_rows(L, u, r0, r1);
+        const uint4 *dk = list_desc(L, k);
+        unsigned long long len = 0;                     // of this lane
+        for (uint32_t rb = r0; rb < r1; rb += 1024) {
+            const uint32_t bits = row_bits(L, k, dk, rb, r1, lane);
+            for (unsigned nz = __ballot_sync(FULL_MASK, bits != 0); nz; nz &= nz - 1) {
+                const int j = __ffs(nz) - 1;
+                const uint32_t w = __shfl_sync(FULL_MASK, bits, j);
+                uint4 d = make_uint4(0, 0, 0, 0);
+                if ((w >> lane) & 1u) d = dk[stored_row(L.perm, rb + 32 * j + lane)];
+                if (d.y <= LANE_TILES) len += lane_row_len(L.pool + d.x, d.y);
+                for (unsigned m = __ballot_sync(FULL_MASK, d.y > LANE_TILES); m; m &= m - 1) {
+                    const int l = __ffs(m) - 1;
+                    const uint32_t c = warp_row_len(L.pool + __shfl_sync(FULL_MASK, d.x, l),
+                                                    __shfl_sync(FULL_MASK, d.y, l), lane);
+                    if (lane == l) len += c;
+                }
+            }
         }
         len = warp_sum64(len);
         if (lane == 0) unit_len[u] = len;
     }
 }
 
-// The rows of every unit (a warp per unit, units claimed from cursor[1]):
-// the lanes read 32 rows' descriptors at once and the warp takes the
-// non-empty ones in order.  cursor[0] counts the listed long rows.
+// The rows of every unit (a warp per unit, units claimed from cursor[1]), the
+// non-empty ones in order, 32 rows' descriptors at a time.  Neighbouring rows
+// of few pairs are written together: as many as hold 32 pairs go through one
+// sort of (row, column) keys in registers.  One such row at a time left the
+// warp waiting on its loads for a few pairs (64 Dyck-3 read-outs of 1k to
+// 50k vertices with rows of a few pairs: 20.9 ms, now 7.3).  cursor[0] counts the
+// listed long rows.
 __global__ void __launch_bounds__(256) k_extract_units(ExtractList L,
                                                        const unsigned long long *unit_off,
                                                        uint32_t *out_src, uint32_t *out_dst,
@@ -2537,35 +2635,106 @@ __global__ void __launch_bounds__(256) k_extract_units(ExtractList L,
         const uint32_t k = unit_rows(L, u, r0, r1);
         const uint4 *dk = list_desc(L, k);
         unsigned long long o = unit_off[u];     // absolute; written at o - L.base
-        for (uint32_t rb = r0; rb < r1; rb += 32) {
-            const uint32_t i = rb + lane;
-            const uint4 d = i < r1 ? dk[stored_row(L.perm, i)] : make_uint4(0, 0, 0, 0);
-            for (unsigned m = __ballot_sync(FULL_MASK, d.y != 0); m; m &= m - 1) {
-                const int l = __ffs(m) - 1;
-                const uint32_t nt = __shfl_sync(FULL_MASK, d.y, l);
-                const uint32_t *tl = L.pool + __shfl_sync(FULL_MASK, d.x, l);
-                uint32_t len = 0;
-                for (uint32_t q = lane; q < nt; q += 32) len += __popc(tl[2 * q + 1]);
-                len = __reduce_add_sync(FULL_MASK, len);
-                if (len == 0) continue;
-                if (o + len > L.limit) {
-                    // more pairs than the pair sets count: nothing is written
-                    // past the caller's arrays
-                    if (lane == 0) atomicOr(err, 2u);
-                } else if (len > EXTRACT_WARP_MAX) {
-                    if (lane == 0) {
-                        const unsigned long long pos = atomicAdd(&cursor[0], 1ull);
-                        const unsigned long long ro = o - L.base;
-                        if (pos < big_cap)
-                            big[pos] = make_uint4(rb + l, k, (uint32_t)ro, (uint32_t)(ro >> 32));
-                        else
-                            atomicOr(err, 1u);
-                    }
-                } else {
-                    extract_row_warp(tl, nt, len, rb + l, L.iperm, o - L.base, out_src, out_dst,
-                                     s, lane);
+        // row `src` (tiles tl, nt of them, len pairs) by the whole warp
+        auto one_row = [&](uint32_t src, const uint32_t *tl, uint32_t nt, uint32_t len) {
+            if (o + len > L.limit) {
+                // more pairs than the pair sets count: nothing is written
+                // past the caller's arrays
+                if (lane == 0) atomicOr(err, 2u);
+            } else if (len > EXTRACT_WARP_MAX) {
+                if (lane == 0) {
+                    const unsigned long long pos = atomicAdd(&cursor[0], 1ull);
+                    const unsigned long long ro = o - L.base;
+                    if (pos < big_cap)
+                        big[pos] = make_uint4(src, k, (uint32_t)ro, (uint32_t)(ro >> 32));
+                    else
+                        atomicOr(err, 1u);
                 }
-                o += len;
+            } else if (len) {
+                extract_row_warp(tl, nt, len, src, L.iperm, o - L.base, out_src, out_dst, s,
+                                 lane);
+            }
+            o += len;
+        };
+        for (uint32_t rb = r0; rb < r1; rb += 1024) {
+            const uint32_t bits = row_bits(L, k, dk, rb, r1, lane);
+            for (unsigned nz = __ballot_sync(FULL_MASK, bits != 0); nz; nz &= nz - 1) {
+                const int j = __ffs(nz) - 1;
+                const uint32_t row0 = rb + 32 * j;
+                uint32_t m = __shfl_sync(FULL_MASK, bits, j);
+                uint4 d = make_uint4(0, 0, 0, 0);
+                if ((m >> lane) & 1u) d = dk[stored_row(L.perm, row0 + lane)];
+                const uint32_t *mtl = L.pool + d.x;
+                // rows of few tiles: their pairs, scanned over the lanes
+                const bool few = d.y <= LANE_TILES;
+                const uint32_t mlen = few ? lane_row_len(mtl, d.y) : 0u;
+                const uint32_t incl = warp_incl_scan(mlen, lane);
+                const unsigned lng = __ballot_sync(FULL_MASK, !few);
+                while (m) {
+                    const int l = __ffs(m) - 1;
+                    if ((lng >> l) & 1u) {
+                        const uint32_t nt = __shfl_sync(FULL_MASK, d.y, l);
+                        const uint32_t *tl = L.pool + __shfl_sync(FULL_MASK, d.x, l);
+                        one_row(row0 + l, tl, nt, warp_row_len(tl, nt, lane));
+                        m &= m - 1;
+                        continue;
+                    }
+                    // the rows from l up to the next long one, as far as they
+                    // hold at most 32 pairs together
+                    const uint32_t before = __shfl_sync(FULL_MASK, incl - mlen, l);
+                    const unsigned later = lng & ~((2u << l) - 1);
+                    const int stop = later ? __ffs(later) - 1 : 32;
+                    const bool in = lane >= l && lane < stop && incl - before <= 32;
+                    const unsigned take = __ballot_sync(FULL_MASK, in) & m;
+                    if (!take) {               // row l alone holds more
+                        one_row(row0 + l, L.pool + __shfl_sync(FULL_MASK, d.x, l),
+                                __shfl_sync(FULL_MASK, d.y, l), __shfl_sync(FULL_MASK, mlen, l));
+                        m &= m - 1;
+                        continue;
+                    }
+                    m &= ~take;
+                    const uint32_t cnt =
+                        __shfl_sync(FULL_MASK, incl, 31 - __clz(take)) - before;
+                    if (o + cnt > L.limit) {
+                        if (lane == 0) atomicOr(err, 2u);
+                        o += cnt;
+                        continue;
+                    }
+                    if ((take >> lane) & 1u) {
+                        uint32_t pos = incl - mlen - before;
+                        for (uint32_t q = 0; q < d.y; q++) {
+                            const uint2 t = *reinterpret_cast<const uint2 *>(mtl + 2 * q);
+                            for (uint32_t b = t.y; b; b &= b - 1, pos++) {
+                                s[pos] = t.x * 32 + (__ffs(b) - 1);
+                                s[32 + pos] = lane;
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    unsigned long long key = ~0ull;
+                    if ((uint32_t)lane < cnt) {
+                        const uint32_t v = s[lane];
+                        key = ((unsigned long long)s[32 + lane] << 32) | (L.iperm ? L.iperm[v] : v);
+                    }
+                    // only rows of several pairs need the sort
+                    if (__any_sync(FULL_MASK, ((take >> lane) & 1u) && mlen > 1)) {
+#pragma unroll
+                        for (uint32_t kk = 2; kk <= 32; kk <<= 1) {
+#pragma unroll
+                            for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
+                                const unsigned long long y = __shfl_xor_sync(FULL_MASK, key, jj);
+                                const bool up = (lane & kk) == 0, lower = (lane & jj) == 0;
+                                key = (lower == up) ? min(key, y) : max(key, y);
+                            }
+                        }
+                    }
+                    if ((uint32_t)lane < cnt) {
+                        out_src[o - L.base + lane] = row0 + (uint32_t)(key >> 32);
+                        out_dst[o - L.base + lane] = (uint32_t)key;
+                    }
+                    o += cnt;
+                    __syncwarp();
+                }
             }
         }
     }
@@ -2657,10 +2826,41 @@ void launch_exclusive_scan(const uint32_t *in, uint32_t n, unsigned long long *o
     k_scan_down<uint32_t><<<nb, 256, 0, st>>>(in, n, bsum, out);
 }
 
+// The same in place for up to SCAN_ONE values by one CTA (a launch instead of
+// three: on a small read-out the launches are most of the time).
+constexpr unsigned long long SCAN_ONE = 8192;
+
+__global__ void __launch_bounds__(256) k_scan_one(unsigned long long *v, uint32_t n,
+                                                  unsigned long long *grand) {
+    __shared__ unsigned long long sh[16];
+    unsigned long long carry = 0;
+    for (uint32_t b0 = 0; b0 < n; b0 += SCAN_TILE) {
+        const uint32_t i = b0 + threadIdx.x * 4;
+        unsigned long long x[4], sum = 0, total;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            x[q] = i + q < n ? v[i + q] : 0;
+            sum += x[q];
+        }
+        unsigned long long acc = carry + block_excl_scan256(sum, sh, total);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (i + q < n) v[i + q] = acc;
+            acc += x[q];
+        }
+        carry += total;
+    }
+    if (threadIdx.x == 0 && grand) *grand = carry;
+}
+
 void launch_exclusive_scan64(unsigned long long *in_out, unsigned long long n,
                              unsigned long long *bsum, unsigned long long *grand,
                              cudaStream_t st) {
     if (!n) return;
+    if (n <= SCAN_ONE) {
+        k_scan_one<<<1, 256, 0, st>>>(in_out, (uint32_t)n, grand);
+        return;
+    }
     const unsigned long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     k_scan_reduce<unsigned long long><<<(unsigned)nb, 256, 0, st>>>(in_out, n, bsum);
     k_scan_top<<<1, 256, 0, st>>>(bsum, (uint32_t)nb, grand);
@@ -2911,7 +3111,9 @@ void extract_plan(uint32_t count, uint32_t n, const uint64_t *pairs, int sms,
     const unsigned long long target = (unsigned long long)sms * 64 * 8;   // resident warps x 8
     unsigned long long total = 0;
     for (uint32_t k = 0; k < count; k++) total += pairs[k];
-    const unsigned long long share = std::max<unsigned long long>(256, total / target);
+    // at least 64 pairs a unit: a small result then still has units for many
+    // warps, whose waits on their rows' loads overlap
+    const unsigned long long share = std::max<unsigned long long>(64, total / target);
     unit_first[0] = 0;
     for (uint32_t k = 0; k < count; k++) {
         unsigned long long u = std::max<unsigned long long>(((unsigned long long)n + 4095) / 4096,
@@ -2930,6 +3132,12 @@ void launch_extract_count(const ExtractList &L, unsigned long long *units,
     if (!nu || !L.n) return;
     k_unit_lengths<<<grid_for(nu, 8, sms, 8), 256, 0, st>>>(L, units);
     launch_exclusive_scan64(units, nu, bsum, total, st);
+}
+
+void launch_row_map(const ExtractList &L, const uint32_t *occ, uint32_t occ_w, uint32_t *map,
+                    int sms, cudaStream_t st) {
+    if (!L.count || !L.n) return;
+    k_row_map<<<grid_for((L.n + 31) / 32, 8, sms, 8), 256, 0, st>>>(L, occ, occ_w, map);
 }
 
 void launch_extract_write(const ExtractList &L, uint32_t *out_src, uint32_t *out_dst,

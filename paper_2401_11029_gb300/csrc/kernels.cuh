@@ -309,6 +309,8 @@ struct ExtractList {
     const uint4 *desc;                  // every non-terminal's descriptors, 2 n each
     const uint32_t *pool;
     const uint32_t *perm, *iperm;
+    const uint32_t *map;                // non-empty rows (launch_row_map), or null: the
+                                        // descriptors tell
     const uint32_t *nts;                // listed non-terminal ids (count)
     const uint32_t *rows_per;           // rows per unit of each (count)
     const unsigned long long *unit_first;   // first unit of each (count + 1)
@@ -317,6 +319,11 @@ struct ExtractList {
     unsigned long long u_begin, u_end;  // units written by launch_extract_write
     unsigned long long base, limit;     // output positions: written at o - base, o < limit
 };
+// map[k * ceil(n / 32) + i / 32] (count * ceil(n / 32) words): bit i % 32 set
+// when row i (caller order) of the k-th listed non-terminal is non-empty,
+// from the row form's occupancy bits.
+void launch_row_map(const ExtractList &L, const uint32_t *occ, uint32_t occ_w, uint32_t *map,
+                    int sms, cudaStream_t st);
 // Units of listed non-terminals with pairs[k] pairs each, n rows: about
 // eight units per resident warp in all, each with a like share of the pairs
 // and at most 4096 rows.  Fills rows_per and unit_first (count + 1).

@@ -144,12 +144,12 @@ struct cflr_ctx {
     // extraction scratch
     // (listed non-terminal ids, unit offsets and their block sums, counters
     // and group totals, long-row list, row bitmaps)
-    uint32_t *x_nts = nullptr, *x_bm = nullptr;
+    uint32_t *x_nts = nullptr, *x_bm = nullptr, *x_map = nullptr;
     unsigned long long *x_first = nullptr, *x_unit = nullptr, *x_bsum = nullptr,
                        *x_misc = nullptr;
     uint4 *x_bigl = nullptr;
-    size_t x_nts_n = 0, x_bm_n = 0, x_first_n = 0, x_unit_n = 0, x_bsum_n = 0, x_misc_n = 0,
-           x_bigl_n = 0;
+    size_t x_nts_n = 0, x_bm_n = 0, x_map_n = 0, x_first_n = 0, x_unit_n = 0, x_bsum_n = 0,
+           x_misc_n = 0, x_bigl_n = 0;
     uint32_t *x_src = nullptr, *x_dst = nullptr;
     uint64_t x_out_cap = 0;
     // accounting
@@ -215,6 +215,7 @@ struct cflr_ctx {
         drop(x_nts, x_nts_n);
         drop(x_first, x_first_n);
         drop(x_bm, x_bm_n);
+        drop(x_map, x_map_n);
         drop(x_unit, x_unit_n);
         drop(x_bsum, x_bsum_n);
         drop(x_misc, x_misc_n);
@@ -1896,6 +1897,24 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
     L.n = n;
     L.count = E;
     L.units = U;
+    // the map of non-empty rows; under a memory budget only where it leaves
+    // room for everything else the call may need (staging and lists), and
+    // only for the call
+    const size_t map_n = (size_t)E * (((size_t)n + 31) / 32);
+    const uint64_t budget = c->cfg.mem_budget_bytes;
+    struct MapGuard {
+        cflr_ctx *c;
+        bool keep;
+        ~MapGuard() {
+            if (!keep) c->drop(c->x_map, c->x_map_n);
+        }
+    } map_guard{c, budget == 0};
+    if (!budget || c->bytes_now + 4 * map_n + 17 * total + (1 << 16) <= budget) {
+        c->scratch(c->x_map, c->x_map_n, map_n);
+        launch_row_map(L, c->occ, c->occ_w, c->x_map, c->sms, st);
+        ck(cudaGetLastError(), "row map");
+        L.map = c->x_map;
+    }
     launch_extract_count(L, c->x_unit, c->x_bsum, c->x_misc + 3, c->sms, st);
     ck(cudaGetLastError(), "extract count");
     unsigned long long misc[4] = {0, 0, 0, 0};
