@@ -316,64 +316,50 @@ __device__ __forceinline__ Work gathered_work(const SlotTab &S, uint32_t g, uint
 // The same for a family on its shared operand's delta (optimisation 4): the
 // members reference the consecutive slots g0 .. g0+F-1, whose occupancy bits
 // are consecutive, so a few words per entry say which members have a row.
+// The (entry, word) items, numbered entry * words + word, are shared out: a
+// family of several words keeps a warp's lanes busy on a short delta too.
+// The members' descriptor arrays follow one another (the slots of one
+// instance are consecutive, 2n descriptors each), so member i's row k of
+// orientation o is S.desc[g0][(2i + o) n + k].
 __device__ __forceinline__ Work family_work(const SlotTab &S, uint32_t g0, uint32_t F, uint32_t o,
                                             uint32_t n, const uint32_t *pool, uint32_t dstart,
                                             uint32_t d, uint32_t q0, uint32_t qstep,
                                             unsigned *err) {
     const uint32_t *oc = S.occ[g0];
-    const uint32_t ow = S.occ_w[g0], lx0 = S.local[g0];
+    const uint4 *dg = S.desc[g0] + (size_t)o * n;
+    const uint32_t ow = S.occ_w[g0], lx0 = S.local[g0], lx1 = lx0 + F;
+    const uint32_t w0 = lx0 >> 5, words = ((lx1 - 1) >> 5) - w0 + 1;
+    const unsigned long long items = (unsigned long long)d * words;
     Work w{0, 0};
-    if (qstep == 32 && F >= 16 && d <= 32) {
-        // a whole warp on a short delta (lane q0 of 32): the lanes take the
-        // members of each entry in turn, so the members' descriptors load
-        // together instead of one after another on the entry's lane
-        for (uint32_t q = 0; q < d; q++) {
-            const uint32_t k = pool[dstart + q];
-            if (!CFLR_CHECK(k < n, err)) continue;
-            const uint32_t *ok = oc + ((size_t)o * n + k) * ow;
-            for (uint32_t i = q0; i < F; i += 32) {
-                const uint32_t x = lx0 + i;
-                if ((ok[x >> 5] >> (x & 31)) & 1u) {
-                    const uint4 gd = S.desc[g0 + i][(size_t)o * n + k];
-                    const uint32_t nt = gd.y - (o ? (gd.w & DLAST_MASK) : 0u);
-                    w.f += nt;
-                    w.fb += 16ull + 8ull * nt;
-                }
-            }
-        }
-        return w;
-    }
-    for (uint32_t q = q0; q < d; q += qstep) {
+    for (unsigned long long it = q0; it < items; it += qstep) {
+        const uint32_t q = (uint32_t)(it / words);
+        const uint32_t wi = w0 + (uint32_t)(it - (unsigned long long)q * words);
         const uint32_t k = pool[dstart + q];
         if (!CFLR_CHECK(k < n, err)) continue;
-        const uint32_t *ok = oc + ((size_t)o * n + k) * ow;
-        for (uint32_t wi = lx0 >> 5; wi <= (lx0 + F - 1) >> 5; wi++) {
-            const uint32_t lo = wi * 32;
-            uint32_t m = ok[wi];
-            if (lx0 > lo) m &= ~0u << (lx0 - lo);
-            if (lx0 + F < lo + 32) m &= (1u << (lx0 + F - lo)) - 1;
-            while (m) {
-                // up to four members' descriptors in flight together
-                uint4 gd[4];
-                uint32_t cnt = 0;
+        uint32_t m = oc[((size_t)o * n + k) * ow + wi];
+        if (wi * 32 < lx0) m &= ~0u << (lx0 & 31);
+        if (wi * 32 + 32 > lx1) m &= (1u << (lx1 & 31)) - 1;
+        while (m) {
+            // up to four members' descriptors in flight together
+            uint4 gd[4];
+            uint32_t cnt = 0;
 #pragma unroll
-                for (int t = 0; t < 4; t++) {
-                    gd[t] = make_uint4(0, 0, 0, 0);
-                    if (m) {
-                        const uint32_t i = lo + (__ffs(m) - 1) - lx0;
-                        m &= m - 1;
-                        gd[t] = S.desc[g0 + i][(size_t)o * n + k];
-                        cnt++;
-                    }
+            for (int t = 0; t < 4; t++) {
+                gd[t] = make_uint4(0, 0, 0, 0);
+                if (m) {
+                    const uint32_t i = wi * 32 + (__ffs(m) - 1) - lx0;
+                    m &= m - 1;
+                    gd[t] = dg[(size_t)(2 * i) * n + k];
+                    cnt++;
                 }
-#pragma unroll
-                for (int t = 0; t < 4; t++) {
-                    const uint32_t nt = gd[t].y - (o ? (gd[t].w & DLAST_MASK) : 0u);
-                    w.f += nt;
-                    w.fb += 8ull * nt;
-                }
-                w.fb += 16ull * cnt;
             }
+#pragma unroll
+            for (int t = 0; t < 4; t++) {
+                const uint32_t nt = gd[t].y - (o ? (gd[t].w & DLAST_MASK) : 0u);
+                w.f += nt;
+                w.fb += 8ull * nt;
+            }
+            w.fb += 16ull * cnt;
         }
     }
     return w;
@@ -1227,7 +1213,64 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
                 if (f < total) {
                     const uint32_t nth = f - (o_incl - o_cnt), plo = __popc(o_lo);
                     tag = nth < plo ? select_bit(o_lo, nth) : 32 + select_bit(o_hi, nth - plo);
-                    const uint4 gd = S.desc[g0 + tag][oo + o_k];
+                    // (consecutive slots: member i's descriptors start 2 i n on)
+                    const uint4 gd = dg[(size_t)(2 * tag) * gi.n + o_k];
+                    if (row_in_pool(S, g0 + tag, gd, &W.cnt->overflow)) {
+                        toff = gd.x;
+                        tn = gd.y - (gi.o ? (gd.w & DLAST_MASK) : 0u);
+                    }
+                }
+                walk(toff, tn, tag, o_k);
+            }
+        }
+        return emitted;
+    }
+    if (gi.fam && gi.consec) {
+        // more than 64 members: a lane per (entry, occupancy word) item, 32
+        // at a time, numbered entry * words + word; the set bits of the words
+        // are the (entry, member) pairs that have a row, packed 32 per step
+        // as above.  A step covers 1024 members of an entry, where testing a
+        // member per lane took one chain of dependent loads per 32 members
+        // (bin 0 of the 142-field alias graph: 6.3 ms of an 11 ms solve, now 2.5).
+        const uint32_t *oc = S.occ[g0];
+        const uint32_t ow = S.occ_w[g0], lx0 = S.local[g0], lx1 = lx0 + gi.F;
+        const uint32_t w0 = lx0 >> 5, words = ((lx1 - 1) >> 5) - w0 + 1;
+        const unsigned long long items = (unsigned long long)d * words;
+        const unsigned long long hi_i = items * (warp_id + 1) / nwarps;
+        for (unsigned long long ib = items * warp_id / nwarps; ib < hi_i; ib += 32) {
+            const unsigned long long it = ib + lane;
+            uint32_t k = 0, bits = 0, first = 0;     // first: member of bit 0 (mod 2^32)
+            if (it < hi_i) {
+                const uint32_t e = (uint32_t)(it / words);
+                const uint32_t w = w0 + (uint32_t)(it - (unsigned long long)e * words);
+                k = pool[dstart + e];
+                if (!CFLR_CHECK(k < gi.n, &W.cnt->overflow)) k = 0;
+                bits = oc[(oo + k) * ow + w];
+                if (w * 32 < lx0) bits &= ~0u << (lx0 & 31);
+                if (w * 32 + 32 > lx1) bits &= (1u << (lx1 & 31)) - 1;
+                first = w * 32 - lx0;
+            }
+            const uint32_t cnt = __popc(bits);
+            const uint32_t incl = warp_incl_scan(cnt, lane);
+            const uint32_t total = __shfl_sync(FULL_MASK, incl, 31);
+            for (uint32_t fb = 0; fb < total; fb += 32) {
+                const uint32_t f = fb + lane;
+                int lo = 0, hi = 31;
+#pragma unroll
+                for (int st = 0; st < 5; st++) {     // first lane whose inclusive sum > f
+                    const int mid = (lo + hi) >> 1;
+                    const uint32_t v = __shfl_sync(FULL_MASK, incl, mid);
+                    if (f < v) hi = mid; else lo = mid + 1;
+                }
+                const int owner = lo > 31 ? 31 : lo;
+                const uint32_t o_k = __shfl_sync(FULL_MASK, k, owner);
+                const uint32_t o_bits = __shfl_sync(FULL_MASK, bits, owner);
+                const uint32_t o_first = __shfl_sync(FULL_MASK, first, owner);
+                const uint32_t o_excl = __shfl_sync(FULL_MASK, incl - cnt, owner);
+                uint32_t toff = 0, tn = 0, tag = 0;
+                if (f < total) {
+                    tag = o_first + select_bit(o_bits, f - o_excl);
+                    const uint4 gd = dg[(size_t)(2 * tag) * gi.n + o_k];
                     if (row_in_pool(S, g0 + tag, gd, &W.cnt->overflow)) {
                         toff = gd.x;
                         tn = gd.y - (gi.o ? (gd.w & DLAST_MASK) : 0u);
@@ -1239,8 +1282,8 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
         return emitted;
     }
     if (gi.fam) {
-        // any family: the (entry, member) pairs numbered entry * F + member,
-        // 32 per warp step; a member's row counts when its occupancy bit is set
+        // members on scattered slots: the (entry, member) pairs numbered
+        // entry * F + member, 32 per warp step; a member's row counts when its occupancy bit is set
         const unsigned long long items = (unsigned long long)d * gi.F;
         for (unsigned long long ib = (unsigned long long)warp_id * 32; ib < items;
              ib += (unsigned long long)nwarps * 32) {
