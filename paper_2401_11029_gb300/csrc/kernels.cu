@@ -1500,20 +1500,23 @@ __global__ void __launch_bounds__(256, 4) k_spgemm_bitmap(SlotTab S, ProdTab P, 
 // k_commit: global dedupe of candidates into the per-slot pair sets
 // ---------------------------------------------------------------------------
 
-// The commit stages a CTA's new pairs and touched rows in shared memory and
-// reserves their room in the global lists with one atomic per list per
-// round: per-warp atomics on those few counters serialise at the L2 (every
-// warp of the grid hits the same addresses).
+// A new pair stays where the product kernels put it, in the candidate list:
+// the commit marks the others empty and writes beside each new pair its
+// place among its row's and its column's new entries (the atomics that count
+// them return it), so the scatter appends without cursors of its own and no
+// list of new pairs is written.
+// The rows a CTA touches first are staged in shared memory and their room in
+// the global list reserved with one atomic per round: per-warp atomics on
+// that counter serialise at the L2 (every warp of the grid hits the same
+// address).
 constexpr uint32_t COMMIT_ROUND = 512;    // candidates a CTA takes per round
-constexpr uint32_t COMMIT_SLOTS = 1024;   // per-slot counts kept in shared memory
+constexpr uint32_t COMMIT_SLOTS = 2048;   // per-slot counts kept in shared memory
 
 __global__ void __launch_bounds__(256) k_commit(SlotTab S, WorkBufs W, uint32_t n_slots) {
-    __shared__ unsigned long long st_key[COMMIT_ROUND];
-    __shared__ uint32_t st_slot[COMMIT_ROUND];
     __shared__ uint2 st_touch[2 * COMMIT_ROUND];
     __shared__ uint32_t slot_new[COMMIT_SLOTS];
     __shared__ uint32_t n_new, n_touch;
-    __shared__ unsigned long long base_new, base_touch;
+    __shared__ unsigned long long base_touch;
     __shared__ unsigned stop;
     // one read for the CTA (this kernel's own threads may set OVF_FULL, and
     // every thread must take the same path to the barriers below)
@@ -1525,18 +1528,21 @@ __global__ void __launch_bounds__(256) k_commit(SlotTab S, WorkBufs W, uint32_t 
     unsigned long long *out_n = &W.touched_n[par ^ 1];
     uint2 *t_out = W.touched[par ^ 1];
     const unsigned long long nc = min(W.cnt->cand, W.cand_cap);
+    if ((unsigned long long)blockIdx.x * COMMIT_ROUND >= nc) return;   // no round for this CTA
     const bool hist = n_slots <= COMMIT_SLOTS;
-    for (uint32_t s = threadIdx.x; s < COMMIT_SLOTS; s += blockDim.x) slot_new[s] = 0;
+    if (hist)
+        for (uint32_t s = threadIdx.x; s < n_slots; s += blockDim.x) slot_new[s] = 0;
     if (threadIdx.x == 0) n_new = n_touch = 0;
     __syncthreads();
+    uint32_t mine = 0;                         // new pairs of this warp (lane 0)
     for (unsigned long long r0 = (unsigned long long)blockIdx.x * COMMIT_ROUND; r0 < nc;
          r0 += (unsigned long long)gridDim.x * COMMIT_ROUND) {
         for (uint32_t q = 0; q < COMMIT_ROUND; q += blockDim.x) {
             const unsigned long long t = r0 + q + threadIdx.x;
             bool isnew = false;
             unsigned long long key = 0;
-            uint32_t slot = EMPTY32;
-            if (t < nc) slot = W.cand_slot[t];
+            const uint32_t listed = t < nc ? W.cand_slot[t] : EMPTY32;
+            uint32_t slot = listed;
             if (slot != EMPTY32) {            // not an unused reserved entry
                 key = W.cand_key[t];
                 if (!CFLR_CHECK((key >> 32) < S.n[slot] && (uint32_t)key < S.n[slot],
@@ -1577,57 +1583,48 @@ __global__ void __launch_bounds__(256) k_commit(SlotTab S, WorkBufs W, uint32_t 
             const uint32_t i = (uint32_t)(key >> 32), j = (uint32_t)key;
             if (isnew) {
                 uint2 *dn = S.dn[slot];
-                first_r = atomicAdd(&dn[i].x, 1u) == 0;
-                first_c = atomicAdd(&dn[(size_t)S.n[slot] + j].x, 1u) == 0;
+                const uint32_t pr = atomicAdd(&dn[i].x, 1u);
+                const uint32_t pc = atomicAdd(&dn[(size_t)S.n[slot] + j].x, 1u);
+                first_r = pr == 0;
+                first_c = pc == 0;
+                W.cand_pos[t] = make_uint2(pr, pc);
                 if (hist) atomicAdd(&slot_new[slot], 1u);
                 else atomicAdd(&S.delta[slot], 1ull);
+            } else if (listed != EMPTY32) {
+                W.cand_slot[t] = EMPTY32;
             }
-            // stage the warp's new pairs and first-touched rows (one shared
-            // atomic per warp and list)
-            const unsigned m = __ballot_sync(FULL_MASK, isnew);
-            if (m) {
-                uint32_t p0 = 0;
-                if (lane == 0) p0 = atomicAdd(&n_new, (uint32_t)__popc(m));
-                p0 = __shfl_sync(FULL_MASK, p0, 0);
-                if (isnew) {
-                    const uint32_t p = p0 + __popc(m & ((1u << lane) - 1));
-                    st_key[p] = key;
-                    st_slot[p] = slot;
-                }
-                const unsigned fr = __ballot_sync(FULL_MASK, first_r);
-                const unsigned fc = __ballot_sync(FULL_MASK, first_c);
-                if (fr | fc) {
-                    uint32_t q0 = 0;
-                    if (lane == 0) q0 = atomicAdd(&n_touch, (uint32_t)(__popc(fr) + __popc(fc)));
-                    q0 = __shfl_sync(FULL_MASK, q0, 0);
-                    const unsigned below = (1u << lane) - 1;
-                    if (first_r) st_touch[q0 + __popc(fr & below)] = make_uint2(slot * 2, i);
-                    if (first_c)
-                        st_touch[q0 + __popc(fr) + __popc(fc & below)] = make_uint2(slot * 2 + 1, j);
-                }
+            mine += __popc(__ballot_sync(FULL_MASK, isnew));
+            // stage the warp's first-touched rows (one shared atomic per warp)
+            const unsigned fr = __ballot_sync(FULL_MASK, first_r);
+            const unsigned fc = __ballot_sync(FULL_MASK, first_c);
+            if (fr | fc) {
+                uint32_t q0 = 0;
+                if (lane == 0) q0 = atomicAdd(&n_touch, (uint32_t)(__popc(fr) + __popc(fc)));
+                q0 = __shfl_sync(FULL_MASK, q0, 0);
+                const unsigned below = (1u << lane) - 1;
+                if (first_r) st_touch[q0 + __popc(fr & below)] = make_uint2(slot * 2, i);
+                if (first_c)
+                    st_touch[q0 + __popc(fr) + __popc(fc & below)] = make_uint2(slot * 2 + 1, j);
             }
         }
         __syncthreads();
-        const uint32_t nn = n_new, nt = n_touch;
-        if (threadIdx.x == 0) {
-            base_new = nn ? atomicAdd(&W.cnt->delta, (unsigned long long)nn) : 0;
-            base_touch = nt ? atomicAdd(out_n, (unsigned long long)nt) : 0;
+        const uint32_t nt = n_touch;
+        if (nt) {                              // uniform
+            if (threadIdx.x == 0) base_touch = atomicAdd(out_n, (unsigned long long)nt);
+            __syncthreads();
+            for (uint32_t q = threadIdx.x; q < nt; q += blockDim.x) {
+                const unsigned long long tp = base_touch + q;
+                if (tp < W.touched_cap) t_out[tp] = st_touch[q];
+                else atomicOr(&W.cnt->overflow, OVF_TOUCHED);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) n_touch = 0;
         }
-        __syncthreads();
-        // new pairs <= candidates <= the delta buffer's capacity
-        for (uint32_t q = threadIdx.x; q < nn; q += blockDim.x) {
-            W.delta_key[base_new + q] = st_key[q];
-            W.delta_slot[base_new + q] = st_slot[q];
-        }
-        for (uint32_t q = threadIdx.x; q < nt; q += blockDim.x) {
-            const unsigned long long tp = base_touch + q;
-            if (tp < W.touched_cap) t_out[tp] = st_touch[q];
-            else atomicOr(&W.cnt->overflow, OVF_TOUCHED);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) n_new = n_touch = 0;
         __syncthreads();
     }
+    if (lane == 0 && mine) atomicAdd(&n_new, mine);
+    __syncthreads();
+    if (threadIdx.x == 0 && n_new) atomicAdd(&W.cnt->delta, (unsigned long long)n_new);
     if (hist) {
         for (uint32_t s = threadIdx.x; s < n_slots; s += blockDim.x)
             if (slot_new[s]) atomicAdd(&S.delta[s], (unsigned long long)slot_new[s]);
@@ -1698,11 +1695,38 @@ __device__ __forceinline__ uint32_t warp_fold_tiles(uint32_t *tab, uint32_t cnt,
     return base;
 }
 
+// A row of the touched list by itself: descriptor, owner and new entries.
+struct TouchedRow {
+    uint4 dsc;
+    uint32_t slot, o, w;
+    size_t r;               // o * n + index
+};
+__device__ __forceinline__ TouchedRow touched_row(const SlotTab &S, uint2 t) {
+    TouchedRow x;
+    x.slot = t.x >> 1;
+    x.o = t.x & 1;
+    x.r = (size_t)x.o * S.n[x.slot] + t.y;
+    x.dsc = S.desc[x.slot][x.r];
+    x.w = S.dn[x.slot][x.r].x;
+    return x;
+}
+__device__ __forceinline__ bool row_has_room(const TouchedRow &x) {
+    return (unsigned long long)x.dsc.y + x.w <= x.dsc.z && x.w <= entry_cap(x.dsc);
+}
+
 // Make room for every listed row: its new entries (dn.x) in the entry area
 // and as many tiles at the end of its tile list.  A row without that room
 // moves to a new segment with its tiles folded to one per word; rows of more
-// than TILE_WARP_MAX tiles are left to k_capacity_big.  Also sets the
-// occupancy bit of a row's first entries and clears the append cursors.
+// than TILE_WARP_MAX tiles are listed for k_capacity_big.  Also sets the
+// occupancy bit of a row's first entries.
+// Bound by the latency of the chain list entry -> descriptor -> pool counter.
+// A warp takes 32 rows at a time, at a stride (a short list still spreads
+// over all warps), and a lane looks at each, so 32 chains are in flight; rows
+// that get their first segment (most of those that need room) take it there,
+// with one pool reservation for the warp, and only rows with tiles to fold
+// take the whole warp in turn.  A warp per row waited through the chain for
+// every row (500k-vertex points-to solve: 18.2 ms, now 8.1 ms; 200k-vertex
+// alias solve: 2.5 ms, now 1.4 ms).
 // Idempotent: after a pool overflow the host grows the pool and runs it again.
 __global__ void __launch_bounds__(256) k_capacity(SlotTab S, InstTab I, WorkBufs W) {
     __shared__ __align__(16) uint32_t tabs[8][4 * TILE_WARP_MAX];   // a table per warp
@@ -1712,82 +1736,129 @@ __global__ void __launch_bounds__(256) k_capacity(SlotTab S, InstTab I, WorkBufs
     const int par = *W.parity;
     const uint2 *t_out = W.touched[par ^ 1];
     const unsigned long long n_t = min(W.touched_n[par ^ 1], W.touched_cap);
-    const unsigned long long nw = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    const unsigned long long nw = (unsigned long long)gridDim.x * 8;
     unsigned long long moved = 0;           // tile bytes read and written (lane 0)
-    for (unsigned long long e = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + wib;
-         e < n_t; e += nw) {
-        const uint2 t = t_out[e];
-        const uint32_t slot = t.x >> 1, o = t.x & 1;
-        const size_t r = (size_t)o * S.n[slot] + t.y;
-        uint4 *dp = &S.desc[slot][r];
-        const uint4 dsc = *dp;
-        const uint32_t w = S.dn[slot][r].x;
-        if (lane == 0) {
-            S.dn[slot][r].y = 0;
-            if (dsc.y == 0) {                 // the row gets its first entries
-                const uint32_t lx = S.local[slot];
-                atomicOr(&S.occ[slot][r * S.occ_w[slot] + (lx >> 5)], 1u << (lx & 31));
+    for (unsigned long long e0 = (unsigned long long)blockIdx.x * 8 + wib; e0 < n_t;
+         e0 += 32 * nw) {
+        unsigned long long size = 0;        // pool words of a first segment
+        TouchedRow x{};
+        uint32_t inst = 0;
+        bool fold = false;
+        if (e0 + lane * nw < n_t) {
+            const uint2 t = t_out[e0 + lane * nw];
+            x = touched_row(S, t);
+            inst = S.inst[x.slot];
+            if (x.dsc.y == 0) {               // the row gets its first entries
+                const uint32_t lx = S.local[x.slot];
+                atomicOr(&S.occ[x.slot][x.r * S.occ_w[x.slot] + (lx >> 5)], 1u << (lx & 31));
+            }
+            if (!row_has_room(x)) {
+                if (x.dsc.y == 0) {
+                    size = (unsigned long long)tile_words(tile_cap_after_move(0, x.w)) +
+                           (1ull << entry_log_after_move(x.w));
+                } else if (x.dsc.y > TILE_WARP_MAX) {
+                    // (a list that is full is counted on: k_capacity_big then
+                    // looks through all touched rows)
+                    const uint32_t p = atomicAdd(&W.cnt->cap_n, 1u);
+                    if (p < W.big_cap) W.big_rows[p] = t;
+                } else {
+                    fold = row_in_pool(S, x.slot, x.dsc, &W.cnt->overflow);
+                }
             }
         }
-        if ((unsigned long long)dsc.y + w <= dsc.z && w <= entry_cap(dsc)) continue;
-        if (dsc.y > TILE_WARP_MAX) continue;
-        if (!row_in_pool(S, slot, dsc, &W.cnt->overflow)) continue;
-        uint32_t *pool = S.pool[slot];
-        // fold into the table first (the count sizes the new segment) ...
-        uint32_t lg = 5;
-        while ((1u << lg) < 2 * dsc.y) lg++;
-        clear_table(tab, lg, lane, 32);
-        __syncwarp();
-        const HashAcc acc{tab, (int)lg, &W.cnt->overflow};
-        for (uint32_t q = lane; q < dsc.y; q += 32) {
-            const uint2 tl = *reinterpret_cast<const uint2 *>(pool + dsc.x + 2 * q);
-            acc.ins(tl.x, tl.y);
-        }
-        __syncwarp();
-        uint32_t D = 0;
-        for (uint32_t s = lane; s < (1u << lg); s += 32) D += tab[2 * s] != EMPTY32;
-        for (int dd = 16; dd > 0; dd >>= 1) D += __shfl_xor_sync(FULL_MASK, D, dd);
-        const uint32_t tcap = tile_cap_after_move(D, w), elog = entry_log_after_move(w);
-        const unsigned long long size = (unsigned long long)tile_words(tcap) + (1ull << elog);
-        const uint32_t inst = S.inst[slot];
-        unsigned long long off = 0;
-        if (lane == 0) {
-            off = atomicAdd(&I.pool_top[inst], size);
-            if (off + size > I.pool_cap[inst]) {
-                atomicOr(&W.cnt->overflow, OVF_POOL);
-                off = ~0ull;
+        // first segments: one reservation for the warp when its rows are of
+        // one instance
+        const unsigned need = __ballot_sync(FULL_MASK, size != 0);
+        if (need) {
+            const uint32_t inst0 = __shfl_sync(FULL_MASK, inst, __ffs(need) - 1);
+            unsigned long long off = 0, end = 0;
+            if (__all_sync(FULL_MASK, size == 0 || inst == inst0)) {
+                unsigned long long incl = size;
+#pragma unroll
+                for (int dd = 1; dd < 32; dd <<= 1) {
+                    const unsigned long long y = __shfl_up_sync(FULL_MASK, incl, dd);
+                    if (lane >= dd) incl += y;
+                }
+                unsigned long long base = 0;
+                if (lane == 31) base = atomicAdd(&I.pool_top[inst0], incl);
+                base = __shfl_sync(FULL_MASK, base, 31);
+                off = base + incl - size;
+                end = __shfl_sync(FULL_MASK, base + incl, 31);
+            } else if (size) {
+                off = atomicAdd(&I.pool_top[inst], size);
+                end = off + size;
+            }
+            if (size) {
+                if (end > I.pool_cap[inst])
+                    atomicOr(&W.cnt->overflow, OVF_POOL);
+                else
+                    S.desc[x.slot][x.r] =
+                        make_uint4((uint32_t)off, 0, tile_cap_after_move(0, x.w),
+                                   entry_log_after_move(x.w) << ELOG_SHIFT);
             }
         }
-        off = __shfl_sync(FULL_MASK, off, 0);
-        if (off == ~0ull) {
+        for (unsigned fm = __ballot_sync(FULL_MASK, fold); fm; fm &= fm - 1) {
+            const int l = __ffs(fm) - 1;
+            const uint32_t slot = __shfl_sync(FULL_MASK, x.slot, l);
+            const uint32_t toff = __shfl_sync(FULL_MASK, x.dsc.x, l);
+            const uint32_t tn = __shfl_sync(FULL_MASK, x.dsc.y, l);
+            const uint32_t w = __shfl_sync(FULL_MASK, x.w, l);
+            const uint32_t f_inst = __shfl_sync(FULL_MASK, inst, l);
+            uint32_t *pool = S.pool[slot];
+            // fold into the table first (the count sizes the new segment) ...
+            uint32_t lg = 5;
+            while ((1u << lg) < 2 * tn) lg++;
+            clear_table(tab, lg, lane, 32);
             __syncwarp();
-            continue;
+            const HashAcc acc{tab, (int)lg, &W.cnt->overflow};
+            for (uint32_t q = lane; q < tn; q += 32) {
+                const uint2 tl = *reinterpret_cast<const uint2 *>(pool + toff + 2 * q);
+                acc.ins(tl.x, tl.y);
+            }
+            __syncwarp();
+            uint32_t D = 0;
+            for (uint32_t s = lane; s < (1u << lg); s += 32) D += tab[2 * s] != EMPTY32;
+            D = __reduce_add_sync(FULL_MASK, D);
+            const uint32_t tcap = tile_cap_after_move(D, w), elog = entry_log_after_move(w);
+            const unsigned long long words = (unsigned long long)tile_words(tcap) + (1ull << elog);
+            unsigned long long off = 0;
+            if (lane == 0) {
+                off = atomicAdd(&I.pool_top[f_inst], words);
+                if (off + words > I.pool_cap[f_inst]) {
+                    atomicOr(&W.cnt->overflow, OVF_POOL);
+                    off = ~0ull;
+                }
+            }
+            off = __shfl_sync(FULL_MASK, off, 0);
+            if (off != ~0ull) {
+                // ... then write the table's words as the new tile list
+                uint32_t *np = pool + off;
+                uint32_t base = 0;
+                for (uint32_t sb = 0; sb < (1u << lg); sb += 32) {
+                    const uint2 sl = reinterpret_cast<const uint2 *>(tab)[sb + lane];
+                    const bool has = sl.x != EMPTY32;
+                    const unsigned m = __ballot_sync(FULL_MASK, has);
+                    if (has)
+                        reinterpret_cast<uint2 *>(np)[base + __popc(m & ((1u << lane) - 1))] = sl;
+                    base += __popc(m);
+                }
+                if (lane == l)
+                    S.desc[slot][x.r] = make_uint4((uint32_t)off, D, tcap, elog << ELOG_SHIFT);
+                if (lane == 0) moved += 8ull * (tn + D);
+            }
+            __syncwarp();
         }
-        // ... then write the table's words as the new tile list
-        uint32_t *np = pool + off;
-        uint32_t base = 0;
-        for (uint32_t sb = 0; sb < (1u << lg); sb += 32) {
-            const uint2 sl = reinterpret_cast<const uint2 *>(tab)[sb + lane];
-            const bool has = sl.x != EMPTY32;
-            const unsigned m = __ballot_sync(FULL_MASK, has);
-            if (has) reinterpret_cast<uint2 *>(np)[base + __popc(m & ((1u << lane) - 1))] = sl;
-            base += __popc(m);
-        }
-        __syncwarp();
-        if (lane == 0) {
-            *dp = make_uint4((uint32_t)off, D, tcap, elog << ELOG_SHIFT);
-            moved += 8ull * (dsc.y + D);
-        }
-        __syncwarp();
     }
     if (lane == 0 && moved) atomicAdd(&W.cnt->bytes_move[0], moved);
 }
 
-// The rows k_capacity leaves (more than TILE_WARP_MAX tiles): the CTA lists
-// the large rows among 256 touched rows at a time, then folds each through
-// an n-bit bitmap in shared memory (its tiles come out in word order).
-// Without room for the bitmap (use_smem 0) the tiles are copied as they are.
-// Idempotent like k_capacity.
+// The rows k_capacity leaves (more than TILE_WARP_MAX tiles), from its list,
+// or by a look at every touched row (256 at a time) when the list was too
+// short for them: a CTA folds each through an n-bit bitmap in shared memory
+// (its tiles come out in word order).  Without room for the bitmap (use_smem
+// 0) the tiles are copied as they are.  Idempotent like k_capacity.
+// (Looking through the touched rows on every launch took 4.8 ms of the
+// 500k-vertex points-to solve, in which few rows are that long.)
 __global__ void __launch_bounds__(256) k_capacity_big(SlotTab S, InstTab I, WorkBufs W,
                                                       int use_smem) {
     extern __shared__ uint32_t bm[];
@@ -1795,118 +1866,118 @@ __global__ void __launch_bounds__(256) k_capacity_big(SlotTab S, InstTab I, Work
     __shared__ uint32_t list_n;
     __shared__ unsigned long long sh[16];
     __shared__ unsigned long long off_sh;
-    if (W.cnt->overflow & OVF_STOP) return;
-    const int par = *W.parity;
-    const uint2 *t_out = W.touched[par ^ 1];
-    const unsigned long long n_t = min(W.touched_n[par ^ 1], W.touched_cap);
+    __shared__ unsigned stop;
+    if (threadIdx.x == 0) stop = W.cnt->overflow & OVF_STOP;
+    __syncthreads();
+    if (stop) return;
     unsigned long long moved = 0;           // tile bytes read and written (thread 0)
-    for (unsigned long long cb = (unsigned long long)blockIdx.x * 256; cb < n_t;
-         cb += (unsigned long long)gridDim.x * 256) {
-        if (threadIdx.x == 0) list_n = 0;
-        __syncthreads();
-        const unsigned long long e = cb + threadIdx.x;
-        if (e < n_t) {
-            const uint2 t = t_out[e];
-            const uint32_t slot = t.x >> 1, o = t.x & 1;
-            const size_t r = (size_t)o * S.n[slot] + t.y;
-            const uint4 dsc = S.desc[slot][r];
-            const uint32_t w = S.dn[slot][r].x;
-            if (((unsigned long long)dsc.y + w > dsc.z || w > entry_cap(dsc)) &&
-                dsc.y > TILE_WARP_MAX)
-                list[atomicAdd(&list_n, 1u)] = threadIdx.x;
+    auto move_row = [&](uint2 t) {          // by the whole CTA
+        const TouchedRow x = touched_row(S, t);
+        const uint4 dsc = x.dsc;
+        const uint32_t n = S.n[x.slot];
+        uint32_t *pool = S.pool[x.slot];
+        const uint32_t words = (n + 31) >> 5;
+        const uint32_t per = (words + blockDim.x - 1) / blockDim.x;
+        const uint32_t w0 = min(words, threadIdx.x * per), w1 = min(words, w0 + per);
+        uint32_t cnt = 0;
+        if (use_smem) {
+            for (uint32_t q = threadIdx.x; q < words; q += blockDim.x) bm[q] = 0;
+            __syncthreads();
+            for (uint32_t q = threadIdx.x; q < dsc.y; q += blockDim.x) {
+                const uint2 tl = *reinterpret_cast<const uint2 *>(pool + dsc.x + 2 * q);
+                atomicOr(&bm[tl.x], tl.y);
+            }
+            __syncthreads();
+            for (uint32_t q = w0; q < w1; q++) cnt += bm[q] != 0;
+        }
+        unsigned long long D = 0;
+        const unsigned long long before = block_excl_scan256(cnt, sh, D);
+        const uint32_t ntn = use_smem ? (uint32_t)D : dsc.y;
+        const uint32_t tcap = tile_cap_after_move(ntn, x.w), elog = entry_log_after_move(x.w);
+        const unsigned long long size = (unsigned long long)tile_words(tcap) + (1ull << elog);
+        if (threadIdx.x == 0) {
+            unsigned long long off = atomicAdd(&I.pool_top[S.inst[x.slot]], size);
+            if (off + size > I.pool_cap[S.inst[x.slot]]) {
+                atomicOr(&W.cnt->overflow, OVF_POOL);
+                off = ~0ull;
+            }
+            off_sh = off;
         }
         __syncthreads();
-        const uint32_t ln = list_n;
-        for (uint32_t li = 0; li < ln; li++) {
-            const uint2 t = t_out[cb + list[li]];
-            const uint32_t slot = t.x >> 1, o = t.x & 1;
-            const uint32_t n = S.n[slot];
-            const size_t r = (size_t)o * n + t.y;
-            uint4 *dp = &S.desc[slot][r];
-            const uint4 dsc = *dp;
-            const uint32_t w = S.dn[slot][r].x;
-            uint32_t *pool = S.pool[slot];
-            const uint32_t words = (n + 31) >> 5;
-            const uint32_t per = (words + blockDim.x - 1) / blockDim.x;
-            const uint32_t w0 = min(words, threadIdx.x * per), w1 = min(words, w0 + per);
-            uint32_t cnt = 0;
+        const unsigned long long off = off_sh;
+        if (off != ~0ull) {
+            uint32_t *np = pool + off;
             if (use_smem) {
-                for (uint32_t q = threadIdx.x; q < words; q += blockDim.x) bm[q] = 0;
-                __syncthreads();
-                for (uint32_t q = threadIdx.x; q < dsc.y; q += blockDim.x) {
-                    const uint2 tl = *reinterpret_cast<const uint2 *>(pool + dsc.x + 2 * q);
-                    atomicOr(&bm[tl.x], tl.y);
-                }
-                __syncthreads();
-                for (uint32_t q = w0; q < w1; q++) cnt += bm[q] != 0;
-            }
-            unsigned long long D = 0;
-            const unsigned long long before = block_excl_scan256(cnt, sh, D);
-            const uint32_t ntn = use_smem ? (uint32_t)D : dsc.y;
-            const uint32_t tcap = tile_cap_after_move(ntn, w), elog = entry_log_after_move(w);
-            const unsigned long long size = (unsigned long long)tile_words(tcap) + (1ull << elog);
-            if (threadIdx.x == 0) {
-                unsigned long long off = atomicAdd(&I.pool_top[S.inst[slot]], size);
-                if (off + size > I.pool_cap[S.inst[slot]]) {
-                    atomicOr(&W.cnt->overflow, OVF_POOL);
-                    off = ~0ull;
-                }
-                off_sh = off;
-            }
-            __syncthreads();
-            const unsigned long long off = off_sh;
-            if (off != ~0ull) {
-                uint32_t *np = pool + off;
-                if (use_smem) {
-                    unsigned long long pos = before;
-                    for (uint32_t q = w0; q < w1; q++) {
-                        const uint32_t b = bm[q];
-                        if (b) {
-                            np[2 * pos] = q;
-                            np[2 * pos + 1] = b;
-                            pos++;
-                        }
+                unsigned long long pos = before;
+                for (uint32_t q = w0; q < w1; q++) {
+                    const uint32_t b = bm[q];
+                    if (b) {
+                        np[2 * pos] = q;
+                        np[2 * pos + 1] = b;
+                        pos++;
                     }
-                } else {
-                    for (uint32_t q = threadIdx.x; q < 2 * dsc.y; q += blockDim.x)
-                        np[q] = pool[dsc.x + q];
                 }
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    *dp = make_uint4((uint32_t)off, ntn, tcap, elog << ELOG_SHIFT);
-                    moved += 8ull * (dsc.y + ntn);
-                }
+            } else {
+                for (uint32_t q = threadIdx.x; q < 2 * dsc.y; q += blockDim.x)
+                    np[q] = pool[dsc.x + q];
             }
             __syncthreads();
+            if (threadIdx.x == 0) {
+                S.desc[x.slot][x.r] = make_uint4((uint32_t)off, ntn, tcap, elog << ELOG_SHIFT);
+                moved += 8ull * (dsc.y + ntn);
+            }
+        }
+        __syncthreads();
+    };
+    const uint32_t listed = W.cnt->cap_n;
+    if (listed <= W.big_cap) {
+        for (uint32_t e = blockIdx.x; e < listed; e += gridDim.x) move_row(W.big_rows[e]);
+    } else {
+        const int par = *W.parity;
+        const uint2 *t_out = W.touched[par ^ 1];
+        const unsigned long long n_t = min(W.touched_n[par ^ 1], W.touched_cap);
+        for (unsigned long long cb = (unsigned long long)blockIdx.x * 256; cb < n_t;
+             cb += (unsigned long long)gridDim.x * 256) {
+            if (threadIdx.x == 0) list_n = 0;
+            __syncthreads();
+            const unsigned long long e = cb + threadIdx.x;
+            if (e < n_t) {
+                const TouchedRow x = touched_row(S, t_out[e]);
+                if (!row_has_room(x) && x.dsc.y > TILE_WARP_MAX)
+                    list[atomicAdd(&list_n, 1u)] = threadIdx.x;
+            }
+            __syncthreads();
+            const uint32_t ln = list_n;
+            for (uint32_t li = 0; li < ln; li++) move_row(t_out[cb + list[li]]);
         }
     }
     if (threadIdx.x == 0 && moved) atomicAdd(&W.cnt->bytes_move[1], moved);
 }
 
 // Append the new pairs as single entries: (i, j) goes to the entry area of
-// row i of the row form and of row j of the column form.
+// row i of the row form and of row j of the column form, at the places the
+// commit gave it (an atomic cursor per row took two round trips to L2 for
+// every pair).
 __global__ void __launch_bounds__(256) k_scatter(SlotTab S, WorkBufs W) {
     if (W.cnt->overflow & (OVF_STOP | OVF_POOL)) return;
-    const unsigned long long nd = W.cnt->delta;
+    const unsigned long long nc = min(W.cnt->cand, W.cand_cap);
     for (unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-         t < nd; t += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long key = W.delta_key[t];
-        const uint32_t slot = W.delta_slot[t];
+         t < nc; t += (unsigned long long)gridDim.x * blockDim.x) {
+        const uint32_t slot = W.cand_slot[t];
+        if (slot == EMPTY32) continue;        // not new
+        const unsigned long long key = W.cand_key[t];
+        const uint2 at = W.cand_pos[t];
         const uint32_t i = (uint32_t)(key >> 32), j = (uint32_t)key;
         const uint4 *dsc = S.desc[slot];
-        uint2 *dn = S.dn[slot];
         uint32_t *pool = S.pool[slot];
-        const uint32_t n = S.n[slot];
         const uint4 dr = dsc[i];
-        const uint32_t pr = atomicAdd(&dn[i].y, 1u);
+        const uint4 dc = dsc[(size_t)S.n[slot] + j];
         if (row_in_pool(S, slot, dr, &W.cnt->overflow) &&
-            CFLR_CHECK(dr.z && pr < entry_cap(dr), &W.cnt->overflow))
-            pool[(size_t)dr.x + tile_words(dr.z) + pr] = j;
-        const uint4 dc = dsc[(size_t)n + j];
-        const uint32_t pc = atomicAdd(&dn[(size_t)n + j].y, 1u);
+            CFLR_CHECK(dr.z && at.x < entry_cap(dr), &W.cnt->overflow))
+            pool[(size_t)dr.x + tile_words(dr.z) + at.x] = j;
         if (row_in_pool(S, slot, dc, &W.cnt->overflow) &&
-            CFLR_CHECK(dc.z && pc < entry_cap(dc), &W.cnt->overflow))
-            pool[(size_t)dc.x + tile_words(dc.z) + pc] = i;
+            CFLR_CHECK(dc.z && at.y < entry_cap(dc), &W.cnt->overflow))
+            pool[(size_t)dc.x + tile_words(dc.z) + at.y] = i;
     }
 }
 
@@ -1914,7 +1985,15 @@ __global__ void __launch_bounds__(256) k_scatter(SlotTab S, WorkBufs W) {
 // entries at a time) at the end of its tile list.  The new pairs are not in
 // the row yet, so the tiles of a row never share a set bit; a word may get a
 // second tile, until the row's next move folds them.
-__global__ void __launch_bounds__(256) k_pack(SlotTab S, WorkBufs W) {
+// As in k_capacity a warp takes 32 rows at a time and a lane looks at each:
+// up to four entries the lane packs itself, from one 16-byte load; rows with
+// more take the warp in turn, which loads the next row's first entries before
+// it folds the present ones.  (A warp per row, from the list entry to the
+// tiles, waited through six dependent loads for every row: 500k-vertex
+// points-to solve 13.3 ms, now 7.5 ms; 200k-vertex alias solve 3.6 ms, now
+// 3.3 ms.  Sharing 256 rows over a CTA had the warps wait for the longest
+// row: 15.8 and 6.9 ms.)
+__global__ void __launch_bounds__(256, 5) k_pack(SlotTab S, WorkBufs W) {
     __shared__ __align__(16) uint32_t tabs[8][4 * TILE_WARP_MAX];
     if (W.cnt->overflow & (OVF_STOP | OVF_POOL)) return;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1922,48 +2001,83 @@ __global__ void __launch_bounds__(256) k_pack(SlotTab S, WorkBufs W) {
     const int par = *W.parity;
     const uint2 *t_out = W.touched[par ^ 1];
     const unsigned long long n_t = min(W.touched_n[par ^ 1], W.touched_cap);
-    const unsigned long long nw = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    for (unsigned long long e = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + wib;
-         e < n_t; e += nw) {
-        const uint2 t = t_out[e];
-        const uint32_t slot = t.x >> 1, o = t.x & 1;
-        const size_t r = (size_t)o * S.n[slot] + t.y;
-        uint4 *dp = &S.desc[slot][r];
-        const uint4 dsc = *dp;
-        const uint32_t w = S.dn[slot][r].x;
-        if (!row_in_pool(S, slot, dsc, &W.cnt->overflow) ||
-            !CFLR_CHECK(w <= entry_cap(dsc) && dsc.y + w <= dsc.z, &W.cnt->overflow))
-            continue;
-        const uint32_t *ent = S.pool[slot] + dsc.x + tile_words(dsc.z);
-        uint32_t *tl = S.pool[slot] + dsc.x;
-        if (w == 1) {                  // one new pair: one tile, no table
-            if (lane == 0) {
-                const uint32_t v = ent[0];
-                reinterpret_cast<uint2 *>(tl)[dsc.y] = make_uint2(v >> 5, 1u << (v & 31));
-                dp->y = dsc.y + 1;
-                dp->w = (dsc.w & ~DLAST_MASK) | 1u;
+    const unsigned long long nw = (unsigned long long)gridDim.x * 8;
+    for (unsigned long long e0 = (unsigned long long)blockIdx.x * 8 + wib; e0 < n_t;
+         e0 += 32 * nw) {
+        TouchedRow x{};
+        uint32_t *pool = nullptr;
+        bool fold = false;
+        if (e0 + lane * nw < n_t) {
+            x = touched_row(S, t_out[e0 + lane * nw]);
+            pool = S.pool[x.slot];
+            const uint4 dsc = x.dsc;
+            if (row_in_pool(S, x.slot, dsc, &W.cnt->overflow) &&
+                CFLR_CHECK(x.w <= entry_cap(dsc) && dsc.y + x.w <= dsc.z, &W.cnt->overflow)) {
+                fold = x.w > 4;
+                if (!fold) {
+                    // (an entry area holds at least eight entries)
+                    const uint4 v4 =
+                        *reinterpret_cast<const uint4 *>(pool + dsc.x + tile_words(dsc.z));
+                    const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
+                    uint2 *tl = reinterpret_cast<uint2 *>(pool + dsc.x) + dsc.y;
+                    uint32_t nt = 0;
+#pragma unroll
+                    for (uint32_t q = 0; q < 4; q++) {
+                        if (q >= x.w) break;
+                        // the first entry of a word takes the others' bits along
+                        bool lead = true;
+                        uint32_t bits = 0;
+#pragma unroll
+                        for (uint32_t p = 0; p < 4; p++) {
+                            if (p >= x.w || (v[p] >> 5) != (v[q] >> 5)) continue;
+                            lead &= p >= q;
+                            bits |= 1u << (v[p] & 31);
+                        }
+                        if (lead) tl[nt++] = make_uint2(v[q] >> 5, bits);
+                    }
+                    S.desc[x.slot][x.r] =
+                        make_uint4(dsc.x, dsc.y + nt, dsc.z, (dsc.w & ~DLAST_MASK) | nt);
+                }
             }
-            __syncwarp();
-            continue;
         }
-        uint32_t nt = dsc.y;
-        for (uint32_t c0 = 0; c0 < w; c0 += TILE_WARP_MAX) {
-            const uint32_t cnt = min(TILE_WARP_MAX, w - c0);
-            nt += warp_fold_tiles(tab, cnt,
-                                  [&](uint32_t q) {
-                                      const uint32_t v = ent[c0 + q];
-                                      return make_uint2(v >> 5, 1u << (v & 31));
-                                  },
-                                  tl + 2 * nt, lane, &W.cnt->overflow);
+        const uint32_t *ent = pool + x.dsc.x + tile_words(x.dsc.z);   // of this lane's row
+        unsigned fm = __ballot_sync(FULL_MASK, fold);
+        // the entry `lane` of row l, when it has so many
+        auto first_entry = [&](int l) {
+            const uint32_t *el = (const uint32_t *)__shfl_sync(FULL_MASK, (unsigned long long)ent, l);
+            return (uint32_t)lane < __shfl_sync(FULL_MASK, x.w, l) ? el[lane] : 0u;
+        };
+        uint32_t head = fm ? first_entry(__ffs(fm) - 1) : 0u;
+        while (fm) {
+            const int l = __ffs(fm) - 1;
+            fm &= fm - 1;
+            const uint32_t v0 = head;
+            if (fm) head = first_entry(__ffs(fm) - 1);
+            const uint32_t *el = (const uint32_t *)__shfl_sync(FULL_MASK, (unsigned long long)ent, l);
+            uint32_t *tl = (uint32_t *)__shfl_sync(FULL_MASK, (unsigned long long)pool, l) +
+                           __shfl_sync(FULL_MASK, x.dsc.x, l);
+            const uint32_t w = __shfl_sync(FULL_MASK, x.w, l);
+            const uint32_t t0 = __shfl_sync(FULL_MASK, x.dsc.y, l);
+            uint32_t nt = t0;
+            for (uint32_t c0 = 0; c0 < w; c0 += TILE_WARP_MAX) {
+                const uint32_t cnt = min(TILE_WARP_MAX, w - c0);
+                nt += warp_fold_tiles(tab, cnt,
+                                      [&](uint32_t q) {
+                                          const uint32_t v =
+                                              c0 + q == (uint32_t)lane ? v0 : el[c0 + q];
+                                          return make_uint2(v >> 5, 1u << (v & 31));
+                                      },
+                                      tl + 2 * nt, lane, &W.cnt->overflow);
+            }
+            if (lane == l) {
+                // the delta's tiles (a count beyond the field falls back to
+                // gathering all of A, a superset of A_old with the same union)
+                const uint32_t dl = nt - t0;
+                S.desc[x.slot][x.r] = make_uint4(x.dsc.x, nt, x.dsc.z,
+                                                 (x.dsc.w & ~DLAST_MASK) |
+                                                     (dl <= DLAST_MASK ? dl : 0u));
+            }
         }
-        if (lane == 0) {
-            dp->y = nt;
-            // the delta's tiles (a count beyond the field falls back to
-            // gathering all of A, a superset of A_old with the same union)
-            const uint32_t dl = nt - dsc.y;
-            dp->w = (dsc.w & ~DLAST_MASK) | (dl <= DLAST_MASK ? dl : 0u);
-        }
-        __syncwarp();
     }
 }
 

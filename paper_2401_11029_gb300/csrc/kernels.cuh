@@ -18,7 +18,7 @@
 //                    before them are M_old)
 //   dn[s]       uint2 per row and orientation: .x = pairs the last merge
 //               added to the row (its delta for optimisation 1, kept as
-//               single entries in the entry area), .y = append cursor
+//               single entries in the entry area), .y unused
 //   pool        uint32 arena of row segments; rows grow by relocation,
 //               and a relocation folds the tiles (one tile per word).
 //   htab[s]     open-addressing set of 64-bit keys (i << 32 | j): every pair
@@ -80,7 +80,7 @@ constexpr uint32_t WIT_BINARY = 0u << 30, WIT_EDGE = 1u << 30, WIT_UNIT = 2u << 
 
 struct SlotTab {              // per slot (device arrays, length n_slots)
     uint4 **desc;             // row descriptors (2*n per slot)
-    uint2 **dn;               // delta counts and append cursors (2*n per slot)
+    uint2 **dn;               // delta counts (2*n per slot)
     uint32_t **pool;          // instance pool of the slot
     uint32_t *n;              // vertices of the slot's instance
     uint32_t *inst;           // instance index of the slot
@@ -153,7 +153,7 @@ struct Counters {
                                         // (k_capacity, k_capacity_big)
     unsigned long long tiles_bin3[2];   // product and mask tiles of the bitmap bin
     unsigned int overflow;          // OVF_* bits
-    unsigned int pad;
+    unsigned int cap_n;             // rows listed for k_capacity_big (cleared with the bits)
 };
 
 constexpr unsigned OVF_GROUPS = 1u;    // work list overflow        (before the commit)
@@ -193,9 +193,12 @@ struct WorkBufs {
     uint2 *groups[N_BINS]; unsigned long long group_cap[N_BINS];   // {code, idx}
     unsigned long long *cand_key; uint32_t *cand_slot; unsigned long long cand_cap;
     uint2 *cand_wit;                   // witness of each candidate (null: off)
-    unsigned long long *delta_key; uint32_t *delta_slot;
+    // place of each new pair among the new entries of its row and its column
+    // (k_commit, which also marks the candidates that are not new empty)
+    uint2 *cand_pos;
     uint32_t *bitmap_scratch; unsigned long long bitmap_words;  // per CTA, global
-    uint2 *big_rows; unsigned long long big_cap;   // long delta rows (k_symbolic)
+    // long delta rows (k_symbolic), then rows of many tiles to move (k_capacity)
+    uint2 *big_rows; unsigned long long big_cap;
     Counters *cnt;
 };
 

@@ -116,7 +116,7 @@ struct cflr_ctx {
     uint32_t n = 0;
     uint64_t ignored = 0;
     uint4 *desc = nullptr;              // n_nt * 2 * n descriptors
-    uint2 *dn = nullptr;                // n_nt * 2 * n delta counts / append cursors
+    uint2 *dn = nullptr;                // n_nt * 2 * n delta counts
     uint32_t *occ = nullptr;            // occupancy bits: 2 * n * occ_w words
     uint32_t occ_w = 0;
     bool rows_set = false;              // desc, dn and occ hold a (possibly empty) graph's rows
@@ -384,8 +384,9 @@ struct Runner {
     DevArr<uint2> d_touched[2];
     DevArr<unsigned long long> d_touched_n;   // [2]
     DevArr<uint2> d_groups[N_BINS];
-    DevArr<unsigned long long> d_cand_key, d_delta_key;
-    DevArr<uint32_t> d_cand_slot, d_delta_slot;
+    DevArr<unsigned long long> d_cand_key;
+    DevArr<uint32_t> d_cand_slot;
+    DevArr<uint2> d_cand_pos;
     DevArr<uint32_t> d_bitmap;
     DevArr<uint2> d_big;                      // long delta rows for the symbolic CTA pass
     DevArr<Counters> d_cnt;
@@ -721,7 +722,7 @@ struct Runner {
         }
         W.cand_key = d_cand_key.p; W.cand_slot = d_cand_slot.p; W.cand_cap = cand_cap;
         W.cand_wit = wit ? d_cand_wit.p : nullptr;
-        W.delta_key = d_delta_key.p; W.delta_slot = d_delta_slot.p;
+        W.cand_pos = d_cand_pos.p;
         W.bitmap_scratch = d_bitmap.p;
         W.bitmap_words = (max_n + 31) / 32;
         W.big_rows = d_big.p;
@@ -743,8 +744,7 @@ struct Runner {
         d_cand_key.alloc(own, cap);
         d_cand_slot.alloc(own, cap);
         if (wit) d_cand_wit.alloc(own, cap);
-        d_delta_key.alloc(own, cap);
-        d_delta_slot.alloc(own, cap);
+        d_cand_pos.alloc(own, cap);
         graph_valid = false;
     }
     // Both touched lists; the list touched[parity] keeps its rows.  Each must
@@ -934,8 +934,8 @@ struct Runner {
         ck(cudaMemcpyAsync(h_parity, d_parity.p, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H");
         sync("status");
     }
-    void clear_overflow() {
-        ck(cudaMemsetAsync(&d_cnt.p->overflow, 0, sizeof(unsigned), st), "memset");
+    void clear_overflow() {            // and the list of rows to move beside it
+        ck(cudaMemsetAsync(&d_cnt.p->overflow, 0, 2 * sizeof(unsigned), st), "memset");
     }
 
     // New size of a work buffer that overflowed at `count` entries.  The
@@ -1137,12 +1137,12 @@ struct Runner {
         read_status();
         own->k_bytes[KID_SYMBOLIC] += h_ctl->bytes_sym;
         for (int b = 0; b < N_BINS; b++) own->k_bytes[KID_BIN0 + b] += h_ctl->bytes_bin[b];
-        own->k_bytes[KID_COMMIT] += 20 * h_ctl->total_cand + 20 * h_ctl->total_delta +
+        own->k_bytes[KID_COMMIT] += 24 * h_ctl->total_cand + 12 * h_ctl->total_delta +
                                     8 * h_ctl->total_touched_out;
         own->k_bytes[KID_RESET] += 12 * h_ctl->total_touched_in;
         own->k_bytes[KID_CAPACITY] += 24 * h_ctl->total_touched_out + h_ctl->bytes_move[0];
         own->k_bytes[KID_CAPACITY_BIG] += h_ctl->bytes_move[1];
-        own->k_bytes[KID_SCATTER] += 60 * h_ctl->total_delta;
+        own->k_bytes[KID_SCATTER] += 4 * h_ctl->total_cand + 56 * h_ctl->total_delta;
         own->k_bytes[KID_PACK] += 24 * h_ctl->total_delta + 24 * h_ctl->total_touched_out;
     }
 };
