@@ -1635,9 +1635,29 @@ __global__ void __launch_bounds__(256) k_commit(SlotTab S, WorkBufs W, uint32_t 
 // merge: M <- M u dC in the row and column forms
 // ---------------------------------------------------------------------------
 
+// Whether some pair set could pass half full with this iteration's
+// candidates (CTA-collective).
+__device__ __forceinline__ bool sets_short(const SlotTab &S, uint32_t n_slots) {
+    bool grow = false;
+    for (uint32_t s = threadIdx.x; s < n_slots; s += blockDim.x)
+        grow |= 2 * (S.nnz[s] + S.cand[s]) > S.hmask[s] + 1;
+    return __syncthreads_or(grow);
+}
+
 // Rows that received entries in the previous merge stop being "new".
-__global__ void k_reset_dnew(SlotTab S, WorkBufs W) {
-    if (W.cnt->overflow & OVF_STOP) return;
+// check_slots > 0: before that, stop the iteration if some of so many pair
+// sets is too small (k_check's test, which every CTA makes for itself: none
+// may reset a row of an iteration that is stopped, and the counts it reads do
+// not change here; it was a launch of its own in every iteration).
+__global__ void __launch_bounds__(256) k_reset_dnew(SlotTab S, WorkBufs W, uint32_t check_slots) {
+    __shared__ unsigned stop;
+    if (threadIdx.x == 0) stop = W.cnt->overflow & OVF_STOP;
+    __syncthreads();
+    if (stop) return;
+    if (check_slots && sets_short(S, check_slots)) {
+        if (threadIdx.x == 0) atomicOr(&W.cnt->overflow, OVF_HASH);
+        return;
+    }
     const int par = *W.parity;
     const unsigned long long n_in = W.touched_n[par];
     const uint2 *t_in = W.touched[par];
@@ -2085,12 +2105,13 @@ __global__ void __launch_bounds__(256, 5) k_pack(SlotTab S, WorkBufs W) {
 // iteration frame (device-side checks; lets the loop run inside a CUDA graph)
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) k_iter_begin(SlotTab S, InstTab I, WorkBufs W,
-                                                    uint32_t n_slots, uint32_t n_inst) {
-    const int par = *W.parity;
+// Counters of an iteration back to zero (CTA-collective).
+__device__ __forceinline__ void zero_counters(const SlotTab &S, const InstTab &I,
+                                              const WorkBufs &W, uint32_t n_slots,
+                                              uint32_t n_inst, int out_list) {
     if (threadIdx.x == 0) {
         *W.cnt = Counters{};
-        W.touched_n[par ^ 1] = 0;
+        W.touched_n[out_list] = 0;
     }
     for (uint32_t s = threadIdx.x; s < n_slots; s += blockDim.x) {
         S.cand[s] = 0;
@@ -2099,26 +2120,31 @@ __global__ void __launch_bounds__(256) k_iter_begin(SlotTab S, InstTab I, WorkBu
     for (uint32_t k = threadIdx.x; k < n_inst; k += blockDim.x) I.delta[k] = 0;
 }
 
+__global__ void __launch_bounds__(256) k_iter_begin(SlotTab S, InstTab I, WorkBufs W,
+                                                    uint32_t n_slots, uint32_t n_inst) {
+    zero_counters(S, I, W, n_slots, n_inst, *W.parity ^ 1);
+}
+
 // Before the commit: stop the iteration if a buffer overflowed or if some
 // pair set could pass half full with this iteration's candidates.
-__global__ void __launch_bounds__(256) k_check(SlotTab S, WorkBufs W, uint32_t n_slots,
-                                               int growth) {
-    if (!growth) return;               // sets kept at their size (a test setting)
-    bool grow = false;
-    for (uint32_t s = threadIdx.x; s < n_slots; s += blockDim.x)
-        grow |= 2 * (S.nnz[s] + S.cand[s]) > S.hmask[s] + 1;
-    if (__syncthreads_or(grow) && threadIdx.x == 0) atomicOr(&W.cnt->overflow, OVF_HASH);
+__global__ void __launch_bounds__(256) k_check(SlotTab S, WorkBufs W, uint32_t n_slots) {
+    if (sets_short(S, n_slots) && threadIdx.x == 0) atomicOr(&W.cnt->overflow, OVF_HASH);
 }
 
 // After the merge: add the new pairs to the counts, advance every
-// instance's iteration count, flip the touched-list parity and decide
-// whether the closure loop goes on (Algorithm 1: while M is changing).
+// instance's iteration count, flip the touched-list parity, decide whether
+// the closure loop goes on (Algorithm 1: while M is changing) and zero the
+// counters for the next iteration (k_iter_begin does so only before the
+// first one and after a stopped one).
 __global__ void __launch_bounds__(256) k_iter_end(SlotTab S, InstTab I, WorkBufs W, LoopCtl *ctl,
                                                   uint32_t n_slots, uint32_t n_inst,
                                                   int count_iteration,
                                                   cudaGraphConditionalHandle handle,
                                                   int in_graph) {
-    const unsigned flags = W.cnt->overflow & (OVF_STOP | OVF_POOL);
+    __shared__ int out_list;
+    __shared__ unsigned flags;
+    if (threadIdx.x == 0) flags = W.cnt->overflow & (OVF_STOP | OVF_POOL);
+    __syncthreads();
     if (flags) {                        // the host grows a buffer and finishes the iteration
         if (threadIdx.x == 0) {
             ctl->status = flags;
@@ -2169,7 +2195,10 @@ __global__ void __launch_bounds__(256) k_iter_end(SlotTab S, InstTab I, WorkBufs
         const bool more = total > 0 && ctl->iter < ctl->limit &&
                           !(ctl->stop_on_converge && finished);
         if (in_graph) cudaGraphSetConditional(handle, more ? 1u : 0u);
+        out_list = par;                 // this iteration's rows are done with
     }
+    __syncthreads();
+    zero_counters(S, I, W, n_slots, n_inst, out_list);
 }
 
 // ---------------------------------------------------------------------------
@@ -3145,11 +3174,6 @@ void launch_iter_begin(const SlotTab &S, const InstTab &I, const WorkBufs &W, ui
     k_iter_begin<<<1, 256, 0, st>>>(S, I, W, n_slots, n_inst);
 }
 
-void launch_check(const SlotTab &S, const WorkBufs &W, uint32_t n_slots, bool growth,
-                  cudaStream_t st) {
-    k_check<<<1, 256, 0, st>>>(S, W, n_slots, growth ? 1 : 0);
-}
-
 void launch_iter_end(const SlotTab &S, const InstTab &I, const WorkBufs &W, LoopCtl *ctl,
                      uint32_t n_slots, uint32_t n_inst, bool count_iteration,
                      cudaGraphConditionalHandle handle, bool in_graph, cudaStream_t st) {
@@ -3157,10 +3181,16 @@ void launch_iter_end(const SlotTab &S, const InstTab &I, const WorkBufs &W, Loop
                                   in_graph ? 1 : 0);
 }
 
-void launch_reset_dnew(const SlotTab &S, const WorkBufs &W, int sms, cudaStream_t st) {
-    k_reset_dnew<<<sms * 4, 256, 0, st>>>(S, W);
-}
+// Slots up to which every CTA of the reset checks the pair sets itself (eight
+// per thread); more are checked by a launch of one CTA.
+constexpr uint32_t CHECK_SLOTS = 2048;
 
+void launch_check_reset(const SlotTab &S, const WorkBufs &W, uint32_t n_slots, bool check,
+                        int sms, cudaStream_t st) {
+    const bool own = check && n_slots > CHECK_SLOTS;
+    if (own) k_check<<<1, 256, 0, st>>>(S, W, n_slots);
+    k_reset_dnew<<<sms * 4, 256, 0, st>>>(S, W, check && !own ? n_slots : 0u);
+}
 
 void launch_capacity(const SlotTab &S, const InstTab &I, const WorkBufs &W, int sms,
                      cudaStream_t st) {

@@ -212,19 +212,21 @@ void launch_spgemm(int bin, const SlotTab &S, const ProdTab &P, const WorkBufs &
                    uint32_t max_n, const Tuning &T, int sms, cudaStream_t st);
 void launch_commit(const SlotTab &S, const WorkBufs &W, uint32_t n_slots, int sms,
                    cudaStream_t st);
-// Iteration frame: zero the per-iteration counters; check the pre-commit
-// conditions (buffer overflow, pair-set load); finish the iteration (pair
-// counts, per-instance iteration counts, parity flip, loop condition).
+// Iteration frame: zero the per-iteration counters (before the first
+// iteration and after a stopped one); finish the iteration (pair counts,
+// per-instance iteration counts, parity flip, loop condition, counters zeroed
+// for the next one).
 void launch_iter_begin(const SlotTab &S, const InstTab &I, const WorkBufs &W, uint32_t n_slots,
                        uint32_t n_inst, cudaStream_t st);
-// growth false (a test setting): never stop for a pair set's load, so a set
-// may fill up (the capped probes then report OVF_FULL)
-void launch_check(const SlotTab &S, const WorkBufs &W, uint32_t n_slots, bool growth,
-                  cudaStream_t st);
 void launch_iter_end(const SlotTab &S, const InstTab &I, const WorkBufs &W, LoopCtl *ctl,
                      uint32_t n_slots, uint32_t n_inst, bool count_iteration,
                      cudaGraphConditionalHandle handle, bool in_graph, cudaStream_t st);
-void launch_reset_dnew(const SlotTab &S, const WorkBufs &W, int sms, cudaStream_t st);
+// Check the pre-commit conditions (check: pair-set load; false for the
+// terminal initialisation, whose sets are sized for it, and in a test setting
+// in which a set may fill up and the capped probes report OVF_FULL), then end
+// the previous deltas.
+void launch_check_reset(const SlotTab &S, const WorkBufs &W, uint32_t n_slots, bool check,
+                        int sms, cudaStream_t st);
 // Room for every row the merge appends to (its new entries, and as many
 // tiles again): rows that must grow move to a new segment with their tiles
 // folded to one per word (one warp per row up to TILE_WARP_MAX tiles, then

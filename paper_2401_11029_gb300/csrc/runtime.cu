@@ -348,6 +348,61 @@ struct DevArr {           // device array owned by a context's accounting
     ~DevArr() { release(); }
 };
 
+// Streams beside the solve stream for launches that run side by side, and
+// the events that fork and join them.  A runner takes a set for its life and
+// gives it back; up to SIDE_KEEP sets per process wait for the next runner, so
+// that a context per small graph does not make streams each time.  A set in
+// use belongs to one runner, so contexts of several threads never share one;
+// everything launched on it is joined back to the solve stream, and a runner
+// is destroyed after its stream's work is done with.
+struct SideStreams {
+    int device = 0;
+    cudaStream_t s[N_BINS - 1] = {};
+    cudaEvent_t fork = nullptr, join[N_BINS - 1] = {};
+    ~SideStreams() {
+        for (cudaStream_t q : s)
+            if (q) cudaStreamDestroy(q);
+        for (cudaEvent_t e : join)
+            if (e) cudaEventDestroy(e);
+        if (fork) cudaEventDestroy(fork);
+    }
+};
+constexpr size_t SIDE_KEEP = 16;
+std::mutex g_side_mu;
+std::vector<SideStreams *> g_side_free;
+
+SideStreams *take_side(int device) {
+    {
+        std::lock_guard<std::mutex> lock(g_side_mu);
+        for (size_t k = 0; k < g_side_free.size(); k++) {
+            if (g_side_free[k]->device != device) continue;
+            SideStreams *x = g_side_free[k];
+            g_side_free.erase(g_side_free.begin() + k);
+            return x;
+        }
+    }
+    std::unique_ptr<SideStreams> x(new SideStreams());
+    x->device = device;
+    ck(cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming), "cudaEventCreate");
+    for (int q = 0; q < N_BINS - 1; q++) {
+        ck(cudaStreamCreateWithFlags(&x->s[q], cudaStreamNonBlocking), "cudaStreamCreate");
+        ck(cudaEventCreateWithFlags(&x->join[q], cudaEventDisableTiming), "cudaEventCreate");
+    }
+    return x.release();
+}
+
+void give_side(SideStreams *x) {
+    if (!x) return;
+    {
+        std::lock_guard<std::mutex> lock(g_side_mu);
+        if (g_side_free.size() < SIDE_KEEP) {
+            g_side_free.push_back(x);
+            return;
+        }
+    }
+    delete x;
+}
+
 // The closure-loop driver over one or more contexts (a batch).  Every
 // context's non-terminals get global slot ids; work items name slots, so
 // one launch sequence serves the whole batch.
@@ -406,6 +461,8 @@ struct Runner {
     cudaGraphExec_t gexec = nullptr;
     cudaGraphConditionalHandle handle = 0;
     bool graph_valid = false;
+    SideStreams *side = nullptr;       // for the product bins
+    bool side_broken = false;          // a capture on them failed
 
     explicit Runner(cflr_ctx *owner) : own(owner), st(owner->stream), sms(owner->sms) {
         prof.owner = own;
@@ -414,9 +471,12 @@ struct Runner {
         ck(cudaMallocHost(&h_cnt, sizeof(Counters)), "cudaMallocHost");
         ck(cudaMallocHost(&h_ctl, sizeof(LoopCtl)), "cudaMallocHost");
         ck(cudaMallocHost(&h_parity, sizeof(int)), "cudaMallocHost");
+        side = take_side(own->device);
     }
     ~Runner() {
         drop_graph();
+        if (side_broken) delete side;
+        else give_side(side);
         if (h_cnt) cudaFreeHost(h_cnt);
         if (h_ctl) cudaFreeHost(h_ctl);
         if (h_parity) cudaFreeHost(h_parity);
@@ -865,18 +925,39 @@ struct Runner {
             }
         } else {
             run(KID_SYMBOLIC, [&] { launch_symbolic(S, P, W, -1, tuning(), sms, st); });
-            for (int b = 0; b < N_BINS; b++)
-                run(KID_BIN0 + b, [&] { launch_spgemm(b, S, P, W, max_n, tuning(), sms, st); });
+            if (timed && prof.on) {       // one after another: each bin's own time
+                for (int b = 0; b < N_BINS; b++)
+                    run(KID_BIN0 + b,
+                        [&] { launch_spgemm(b, S, P, W, max_n, tuning(), sms, st); });
+                return;
+            }
+            // The bins share no group and only add to the candidate list, so
+            // they run side by side: each is bound by latency and ends in a
+            // few long groups, and the next one's blocks fill in as its own
+            // leave.  The heaviest kind of group (bin 3) starts first.  (200k
+            // alias solve 53.5 -> 48.9 ms, 500k points-to 108 -> 98.5, Dyck-1
+            // of 1000 vertices 2.1 -> 1.7, with two launches less a turn.)
+            ck(cudaEventRecord(side->fork, st), "fork");
+            for (int b = N_BINS - 1; b >= 0; b--) {
+                const int q = b - 1;          // bin 0 stays on the solve stream
+                cudaStream_t on = b ? side->s[q] : st;
+                if (b) ck(cudaStreamWaitEvent(on, side->fork, 0), "fork");
+                launch_spgemm(b, S, P, W, max_n, tuning(), sms, on);
+                ck(cudaGetLastError(), kKernelNames[KID_BIN0 + b]);
+                if (b) ck(cudaEventRecord(side->join[q], on), "join");
+            }
+            for (int q = 0; q < N_BINS - 1; q++)
+                ck(cudaStreamWaitEvent(st, side->join[q], 0), "join");
         }
     }
     // Commit and union, from the dedupe (stage 0), the capacity pass
     // (stage 1) or the scatter (stage 2), then the end of the iteration.
     void launch_merge(const SlotTab &S, const InstTab &I, const WorkBufs &W, int stage,
-                      bool count_iteration, bool in_graph, bool timed) {
+                      bool count_iteration, bool in_graph, bool timed, bool check) {
         auto run = [&](int kid, auto f) { if (timed) prof.run(kid, f); else f(); };
         if (stage <= 0) {
             // the previous deltas end before the commit counts the new ones
-            run(KID_RESET, [&] { launch_reset_dnew(S, W, sms, st); });
+            run(KID_RESET, [&] { launch_check_reset(S, W, n_slots, check, sms, st); });
             run(KID_COMMIT, [&] { launch_commit(S, W, n_slots, sms, st); });
         }
         if (stage <= 1) {
@@ -889,18 +970,21 @@ struct Runner {
                         handle, in_graph, st);
         ck(cudaGetLastError(), "k_iter_end");
     }
-    // One whole iteration as a launch sequence (also the graph's body).
+    // One whole iteration as a launch sequence (also the graph's body; the
+    // counters are zero when it starts).
     void launch_iteration(bool in_graph, bool timed) {
         const SlotTab S = slots();
         const ProdTab P = prodtab();
         const InstTab I = insttab();
         const WorkBufs W = work();
-        launch_iter_begin(S, I, W, n_slots, (uint32_t)cx.size(), st);
         launch_products(S, P, W, timed);
         bool growth = true;
         for (auto *c : cx) growth &= c->cfg.test_fixed_pair_sets == 0;
-        launch_check(S, W, n_slots, growth, st);
-        launch_merge(S, I, W, 0, true, in_graph, timed);
+        launch_merge(S, I, W, 0, true, in_graph, timed, growth);
+    }
+    void zero_counters() {
+        launch_iter_begin(slots(), insttab(), work(), n_slots, (uint32_t)cx.size(), st);
+        ck(cudaGetLastError(), "k_iter_begin");
     }
 
     void ensure_graph() {
@@ -921,8 +1005,15 @@ struct Runner {
         ck(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0,
                                          cudaStreamCaptureModeThreadLocal),
            "cudaStreamBeginCaptureToGraph");
-        launch_iteration(true, false);
         cudaGraph_t captured = nullptr;
+        try {
+            launch_iteration(true, false);
+        } catch (...) {
+            // end the capture; side streams caught in it go to nobody else
+            cudaStreamEndCapture(st, &captured);
+            side_broken = true;
+            throw;
+        }
         ck(cudaStreamEndCapture(st, &captured), "cudaStreamEndCapture");
         ck(cudaGraphInstantiate(&gexec, graph, 0), "cudaGraphInstantiate");
         graph_valid = true;
@@ -986,7 +1077,7 @@ struct Runner {
             }
             upload_htabs();
             clear_overflow();
-            launch_merge(S, I, W, 0, true, false, true);
+            launch_merge(S, I, W, 0, true, false, true, false);
             read_status();
         }
         for (int guard = 0; h_ctl->status & OVF_POOL; guard++) {   // grow pools, redo the union
@@ -998,7 +1089,7 @@ struct Runner {
                 if (top[k] > cx[k]->pool_cap) grow_pool(k, top[k]);
             upload_pools(false);
             clear_overflow();
-            launch_merge(S, I, W, 1, true, false, true);
+            launch_merge(S, I, W, 1, true, false, true, false);
             read_status();
         }
         if (h_ctl->status & OVF_FULL)
@@ -1019,6 +1110,7 @@ struct Runner {
         // them needs no growth, and only then captures the graph again (a
         // fresh context grows several buffers in its first iterations).
         bool settled = graph_valid;
+        zero_counters();
         for (;;) {
             if (use_graph && settled) {
                 Range range("cflr: closure loop (CUDA graph)");
@@ -1032,7 +1124,10 @@ struct Runner {
             }
             prof.collect();
             settled = h_ctl->status == 0;
-            if (h_ctl->status && !recover()) continue;
+            if (h_ctl->status && !recover()) {
+                zero_counters();
+                continue;
+            }
             if (h_ctl->last_delta == 0) return true;
             if (h_ctl->iter >= h_ctl->limit) return false;
             if (h_ctl->stop_on_converge && first_converged()) return false;
@@ -1532,7 +1627,7 @@ void reset_matrices(cflr_ctx *c) {
     c->k_bytes[KID_INIT] += 12 * c->m_edges + 12 * c->n_init;
     // the pair sets were sized from the exact initial counts, so the commit
     // needs no capacity check; the pool may still grow
-    r.launch_merge(S, I, W, 0, false, false, true);
+    r.launch_merge(S, I, W, 0, false, false, true, false);
     r.read_status();
     if (r.h_cnt->overflow & OVF_CAND) throw Status{CFLR_ECUDA, "internal: init overflow"};
     if (r.h_ctl->status) r.recover();
