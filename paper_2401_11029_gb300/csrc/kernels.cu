@@ -508,16 +508,23 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
     // members write different non-terminals probe their pair sets (there is
     // no single mask row) and stay in the hash bins (force_probe).
     bool acct = true;   // whether this lane adds the group's work and bytes
-    auto classify = [&](uint32_t code, uint32_t part, uint32_t idx, uint32_t d, uint32_t mlen,
-                        unsigned long long mbytes, unsigned long long f,
+    auto classify = [&](uint32_t code, uint32_t part, uint32_t idx, uint32_t n, uint32_t d,
+                        uint32_t mlen, unsigned long long mbytes, unsigned long long f,
                         unsigned long long fbytes, bool force_probe, uint2 &grp) -> int {
         const bool probe =
             force_probe || (unsigned long long)mlen > (unsigned long long)T.probe_ratio * f;
         const unsigned long long need = probe ? f : f + mlen;
-        const int b = need <= T.limit[0] ? 0 : need <= T.limit[1] ? 1 : need <= T.limit[2] ? 2 : 3;
+        int b = need <= T.limit[0] ? 0 : need <= T.limit[1] ? 1 : need <= T.limit[2] ? 2 : 3;
         // table of the smallest power of two >= 2*need slots (>= 32)
         uint32_t lg = 5;
         while (b < 3 && (1ull << lg) < 2 * need) lg++;
+        // A group of bins 1 and 2 whose table (8 bytes a slot) would be no
+        // smaller than the row's bitmap takes the bitmap: a tile then costs
+        // one shared-memory read instead of a probe sequence.  (Groups of
+        // bin 0 stay: a few tiles on one warp.)  With bin 1 on two warps a
+        // group, this took the 200k alias solve from 48.9 to 44.8 ms, the 100k
+        // one from 22.8 to 19.9 and the 20k one from 10.4 to 9.7.
+        if ((b == 1 || b == 2) && !force_probe && (n + 31) / 32 <= 2ull << lg) b = 3;
         grp = make_uint2(((code >> 2) << 8) | (lg << 3) | (probe ? MODE_PROBE : 0u) | part, idx);
         // algorithmic bytes: the delta entries (4 B each), the descriptor
         // (16 B) and tiles (8 B each) of every referenced row, and the mask
@@ -579,11 +586,11 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                     uint2 grp;
                     if (fm.z & FAM_CSHARED) {   // every member writes c: one mask row
                         const uint32_t mt = S.desc[pr0.x][r].y;
-                        emit(classify(code, PART_F, idx, d, mt, 8ull * mt, wk.f, wk.fb, false,
+                        emit(classify(code, PART_F, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false,
                                       grp),
                              grp);
                     } else if (wk.f <= T.limit[2]) {
-                        emit(classify(code, PART_F, idx, d, 0, 0, wk.f, wk.fb, true, grp), grp);
+                        emit(classify(code, PART_F, idx, n, d, 0, 0, wk.f, wk.fb, true, grp), grp);
                     } else {
                         // too large for a hash bin: one group per member,
                         // the threads taking the members
@@ -595,7 +602,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                             uint2 mg = make_uint2(0, 0);
                             if (i < fm.y && mf[i]) {
                                 const uint32_t mt = S.desc[P.prod[mp[i]].x][r].y;
-                                b = classify((mp[i] << 2) | fm.w, fm.w, idx, d, mt, 8ull * mt,
+                                b = classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt,
                                              mf[i], 16ull * mc[i] + 8ull * mf[i], false, mg);
                             }
                             if (cta) {
@@ -627,9 +634,9 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
             uint2 grp;
             if (fm.z & FAM_CSHARED) {   // every member writes c: one mask row
                 const uint32_t mt = S.desc[pr0.x][r].y;
-                emit(classify(code, PART_F, idx, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
+                emit(classify(code, PART_F, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
             } else if (wk.f <= T.limit[2]) {
-                emit(classify(code, PART_F, idx, d, 0, 0, wk.f, wk.fb, true, grp), grp);
+                emit(classify(code, PART_F, idx, n, d, 0, 0, wk.f, wk.fb, true, grp), grp);
             } else if (qstep == 32) {
                 // too large for a hash bin: one group per member; with a
                 // whole warp on the use, the lanes take the members (each
@@ -646,7 +653,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                         const Work wi = gathered_work(S, (fm.w == PART_A) ? pr.z : pr.y, o, n,
                                                       pool, dstart, d, 0, 1, &W.cnt->overflow);
                         if (wi.f)
-                            b = classify((mp[i] << 2) | fm.w, fm.w, idx, d, mt, 8ull * mt, wi.f,
+                            b = classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt, wi.f,
                                          wi.fb, false, mg);
                     }
                     append_lanes(b, mg);
@@ -658,7 +665,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                                                       q0, qstep, &W.cnt->overflow));
                     if (wi.f == 0) continue;
                     const uint32_t mt = S.desc[P.prod[mp[i]].x][r].y;
-                    emit(classify((mp[i] << 2) | fm.w, fm.w, idx, d, mt, 8ull * mt, wi.f, wi.fb,
+                    emit(classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt, wi.f, wi.fb,
                                   false, grp),
                          grp);
                 }
@@ -678,7 +685,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
         }
         if (wk.f == 0) return;
         uint2 grp;
-        emit(classify(code, part, idx, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
+        emit(classify(code, part, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
     };
 
     if (mode == 1) {
@@ -1347,11 +1354,11 @@ __device__ __forceinline__ void preload_mask(const SlotTab &S, const GroupInfo &
     }
 }
 
-// Bins 0 and 1: one warp per group, a private shared-memory table per warp
-// (2^LG words and their bits).
+// Bin 0: one warp per group, a private shared-memory table per warp (2^LG
+// words and their bits).
 template <int LG, int WARPS, bool WIT>
-__global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 4 : 3) k_spgemm_warp(SlotTab S, ProdTab P, WorkBufs W,
-                                                            int bin) {
+__global__ void __launch_bounds__(WARPS * 32, 4) k_spgemm_warp(SlotTab S, ProdTab P, WorkBufs W,
+                                                               int bin) {
     extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     uint32_t *tab = smem + (size_t)wib * (2u << LG);
@@ -1384,46 +1391,62 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 4 : 3) k_spgemm_warp(
     if (lane == 0 && bytes) atomicAdd(&W.cnt->bytes_bin[bin], bytes);
 }
 
-// Bin 2: one CTA per group sharing a 2^LG-word shared-memory table.
-template <int LG, bool WIT>
-__global__ void __launch_bounds__(256, LG == 12 ? 4 : 3) k_spgemm_cta(SlotTab S, ProdTab P, WorkBufs W, int bin) {
+// Bins 1 and 2: a CTA's PARTS equal parts take a group each, with a 2^LG-slot
+// table per part in shared memory and a named barrier of their own.  Bin 2's
+// groups take the whole CTA.  Bin 1's take two warps: with a warp each and
+// 16 KB tables an SM held 12 warps, and a launch of few groups (most of a
+// solve's iterations) waited for one warp walking a group of up to a thousand
+// tiles (70 us on the 61k-vertex points-to graph, 0.3 % of the issue slots).
+// Bin 1 of the 500k points-to solve: 18.9 -> 12.6 ms, of the 200k alias solve
+// 7.9 -> 4.8.
+template <int LG, int PARTS, bool WIT, bool PACKED>
+__global__ void __launch_bounds__(256, (PARTS << LG) > 6144 ? 3 : 4)
+    k_spgemm_part(SlotTab S, ProdTab P, WorkBufs W, int bin) {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ uint32_t emitted_sh;
+    __shared__ uint32_t emitted_sh[PARTS];
+    __shared__ unsigned long long next_sh[PARTS][2];
+    constexpr int TPG = 256 / PARTS;                  // threads per group
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    __shared__ unsigned long long next_sh[2];
+    const int part = threadIdx.x / TPG, ptid = threadIdx.x % TPG;
+    auto psync = [&]() {
+        if (PARTS == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(part + 1), "r"(TPG) : "memory");
+    };
+    uint32_t *tab = smem + (size_t)part * (2u << LG);
     const unsigned long long n_groups = min(W.cnt->groups[bin], W.group_cap[bin]);
+    if (n_groups == 0) return;
     CandChunk ck{0, 0};
     unsigned long long bytes = 0;
     // groups are claimed one at a time from a cursor (their sizes vary a
     // lot), the next one while the current one starts
-    if (threadIdx.x == 0) next_sh[0] = atomicAdd(&W.cnt->claim[bin], 1ull);
-    __syncthreads();
-    unsigned long long g = next_sh[0];
+    if (ptid == 0) next_sh[part][0] = atomicAdd(&W.cnt->claim[bin], 1ull);
+    psync();
+    unsigned long long g = next_sh[part][0];
     for (uint32_t q = 1; g < n_groups; q ^= 1) {
         const GroupInfo gi = decode_group(P, S, W.groups[bin][g]);
         const int lg = min((int)gi.lg, LG);
-        clear_table(smem, lg, threadIdx.x, blockDim.x);
-        if (threadIdx.x == 0) {
-            emitted_sh = 0;
-            next_sh[q] = atomicAdd(&W.cnt->claim[bin], 1ull);
+        clear_table(tab, lg, ptid, TPG);
+        if (ptid == 0) {
+            emitted_sh[part] = 0;
+            next_sh[part][q] = atomicAdd(&W.cnt->claim[bin], 1ull);
         }
-        __syncthreads();
-        const HashAcc acc{smem, lg, &W.cnt->overflow};
-        if (!gi.probe) preload_mask(S, gi, acc, threadIdx.x, blockDim.x, &W.cnt->overflow);
-        __syncthreads();
+        psync();
+        const HashAcc acc{tab, lg, &W.cnt->overflow};
+        if (!gi.probe) preload_mask(S, gi, acc, ptid, TPG, &W.cnt->overflow);
+        psync();
         const uint2 own = owner_delta(S, gi, &W.cnt->overflow);
-        const uint32_t e = expand_rows<WIT, true, true, 2>(S, P, W, gi, own, wib,
-                                                            blockDim.x >> 5, lane, acc, ck);
-        if (lane == 0 && e) atomicAdd(&emitted_sh, e);
-        __syncthreads();
-        if (threadIdx.x == 0 && emitted_sh) {
-            if (!gi.tagged) atomicAdd(&S.cand[gi.c], (unsigned long long)emitted_sh);
-            bytes += 12ull * emitted_sh;
+        const uint32_t e = expand_rows<WIT, true, PACKED, 2>(S, P, W, gi, own, wib % (8 / PARTS),
+                                                             8 / PARTS, lane, acc, ck);
+        if (lane == 0 && e) atomicAdd(&emitted_sh[part], e);
+        psync();
+        if (ptid == 0 && emitted_sh[part]) {
+            if (!gi.tagged) atomicAdd(&S.cand[gi.c], (unsigned long long)emitted_sh[part]);
+            bytes += 12ull * emitted_sh[part];
         }
-        g = next_sh[q];
+        g = next_sh[part][q];
     }
     release_chunk(W, ck, lane);
-    if (threadIdx.x == 0 && bytes) atomicAdd(&W.cnt->bytes_bin[bin], bytes);
+    if (ptid == 0 && bytes) atomicAdd(&W.cnt->bytes_bin[bin], bytes);
 }
 
 // Bin 3: one CTA per group with an n-bit bitmap of the output row (shared
@@ -1454,6 +1477,7 @@ __global__ void __launch_bounds__(256, 4) k_spgemm_bitmap(SlotTab S, ProdTab P, 
 #else
     const BitmapAcc acc{bm};
 #endif
+    if (n_groups == 0) return;
     CandChunk ck{0, 0};
     unsigned long long bytes = 0;
     // each part claims groups one at a time from a cursor (their sizes vary
@@ -3066,23 +3090,24 @@ static inline int grid_for(unsigned long long work, int per_block, int sms, int 
 
 // tables of words and bits: 2 x 4 bytes per slot
 constexpr size_t BIN0_SMEM = 8 * 2 * 256 * 4;    // 8 warps x 256 slots
-constexpr size_t BIN1_SMEM = 4 * 2 * 2048 * 4;   // 4 warps x 2048 slots
-constexpr size_t BIN1S_SMEM = 8 * 2 * 1024 * 4;  // 8 warps x 1024 slots (limit <= 512)
+constexpr size_t BIN1_SMEM = 4 * 2 * 2048 * 4;   // 4 parts x 2048 slots
+constexpr size_t BIN1S_SMEM = 4 * 2 * 1024 * 4;  // 4 parts x 1024 slots (limit <= 512)
 constexpr size_t BIN2_SMEM = 2 * 8192 * 4;
 constexpr size_t BIN2S_SMEM = 2 * 4096 * 4;       // limit <= 2048
 constexpr size_t SMEM_BITMAP_MAX = 200 * 1024;
+// Bin 1 walks list by list: the packed walk took 93.3 ms for the 500k-vertex
+// points-to solve against 91.9, and 44.5 against 44.8 for the 200k alias solve.
+constexpr bool BIN1_PACKED = false;
 
 static void set_smem_attrs();
 void prepare_launch_attributes() { set_smem_attrs(); }
 
 template <bool WIT>
 static void set_bin_smem_attrs() {
-    cudaFuncSetAttribute(k_spgemm_warp<11, 4, WIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)BIN1_SMEM);
-    cudaFuncSetAttribute(k_spgemm_cta<13, WIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)BIN2_SMEM);
-    cudaFuncSetAttribute(k_spgemm_warp<10, 8, WIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)BIN1S_SMEM);
+    cudaFuncSetAttribute(k_spgemm_part<11, 4, WIT, BIN1_PACKED>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIN1_SMEM);
+    cudaFuncSetAttribute(k_spgemm_part<13, 1, WIT, true>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIN2_SMEM);
     cudaFuncSetAttribute(k_spgemm_bitmap<WIT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)SMEM_BITMAP_MAX);
     cudaFuncSetAttribute(k_spgemm_bitmap<WIT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -3127,15 +3152,19 @@ static void launch_bin(int bin, const SlotTab &S, const ProdTab &P, const WorkBu
         break;
     case 1:   // the smaller table when the limit allows it: more warps per SM
         if (T.limit[1] <= 512)
-            k_spgemm_warp<10, 8, WIT><<<sms * T.ctas_per_sm[1], 256, BIN1S_SMEM, st>>>(S, P, W, 1);
+            k_spgemm_part<10, 4, WIT, BIN1_PACKED>
+                <<<sms * T.ctas_per_sm[1], 256, BIN1S_SMEM, st>>>(S, P, W, 1);
         else
-            k_spgemm_warp<11, 4, WIT><<<sms * T.ctas_per_sm[1], 128, BIN1_SMEM, st>>>(S, P, W, 1);
+            k_spgemm_part<11, 4, WIT, BIN1_PACKED>
+                <<<sms * T.ctas_per_sm[1], 256, BIN1_SMEM, st>>>(S, P, W, 1);
         break;
     case 2:
         if (T.limit[2] <= 2048)
-            k_spgemm_cta<12, WIT><<<sms * T.ctas_per_sm[2], 256, BIN2S_SMEM, st>>>(S, P, W, 2);
+            k_spgemm_part<12, 1, WIT, true>
+                <<<sms * T.ctas_per_sm[2], 256, BIN2S_SMEM, st>>>(S, P, W, 2);
         else
-            k_spgemm_cta<13, WIT><<<sms * T.ctas_per_sm[2], 256, BIN2_SMEM, st>>>(S, P, W, 2);
+            k_spgemm_part<13, 1, WIT, true>
+                <<<sms * T.ctas_per_sm[2], 256, BIN2_SMEM, st>>>(S, P, W, 2);
         break;
     default: {
         // bitmap words rounded to 16 bytes; two groups per CTA when four CTAs
