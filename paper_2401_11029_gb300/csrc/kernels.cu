@@ -256,7 +256,7 @@ __device__ __forceinline__ unsigned long long block_excl_scan256(unsigned long l
 // k_symbolic: groups of this iteration, binned by shared-memory need
 // ---------------------------------------------------------------------------
 
-constexpr int SYM_BUF = 16;   // per-warp staging of groups before one atomic
+constexpr int SYM_BUF = 48;   // per-warp staging of groups before one atomic (a turn adds 32)
 
 // Product steps (referenced tiles) of one use and their bytes, over the
 // delta entries q0, q0 + qstep, ... (pool[dstart + q], q < d): each entry k
@@ -447,17 +447,33 @@ __device__ __forceinline__ Work warp_sum(Work w) {
 }
 
 // prod_only >= 0 restricts the work list to one production (the plain form).
-// Mode 0: a warp per touched row; a row whose delta has more than SYM_BIG_D
+// MODE 0: a warp per touched row; a row whose delta has more than SYM_BIG_D
 // entries, or more than SYM_MIN_D entries and more than SYM_BIG_W descriptor
 // reads (entries times the members of its uses, a use of one production
-// counting as one), is listed for mode 1 (while the list has room) instead.
-// Mode 1: a CTA per listed row, its threads sharing the entries (a long
+// counting as one), is listed for MODE 1 (while the list has room) instead.
+// MODE 1: a CTA per listed row, its threads sharing the entries (a long
 // delta row on one warp would hold the launch up long after the other warps
 // finish).
+// Bound by the latency of dependent loads (list entry -> row descriptor ->
+// entries -> occupancy words -> referenced descriptors) and by the
+// instructions per use.  So a warp takes up to 32 rows at a time and its
+// lanes load their descriptors together; then the (row, use, entry) triples of
+// the rows of up to 32 entries are laid out over the lanes, as many whole
+// uses as fit a turn whichever rows they belong to, and a segmented sum gives
+// every use its product steps; longer rows take the warp, a use at a time.
+// The referenced words and descriptors are shared through the L1 cache, so
+// shared memory is kept small (14 KB more of it cost 10 to 20 %), and three
+// CTAs per SM without spills were no slower than four with them.
+// A use per turn, with 64-bit sums over the whole warp and a pass over 64
+// members' counters for a family, took 25.5 ms of the 500k-vertex points-to
+// solve (six entries a row on average), 5.0 ms of the 200k-vertex alias solve
+// (36 entries) and 2.2 ms of 64 batched Dyck-3 instances; now 15.4, 4.0 and
+// 1.0.
 constexpr uint32_t SYM_BIG_D = 1024, SYM_MIN_D = 64, SYM_BIG_W = 32768;
 
-__global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkBufs W,
-                                                     int prod_only, Tuning T, int mode) {
+template <int MODE>
+__global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkBufs W,
+                                                     int prod_only, Tuning T) {
     __shared__ Work red[8];
     __shared__ unsigned long long mem_f[8][64];   // per-member sums of a family (a warp's)
     __shared__ uint32_t mem_c[8][64];
@@ -466,39 +482,55 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
     const int par = *W.parity;
     const unsigned long long n_in = W.touched_n[par];
     const uint2 *t_in = W.touched[par];
-    int fill[N_BINS] = {0, 0, 0, 0};
-    unsigned long long bytes[N_BINS] = {0, 0, 0, 0};
-    unsigned long long flops = 0, sym_bytes = 0;
-    unsigned long long flops3 = 0, mask3 = 0;   // the bitmap bin's product and mask tiles
+    int fill[N_BINS] = {0, 0, 0, 0};              // staged groups (the same in every lane)
+    // each thread's work and byte counts, in shared memory (seven 64-bit
+    // counts in registers made the rest spill): the bins' bytes, product
+    // steps, bytes of this pass, the bitmap bin's product and mask tiles.
+    // 32 bits each, what goes beyond them added to the global count at once.
+    enum { ACC_FLOPS = N_BINS, ACC_SYM, ACC_FLOPS3, ACC_MASK3, N_ACC };
+    __shared__ uint32_t acc_sh[N_ACC][256];
+    for (int q = 0; q < N_ACC; q++) acc_sh[q][threadIdx.x] = 0;
+    auto total_of = [&](int q) -> unsigned long long * {
+        return q < N_BINS ? &W.cnt->bytes_bin[q]
+               : q == ACC_FLOPS ? &W.cnt->flops
+               : q == ACC_SYM ? &W.cnt->bytes_sym
+                              : &W.cnt->tiles_bin3[q - ACC_FLOPS3];
+    };
+    auto add = [&](int q, unsigned long long v) {
+        const unsigned long long t = acc_sh[q][threadIdx.x] + v;
+        acc_sh[q][threadIdx.x] = (uint32_t)t;
+        if (t >> 32) atomicAdd(total_of(q), t & ~0xFFFFFFFFull);
+    };
 
-    auto flush = [&](int b) {   // lane 0 only
-        unsigned long long pos = atomicAdd(&W.cnt->groups[b], (unsigned long long)fill[b]);
-        for (int q = 0; q < fill[b]; q++) {
-            if (pos + q < W.group_cap[b]) W.groups[b][pos + q] = stage[wib][b][q];
+    // warp-collective: the staged groups of bin b to the list, one atomic
+    auto flush = [&](int b, int n) {
+        __syncwarp();
+        unsigned long long pos = 0;
+        if (lane == 0) {
+            pos = atomicAdd(&W.cnt->groups[b], (unsigned long long)n);
+            if (pos + n > W.group_cap[b]) atomicOr(&W.cnt->overflow, OVF_GROUPS);
         }
-        if (pos + fill[b] > W.group_cap[b]) atomicOr(&W.cnt->overflow, OVF_GROUPS);
-        fill[b] = 0;
+        pos = __shfl_sync(FULL_MASK, pos, 0);
+        for (int q = lane; q < n; q += 32)
+            if (pos + q < W.group_cap[b]) W.groups[b][pos + q] = stage[wib][b][q];
+        __syncwarp();
     };
     auto append = [&](int b, uint2 grp) {   // one group, any lane
         const unsigned long long pos = atomicAdd(&W.cnt->groups[b], 1ull);
         if (pos < W.group_cap[b]) W.groups[b][pos] = grp;
         else atomicOr(&W.cnt->overflow, OVF_GROUPS);
     };
-    // warp-collective: each lane's group (bin b >= 0) appended, one atomic
-    // per bin
-    auto append_lanes = [&](int b, uint2 grp) {
+    // warp-collective: each lane's group (bin b >= 0) staged
+    auto stage_lanes = [&](int b, uint2 grp) {
 #pragma unroll
         for (int bb = 0; bb < N_BINS; bb++) {
             const unsigned m = __ballot_sync(FULL_MASK, b == bb);
             if (!m) continue;
-            const int leader = __ffs(m) - 1;
-            unsigned long long pos = 0;
-            if (lane == leader) pos = atomicAdd(&W.cnt->groups[bb], (unsigned long long)__popc(m));
-            pos = __shfl_sync(FULL_MASK, pos, leader);
-            if (b == bb) {
-                pos += __popc(m & ((1u << lane) - 1));
-                if (pos < W.group_cap[bb]) W.groups[bb][pos] = grp;
-                else atomicOr(&W.cnt->overflow, OVF_GROUPS);
+            if (b == bb) stage[wib][bb][fill[bb] + __popc(m & ((1u << lane) - 1))] = grp;
+            fill[bb] += __popc(m);
+            if (fill[bb] > SYM_BUF - 32) {
+                flush(bb, fill[bb]);
+                fill[bb] = 0;
             }
         }
     };
@@ -530,12 +562,12 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
         // (16 B) and tiles (8 B each) of every referenced row, and the mask
         // row's descriptor and tiles when it is loaded
         if (acct) {
-            bytes[b] += 4ull * d + fbytes + (probe ? 0ull : mbytes + 16ull);
-            sym_bytes += 20ull * d + 40ull;
-            flops += f;
+            add(b, 4ull * d + fbytes + (probe ? 0ull : mbytes + 16ull));
+            add(ACC_SYM, 20ull * d + 40ull);
+            add(ACC_FLOPS, f);
             if (b == 3) {
-                flops3 += f;
-                mask3 += probe ? 0ull : mlen;
+                add(ACC_FLOPS3, f);
+                add(ACC_MASK3, probe ? 0ull : mlen);
             }
         }
         return b;
@@ -608,7 +640,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                             if (cta) {
                                 if (b >= 0) append(b, mg);
                             } else {
-                                append_lanes(b, mg);
+                                stage_lanes(b, mg);
                             }
                         }
                         acct = keep_acct;
@@ -656,7 +688,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                             b = classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt, wi.f,
                                          wi.fb, false, mg);
                     }
-                    append_lanes(b, mg);
+                    stage_lanes(b, mg);
                 }
                 acct = keep_acct;
             } else {               // too large for a hash bin: one group per member
@@ -688,7 +720,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
         emit(classify(code, part, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
     };
 
-    if (mode == 1) {
+    if constexpr (MODE == 1) {
         // a CTA per long delta row: the threads share its entries, sums over
         // the CTA, thread 0 classifies and appends
         const unsigned long long n_big = min(W.cnt->big_n, W.big_cap);
@@ -715,7 +747,7 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
             const uint32_t dstart = dsc.x + tile_words(dsc.z);
             const uint32_t *pool = S.pool[slot];
             for (uint32_t u = P.use_off[xo]; u < P.use_off[xo + 1]; u++) {
-                const uint32_t code = P.use_code[u];
+                const uint32_t code = P.use_rec[u].x;
                 if (prod_only >= 0 && (code >> 2) != (uint32_t)prod_only) continue;
                 use_groups(code, o, n, idx, pool, dstart, d, threadIdx.x, 256, block_sum,
                            [&](int bb, uint2 g) {
@@ -723,101 +755,283 @@ __global__ void __launch_bounds__(256, 4) k_symbolic(SlotTab S, ProdTab P, WorkB
                            });
             }
         }
-    }
-    // a warp per touched row, at a stride: rows the same merge touched lie
-    // together in the list and often cost alike (claiming runs of rows from
-    // a cursor was measured slower, more so the longer the runs)
-    for (unsigned long long e = (unsigned long long)blockIdx.x * 8 + wib; mode == 0 && e < n_in;
-         e += (unsigned long long)gridDim.x * 8) {
-        const uint2 t = t_in[e];
-        const uint32_t xo = t.x, idx = t.y, slot = xo >> 1, o = xo & 1;
-        const uint32_t n = S.n[slot];
-        const uint4 dsc = S.desc[slot][(size_t)o * n + idx];
-        const uint32_t d = S.dn[slot][(size_t)o * n + idx].x;
-        const uint32_t dstart = dsc.x + tile_words(dsc.z);
-        const uint32_t *pool = S.pool[slot];
-        const uint32_t u0 = P.use_off[xo], u1 = P.use_off[xo + 1];
-        bool big = d > SYM_BIG_D;
-        if (!big && d > SYM_MIN_D) {
-            uint32_t w = 0;
-            for (uint32_t u = u0 + lane; u < u1; u += 32) {
-                const uint32_t code = P.use_code[u];
-                w += (code & 3) == PART_F ? P.fam[code >> 2].y : 1u;
+    } else {
+        // Batches of up to 32 rows at a stride (rows the same merge touched
+        // lie together in the list and often cost alike: claiming runs of
+        // neighbouring rows was measured slower, more so the longer the
+        // runs), the first one by the warp's number and the others claimed:
+        // with fixed shares the last warps ran long after the first ones
+        // (warps active 34 % of the launch, of 50 % that fit).
+        const unsigned long long nw = (unsigned long long)gridDim.x * 8;
+        const unsigned long long per = (n_in + 4 * nw - 1) / (4 * nw);
+        const uint32_t B = per > 32 ? 32u : per < 1 ? 1u : (uint32_t)per;
+        const unsigned long long nb = (n_in + B - 1) / B;
+        unsigned long long c = (unsigned long long)blockIdx.x * 8 + wib, c_next = nb;
+        for (; c < nb; c = __shfl_sync(FULL_MASK, c_next, 0)) {
+            // (claimed while this batch runs)
+            if (nb > nw && lane == 0) c_next = nw + atomicAdd(&W.cnt->claim[N_BINS], 1ull);
+            uint2 mt = make_uint2(0, 0);            // this lane's row
+            uint32_t m_n = 0, m_dstart = 0, m_d = 0, m_u0 = 0, m_u1 = 0;
+            const unsigned long long e = c + lane * nb;
+            const bool has = (uint32_t)lane < B && e < n_in;
+            if (has) {
+                mt = t_in[e];
+                const uint32_t slot = mt.x >> 1;
+                m_n = S.n[slot];
+                const size_t r = (size_t)(mt.x & 1) * m_n + mt.y;
+                const uint4 dsc = S.desc[slot][r];
+                m_d = S.dn[slot][r].x;
+                m_dstart = dsc.x + tile_words(dsc.z);
+                m_u0 = P.use_off[mt.x];
+                m_u1 = m_d ? P.use_off[mt.x + 1] : m_u0;
             }
-            big = (unsigned long long)__reduce_add_sync(FULL_MASK, w) * d > SYM_BIG_W;
-        }
-        if (big && u1 > u0) {
-            // listed for the CTA pass when there is room, else done here
-            unsigned long long pos = 0;
-            if (lane == 0) pos = atomicAdd(&W.cnt->big_n, 1ull);
-            pos = __shfl_sync(FULL_MASK, pos, 0);
-            if (pos < W.big_cap) {
-                if (lane == 0) W.big_rows[pos] = t;
-                continue;
-            }
-        }
-        if (u1 - u0 >= 32 && d <= 16) {
-            // many productions read this row, each with few products: one
-            // lane per use, groups appended with one atomic per bin
-            for (uint32_t ub = u0; ub < u1; ub += 32) {
-                const uint32_t u = ub + lane;
+            const int rows = __popc(__ballot_sync(FULL_MASK, has));   // the first lanes
+            // a use of a row by the whole warp, which shares the entries:
+            // wide or scattered families, and families that split
+            auto warp_use = [&](uint32_t code, uint32_t xo, uint32_t idx, uint32_t dstart,
+                                uint32_t d) {
+                acct = lane == 0;
+                use_groups(code, xo & 1, S.n[xo >> 1], idx, S.pool[xo >> 1], dstart, d, lane, 32,
+                           [](Work w) { return warp_sum(w); },
+                           [&](int bb, uint2 g) { stage_lanes(lane == 0 ? bb : -1, g); });
+            };
+            // product steps f and referenced rows cnt of entry k under `rec`
+            // (narrow: at most 64 members on consecutive slots; the slots of
+            // an instance follow one another, and so do their descriptors, 2n
+            // each), the members' descriptors four at a time
+            auto entry_work = [&](uint4 rec, uint32_t slot, uint32_t o, uint32_t n,
+                                  const uint4 *db, uint32_t k, unsigned long long &f,
+                                  uint32_t &cnt) {
+                const uint32_t F = rec.w & USE_MEMBERS;
+                const long long dg = (long long)rec.z - slot;
+                const uint32_t l0 = (uint32_t)(S.local[slot] + dg), l1 = l0 + F;
+                const uint32_t w0 = l0 >> 5, wl = (l1 - 1) >> 5, sh = l0 & 31;
+                const uint32_t *ok = S.occ[slot] + ((size_t)o * n + k) * S.occ_w[slot];
+                const uint4 *rows_k = db + dg * 2 * (long long)n + k;
+                const uint32_t x0 = ok[w0];
+                if (F == 1) {
+                    if ((x0 >> sh) & 1u) {
+                        const uint4 gd = *rows_k;
+                        f += gd.y - (o ? (gd.w & DLAST_MASK) : 0u);
+                        cnt++;
+                    }
+                    return;
+                }
+                const uint32_t x1 = w0 < wl ? ok[w0 + 1] : 0u, x2 = w0 + 1 < wl ? ok[w0 + 2] : 0u;
+                const unsigned long long lo64 = ((unsigned long long)x1 << 32) | x0;
+                unsigned long long m = (lo64 >> sh) | (sh ? (unsigned long long)x2 << (64 - sh) : 0);
+                if (F < 64) m &= (1ull << F) - 1;
+                cnt += __popcll(m);
+                while (m) {
+                    uint4 gd[4];
+#pragma unroll
+                    for (int t = 0; t < 4; t++) {
+                        gd[t] = make_uint4(0, 0, 0, 0);
+                        if (m) gd[t] = rows_k[(size_t)(2 * (__ffsll((long long)m) - 1)) * n];
+                        m &= m - 1;               // (0 & -1 stays 0)
+                    }
+#pragma unroll
+                    for (int t = 0; t < 4; t++) f += gd[t].y - (o ? (gd[t].w & DLAST_MASK) : 0u);
+                }
+            };
+            // the group of a use with its sums: staged, or left to warp_use
+            // (true) when a family splits into its members; lanes without a
+            // use to finish pass lead = false
+            auto finish = [&](bool lead, uint4 rec, uint32_t idx, uint32_t n, uint32_t d,
+                              uint32_t mtiles, unsigned long long f, uint32_t cnt) -> bool {
                 int b = -1;
                 uint2 grp = make_uint2(0, 0);
-                if (u < u1) {
-                    const uint32_t code = P.use_code[u];
-                    if (prod_only < 0 || (code >> 2) == (uint32_t)prod_only) {
+                bool split = false;
+                if (lead && f) {
+                    const uint32_t part = rec.x & 3;
+                    const bool tagged = part == PART_F && !(rec.w & USE_SHARED);
+                    if (tagged && f > T.limit[2]) {
+                        split = true;
+                    } else {
                         acct = true;
-                        // a use yields at most one group, except a split
-                        // family, whose member groups are appended at once
-                        bool one = true;
-                        use_groups(code, o, n, idx, pool, dstart, d, 0, 1,
-                                   [](Work w) { return w; },
-                                   [&](int bb, uint2 g) {
-                                       if (one && b < 0) {
-                                           b = bb;
-                                           grp = g;
-                                       } else {
-                                           append(bb, g);
-                                       }
-                                       one = false;
-                                   });
+                        b = classify(rec.x, part, idx, n, d, mtiles, 8ull * mtiles, f,
+                                     part == PART_U ? 4ull * d : 16ull * cnt + 8ull * f, tagged,
+                                     grp);
                     }
                 }
-                append_lanes(b, grp);
+                stage_lanes(b, grp);
+                return split;
+            };
+            auto is_slow = [](uint4 rec) {
+                return (rec.x & 3) == PART_F && !(rec.w & USE_NARROW);
+            };
+            auto wanted = [&](uint4 rec) {
+                return prod_only < 0 || (rec.x >> 2) == (uint32_t)prod_only;
+            };
+            int l = 0;                              // first row with uses left
+            uint32_t u_at = __shfl_sync(FULL_MASK, m_u0, 0);   // its next use
+            while (l < rows) {
+                // lay whole uses out over the lanes: d lanes a use
+                int my_row = -1;
+                uint32_t my_u0 = 0, my_at = 0, at = 0;
+                while (l < rows) {
+                    const uint32_t u1 = __shfl_sync(FULL_MASK, m_u1, l);
+                    const uint32_t d = __shfl_sync(FULL_MASK, m_d, l);
+                    const uint32_t t = d <= 32 ? min(u1 - u_at, (32 - at) / d) : 0u;
+                    if (t && (uint32_t)lane >= at && (uint32_t)lane < at + t * d) {
+                        my_row = l;
+                        my_u0 = u_at;
+                        my_at = at;
+                    }
+                    at += t * d;
+                    u_at += t;
+                    if (u_at < u1) break;           // no room, or a long row
+                    l++;
+                    u_at = __shfl_sync(FULL_MASK, m_u0, l & 31);
+                }
+                // the use a lane finishes (in the lanes with lead), its row and
+                // its sums
+                uint4 rec = make_uint4(0, 0, 0, 0);
+                uint32_t xo, idx, n, d, dstart, cnt = 0, mtiles = 0;
+                unsigned long long f = 0;
+                bool lead, slow;
+                if (at == 0 && l < rows) {
+                    // a longer row: a use at a time, 32 entries a step
+                    xo = __shfl_sync(FULL_MASK, mt.x, l);
+                    idx = __shfl_sync(FULL_MASK, mt.y, l);
+                    n = __shfl_sync(FULL_MASK, m_n, l);
+                    d = __shfl_sync(FULL_MASK, m_d, l);
+                    dstart = __shfl_sync(FULL_MASK, m_dstart, l);
+                    const uint32_t slot = xo >> 1, o = xo & 1;
+                    const uint32_t u0 = u_at, u1 = __shfl_sync(FULL_MASK, m_u1, l);
+                    const bool starts = u0 == __shfl_sync(FULL_MASK, m_u0, l);
+                    bool big = starts && d > SYM_BIG_D;
+                    if (starts && !big && d > SYM_MIN_D) {
+                        uint32_t w = 0;
+                        for (uint32_t u = u0 + lane; u < u1; u += 32)
+                            w += P.use_rec[u].w & USE_MEMBERS;
+                        big = (unsigned long long)__reduce_add_sync(FULL_MASK, w) * d > SYM_BIG_W;
+                    }
+                    if (big) {
+                        // listed for the CTA pass when there is room, else done here
+                        unsigned long long pos = 0;
+                        if (lane == 0) pos = atomicAdd(&W.cnt->big_n, 1ull);
+                        pos = __shfl_sync(FULL_MASK, pos, 0);
+                        big = pos < W.big_cap;
+                        if (big && lane == 0) W.big_rows[pos] = make_uint2(xo, idx);
+                    }
+                    u_at = big ? u1 : u0 + 1;
+                    if (u_at >= u1) {
+                        l++;
+                        u_at = __shfl_sync(FULL_MASK, m_u0, l & 31);
+                    }
+                    if (big) continue;
+                    const uint32_t *ent = S.pool[slot] + dstart;
+                    const uint4 *db = S.desc[slot] + (size_t)o * n;
+                    rec = P.use_rec[u0];
+                    const bool act = wanted(rec);
+                    if (act && (rec.w & USE_MEMBERS) == 1 && (rec.x & 3) < PART_U) {
+                        // one production: four entries a lane in flight
+                        const long long dg = (long long)rec.z - slot;
+                        const uint32_t lx = (uint32_t)(S.local[slot] + dg), ow = S.occ_w[slot];
+                        const uint32_t *ok = S.occ[slot] + (size_t)o * n * ow + (lx >> 5);
+                        const uint4 *gd = db + dg * 2 * (long long)n;
+                        for (uint32_t q = lane; q < d; q += 128) {
+                            uint32_t k[4];
+                            bool has[4];
+#pragma unroll
+                            for (int t = 0; t < 4; t++) {
+                                has[t] = q + 32 * t < d;
+                                k[t] = has[t] ? ent[q + 32 * t] : 0u;
+                                has[t] = has[t] && CFLR_CHECK(k[t] < n, &W.cnt->overflow);
+                            }
+#pragma unroll
+                            for (int t = 0; t < 4; t++)
+                                has[t] = has[t] &&
+                                         ((ok[(size_t)k[t] * ow] >> (lx & 31)) & 1u);
+#pragma unroll
+                            for (int t = 0; t < 4; t++) {
+                                if (!has[t]) continue;
+                                const uint4 x = gd[k[t]];
+                                f += x.y - (o ? (x.w & DLAST_MASK) : 0u);
+                                cnt++;
+                            }
+                        }
+                    } else if (act && !is_slow(rec)) {
+#pragma unroll 2
+                        for (uint32_t q = lane; q < d; q += 32) {
+                            const uint32_t k = ent[q];
+                            if (!CFLR_CHECK(k < n, &W.cnt->overflow)) continue;
+                            if ((rec.x & 3) == PART_U) f++;
+                            else entry_work(rec, slot, o, n, db, k, f, cnt);
+                        }
+                    }
+                    // (f per lane stays below 2^52)
+                    f = __reduce_add_sync(FULL_MASK, (uint32_t)f & 0xFFFFFu) +
+                        ((unsigned long long)__reduce_add_sync(FULL_MASK, (uint32_t)(f >> 20))
+                         << 20);
+                    cnt = __reduce_add_sync(FULL_MASK, cnt);
+                    lead = act && lane == 0;
+                    slow = lead && is_slow(rec);
+                    if (lead && f && ((rec.x & 3) != PART_F || (rec.w & USE_SHARED)))
+                        mtiles = db[((long long)rec.y - slot) * 2 * (long long)n + idx].y;
+                } else {
+                    // a lane per (row, use, entry)
+                    const int src = my_row < 0 ? 0 : my_row;
+                    xo = __shfl_sync(FULL_MASK, mt.x, src);
+                    idx = __shfl_sync(FULL_MASK, mt.y, src);
+                    n = __shfl_sync(FULL_MASK, m_n, src);
+                    d = __shfl_sync(FULL_MASK, m_d, src);
+                    dstart = __shfl_sync(FULL_MASK, m_dstart, src);
+                    const uint32_t slot = xo >> 1, o = xo & 1;
+                    bool act = my_row >= 0;
+                    uint32_t e = 0;
+                    if (act) {
+                        const uint32_t rel = lane - my_at, q = rel / d;
+                        e = rel - q * d;
+                        rec = P.use_rec[my_u0 + q];
+                        act = wanted(rec);
+                    }
+                    lead = act && e == 0;
+                    slow = act && is_slow(rec);
+                    if (act && !slow) {
+                        const uint32_t part = rec.x & 3;
+                        const uint4 *db = S.desc[slot] + (size_t)o * n;
+                        if (e == 0 && (part != PART_F || (rec.w & USE_SHARED)))
+                            mtiles = db[((long long)rec.y - slot) * 2 * (long long)n + idx].y;
+                        if (part == PART_U) {
+                            f = 1;
+                        } else {
+                            const uint32_t k = S.pool[slot][dstart + e];
+                            if (CFLR_CHECK(k < n, &W.cnt->overflow))
+                                entry_work(rec, slot, o, n, db, k, f, cnt);
+                        }
+                    }
+                    // sums over the d lanes of a use, in its first lane
+                    const uint32_t seg = my_row < 0 ? 1u : d;
+                    for (uint32_t q = 1; __any_sync(FULL_MASK, q < seg); q <<= 1) {
+                        const unsigned long long fo = __shfl_down_sync(FULL_MASK, f, q);
+                        const uint32_t co = __shfl_down_sync(FULL_MASK, cnt, q);
+                        if (e + q < seg) {
+                            f += fo;
+                            cnt += co;
+                        }
+                    }
+                }
+                slow |= finish(lead && !slow, rec, idx, n, d, mtiles, f, cnt);
+                for (unsigned sm = __ballot_sync(FULL_MASK, slow && lead); sm; sm &= sm - 1) {
+                    const int q = __ffs(sm) - 1;
+                    warp_use(__shfl_sync(FULL_MASK, rec.x, q), __shfl_sync(FULL_MASK, xo, q),
+                             __shfl_sync(FULL_MASK, idx, q), __shfl_sync(FULL_MASK, dstart, q),
+                             __shfl_sync(FULL_MASK, d, q));
+                }
             }
-            continue;
-        }
-        for (uint32_t u = u0; u < u1; u++) {
-            const uint32_t code = P.use_code[u];
-            if (prod_only >= 0 && (code >> 2) != (uint32_t)prod_only) continue;
-            // the warp shares the delta entries; lane 0 stages and counts
-            // the groups
-            acct = lane == 0;
-            use_groups(code, o, n, idx, pool, dstart, d, lane, 32,
-                       [](Work w) { return warp_sum(w); },
-                       [&](int bb, uint2 g) {
-                           if (lane == 0) {
-                               stage[wib][bb][fill[bb]++] = g;
-                               if (fill[bb] == SYM_BUF) flush(bb);
-                           }
-                       });
         }
     }
-    // every lane may hold byte and work counts (lane-per-use mode)
-    for (int b = 0; b < N_BINS; b++) bytes[b] = warp_sum64(bytes[b]);
-    flops = warp_sum64(flops);
-    sym_bytes = warp_sum64(sym_bytes);
-    flops3 = warp_sum64(flops3);
-    mask3 = warp_sum64(mask3);
-    if (lane == 0) {
-        for (int b = 0; b < N_BINS; b++) {
-            if (fill[b]) flush(b);
-            if (bytes[b]) atomicAdd(&W.cnt->bytes_bin[b], bytes[b]);
-        }
-        if (flops) atomicAdd(&W.cnt->flops, flops);
-        if (flops3) atomicAdd(&W.cnt->tiles_bin3[0], flops3);
-        if (mask3) atomicAdd(&W.cnt->tiles_bin3[1], mask3);
-        if (sym_bytes) atomicAdd(&W.cnt->bytes_sym, sym_bytes);
+    if constexpr (MODE == 0) {
+#pragma unroll
+        for (int b = 0; b < N_BINS; b++)
+            if (fill[b]) flush(b, fill[b]);
+    }
+    // (each thread's counts are its own: no barrier)
+    for (int q = 0; q < N_ACC; q++) {
+        const unsigned long long v = warp_sum64(acc_sh[q][threadIdx.x]);
+        if (lane == 0 && v) atomicAdd(total_of(q), v);
     }
 }
 
@@ -3137,8 +3351,9 @@ static void set_smem_attrs() {
 
 void launch_symbolic(const SlotTab &S, const ProdTab &P, const WorkBufs &W, int prod_only,
                      const Tuning &T, int sms, cudaStream_t st) {
-    k_symbolic<<<sms * 8, 256, 0, st>>>(S, P, W, prod_only, T, 0);
-    k_symbolic<<<sms * 4, 256, 0, st>>>(S, P, W, prod_only, T, 1);
+    // resident CTAs (the rows are claimed); few rows are long
+    k_symbolic<0><<<sms * 3, 256, 0, st>>>(S, P, W, prod_only, T);
+    k_symbolic<1><<<sms * 2, 256, 0, st>>>(S, P, W, prod_only, T);
 }
 
 // The product bins, with the witness plumbing compiled in only when the

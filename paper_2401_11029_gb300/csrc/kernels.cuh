@@ -126,8 +126,11 @@ struct LoopCtl {
 
 struct ProdTab {              // global production table of the batch
     const uint4 *prod;        // {c_slot, a_slot, b_slot, kind(0 binary, 1 unit)}
-    const uint32_t *use_off;  // per slot*2+o: offsets into use_code
-    const uint32_t *use_code; // prod << 2 | part, or family << 2 | PART_F
+    const uint32_t *use_off;  // per slot*2+o: offsets into use_rec
+    // one use of a row's delta: {code, output slot c, gathered slot (a
+    // family's: of its first member), members | USE_* flags}; the code is
+    // prod << 2 | part, or family << 2 | PART_F
+    const uint4 *use_rec;
     // families run as one block product (optimisation 4):
     // {offset into fam_prod, members F, flags, part of the shared operand
     // (PART_A: a shared, PART_B: b shared)}; member i is production
@@ -138,10 +141,14 @@ struct ProdTab {              // global production table of the batch
     const uint32_t *fam_prod;
 };
 constexpr uint32_t FAM_CSHARED = 1, FAM_CONSEC = 2;
+constexpr uint32_t USE_MEMBERS = 0xFFFFu;     // use_rec.w: members (1: one production)
+constexpr uint32_t USE_SHARED = 1u << 16;     // a family whose members write one c
+constexpr uint32_t USE_NARROW = 1u << 17;     // a family of at most 64 consecutive slots
 
 struct Counters {
     unsigned long long groups[N_BINS];
-    unsigned long long claim[N_BINS];   // next group of the bin to take (CTA-level bins)
+    unsigned long long claim[N_BINS + 1];   // next group of the bin to take (CTA-level bins);
+                                        // last: next batch of rows of k_symbolic
     unsigned long long cand;
     unsigned long long delta;
     unsigned long long flops;

@@ -434,7 +434,8 @@ struct Runner {
     DevArr<uint4> d_prod;
     DevArr<uint4> d_fam;
     DevArr<uint32_t> d_fam_prod;
-    DevArr<uint32_t> d_use_off, d_use_code;
+    DevArr<uint32_t> d_use_off;
+    DevArr<uint4> d_use_rec;
     // work buffers
     DevArr<uint2> d_touched[2];
     DevArr<unsigned long long> d_touched_n;   // [2]
@@ -628,10 +629,20 @@ struct Runner {
             }
         }
         n_prods = (uint32_t)prods.size();
-        std::vector<uint32_t> off(1, 0), codes;
+        std::vector<uint32_t> off(1, 0);
+        std::vector<uint4> recs;
         for (auto &u : uses) {
-            codes.insert(codes.end(), u.begin(), u.end());
-            off.push_back((uint32_t)codes.size());
+            for (uint32_t code : u) {
+                const uint32_t part = code & 3;
+                const bool fam = part == PART_F;
+                const uint4 fm = fam ? fams[code >> 2] : make_uint4(0, 1, 0, part);
+                const uint4 pr = prods[fam ? fam_prod[fm.x] : code >> 2];
+                uint32_t w = fm.y;
+                if (fm.z & FAM_CSHARED) w |= USE_SHARED;
+                if ((fm.z & FAM_CONSEC) && fm.y <= 64) w |= USE_NARROW;
+                recs.push_back(make_uint4(code, pr.x, fm.w == PART_A ? pr.z : pr.y, w));
+            }
+            off.push_back((uint32_t)recs.size());
         }
         const size_t ni = cx.size();
         d_desc.ensure(own, n_slots);
@@ -652,7 +663,7 @@ struct Runner {
         d_fam.ensure(own, std::max<size_t>(fams.size(), 1));
         d_fam_prod.ensure(own, std::max<size_t>(fam_prod.size(), 1));
         d_use_off.ensure(own, off.size());
-        d_use_code.ensure(own, codes.size());
+        d_use_rec.ensure(own, recs.size());
         d_pool_top.ensure(own, ni);
         d_pool_cap.ensure(own, ni);
         d_inst_delta.ensure(own, ni);
@@ -677,8 +688,9 @@ struct Runner {
             ck(cudaMemcpyAsync(d_fam_prod.p, fam_prod.data(), fam_prod.size() * 4, cudaMemcpyHostToDevice, st), "H2D");
         }
         ck(cudaMemcpyAsync(d_use_off.p, off.data(), off.size() * 4, cudaMemcpyHostToDevice, st), "H2D");
-        if (!codes.empty())
-            ck(cudaMemcpyAsync(d_use_code.p, codes.data(), codes.size() * 4, cudaMemcpyHostToDevice, st), "H2D");
+        if (!recs.empty())
+            ck(cudaMemcpyAsync(d_use_rec.p, recs.data(), recs.size() * sizeof(uint4),
+                               cudaMemcpyHostToDevice, st), "H2D");
         // loop state: parity 0, no touched rows, iteration count 0
         std::vector<uint32_t> act(ni);
         for (size_t k = 0; k < ni; k++) act[k] = cx[k]->touched_n ? 1u : 0u;
@@ -758,7 +770,7 @@ struct Runner {
     }
     ProdTab prodtab() {
         ProdTab P;
-        P.prod = d_prod.p; P.use_off = d_use_off.p; P.use_code = d_use_code.p;
+        P.prod = d_prod.p; P.use_off = d_use_off.p; P.use_rec = d_use_rec.p;
         P.fam = d_fam.p;
         P.fam_prod = d_fam_prod.p;
         return P;
