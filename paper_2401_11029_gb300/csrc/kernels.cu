@@ -3578,7 +3578,6 @@ void launch_extract_write(const ExtractList &L, uint32_t *out_src, uint32_t *out
     const unsigned long long nu = L.u_end > L.u_begin ? L.u_end - L.u_begin : 0;
     if (!nu || !L.n) return;
     set_smem_attrs();
-    cudaMemsetAsync(cursor, 0, 2 * sizeof(unsigned long long), st);
     k_extract_units<<<grid_for(nu, 8, sms, 8), 256, 0, st>>>(L, units, out_src, out_dst, big,
                                                              big_cap, cursor, err);
     const size_t bm_bytes = (size_t)((L.n + 31) / 32) * 4;

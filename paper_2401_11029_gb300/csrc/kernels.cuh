@@ -315,8 +315,8 @@ void launch_extract(const uint4 *desc, const uint32_t *pool, uint32_t n, const u
 // output position o written at out_src / out_dst[o - base]; a row that
 // would end past position `limit` is not written (bit 1 of *err).  Long rows
 // are listed in big (big_cap entries: the range's pairs / 1024 + 1 always
-// suffice; an overflow sets bit 0 of *err); cursor: two words; bitmap as for
-// launch_extract.
+// suffice; an overflow sets bit 0 of *err); cursor: two words, zero; bitmap as
+// for launch_extract.
 struct ExtractList {
     const uint4 *desc;                  // every non-terminal's descriptors, 2 n each
     const uint32_t *pool;

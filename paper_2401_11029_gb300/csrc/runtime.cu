@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <memory>
@@ -72,6 +73,8 @@ inline uint64_t next_pow2(uint64_t x) {
 
 struct Runner;
 
+std::atomic<uint64_t> g_grammar_versions{0};
+
 // One stream-ordered memory pool per device for all contexts of this
 // library.  Freed blocks stay in the pool (release threshold: none), so
 // loading, solving and dropping graphs repeatedly does not map and unmap
@@ -112,6 +115,7 @@ struct cflr_ctx {
     std::string err;
     int state = ST_CREATED;
     Grammar g;
+    uint64_t grammar_version = 0;       // a number of its own for every loaded grammar
     // graph and matrices
     uint32_t n = 0;
     uint64_t ignored = 0;
@@ -126,6 +130,9 @@ struct cflr_ctx {
     std::vector<unsigned long long *> htab;
     std::vector<uint2 *> hval;          // witnesses beside htab (cfg.witness only)
     std::vector<uint64_t> hcap;
+    std::vector<char> hown;             // 1: the set is an allocation of its own, 0: in hblock
+    unsigned long long *hblock = nullptr;   // the sets' first tables
+    size_t hblock_n = 0;
     std::vector<uint64_t> nnz;
     uint2 *touched = nullptr;           // rows with dnew > 0 (local slot ids)
     uint64_t touched_n = 0;
@@ -142,14 +149,13 @@ struct cflr_ctx {
     std::vector<uint64_t> init_cnt;
     Runner *runner = nullptr;           // cached work buffers of solves led by this context
     // extraction scratch
-    // (listed non-terminal ids, unit offsets and their block sums, counters
-    // and group totals, long-row list, row bitmaps)
-    uint32_t *x_nts = nullptr, *x_bm = nullptr, *x_map = nullptr;
-    unsigned long long *x_first = nullptr, *x_unit = nullptr, *x_bsum = nullptr,
-                       *x_misc = nullptr;
+    // (the call's tables, unit offsets and their block sums, long-row list,
+    // row bitmaps, map of non-empty rows)
+    char *x_tab = nullptr;
+    uint32_t *x_bm = nullptr, *x_map = nullptr;
+    unsigned long long *x_unit = nullptr, *x_bsum = nullptr;
     uint4 *x_bigl = nullptr;
-    size_t x_nts_n = 0, x_bm_n = 0, x_map_n = 0, x_first_n = 0, x_unit_n = 0, x_bsum_n = 0,
-           x_misc_n = 0, x_bigl_n = 0;
+    size_t x_tab_n = 0, x_bm_n = 0, x_map_n = 0, x_unit_n = 0, x_bsum_n = 0, x_bigl_n = 0;
     uint32_t *x_src = nullptr, *x_dst = nullptr;
     uint64_t x_out_cap = 0;
     // accounting
@@ -212,13 +218,11 @@ struct cflr_ctx {
     }
     // extraction scratch
     void free_extract_scratch() {
-        drop(x_nts, x_nts_n);
-        drop(x_first, x_first_n);
+        drop(x_tab, x_tab_n);
         drop(x_bm, x_bm_n);
         drop(x_map, x_map_n);
         drop(x_unit, x_unit_n);
         drop(x_bsum, x_bsum_n);
-        drop(x_misc, x_misc_n);
         drop(x_bigl, x_bigl_n);
     }
     // device staging of cflr_get_pairs's host output
@@ -257,12 +261,14 @@ struct cflr_ctx {
         pool = nullptr;
         pool_cap = pool_top = 0;
         for (size_t s = 0; s < htab.size(); s++) {
-            if (htab[s]) dfree(htab[s], hcap[s] * 8);
+            if (htab[s] && hown[s]) dfree(htab[s], hcap[s] * 8);
             if (s < hval.size() && hval[s]) dfree(hval[s], hcap[s] * 8);
         }
         htab.clear();
         hval.clear();
         hcap.clear();
+        hown.clear();
+        drop(hblock, hblock_n);
         nnz.clear();
         if (touched) dfree(touched, touched_cap * sizeof(uint2));
         touched = nullptr;
@@ -348,42 +354,65 @@ struct DevArr {           // device array owned by a context's accounting
     ~DevArr() { release(); }
 };
 
-// Streams beside the solve stream for launches that run side by side, and
-// the events that fork and join them.  A runner takes a set for its life and
-// gives it back; up to SIDE_KEEP sets per process wait for the next runner, so
-// that a context per small graph does not make streams each time.  A set in
-// use belongs to one runner, so contexts of several threads never share one;
-// everything launched on it is joined back to the solve stream, and a runner
-// is destroyed after its stream's work is done with.
-struct SideStreams {
+// What a runner needs of the host side besides device memory: streams beside
+// the solve stream for launches that run side by side, the events that fork
+// and join them and time a solve, and two pinned blocks (the mirror of the
+// runner's tables, the tables of a read-out).  A runner takes a kit for its
+// life and gives it back; up to KIT_KEEP kits per process wait for the next
+// runner, so that a context per small graph does not make them each time.  A
+// kit in use belongs to one runner, so contexts of several threads never share
+// one; everything launched on its streams is joined back to the solve stream,
+// and a runner waits for that stream before it gives the kit back.
+struct PinnedBlock {
+    char *p = nullptr;
+    size_t n = 0;
+    // at least `need` bytes (the contents are not kept)
+    void ensure(size_t need) {
+        if (need <= n) return;
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        n = 0;
+        const size_t want = std::max<size_t>(need + need / 2, 1 << 16);
+        ck(cudaMallocHost(&p, want), "cudaMallocHost");
+        n = want;
+    }
+    ~PinnedBlock() {
+        if (p) cudaFreeHost(p);
+    }
+};
+struct RunnerKit {
     int device = 0;
     cudaStream_t s[N_BINS - 1] = {};
-    cudaEvent_t fork = nullptr, join[N_BINS - 1] = {};
-    ~SideStreams() {
+    cudaEvent_t fork = nullptr, join[N_BINS - 1] = {}, begin = nullptr, end = nullptr;
+    PinnedBlock tables, readout;
+    ~RunnerKit() {
         for (cudaStream_t q : s)
             if (q) cudaStreamDestroy(q);
         for (cudaEvent_t e : join)
             if (e) cudaEventDestroy(e);
-        if (fork) cudaEventDestroy(fork);
+        for (cudaEvent_t e : {fork, begin, end})
+            if (e) cudaEventDestroy(e);
     }
 };
-constexpr size_t SIDE_KEEP = 16;
-std::mutex g_side_mu;
-std::vector<SideStreams *> g_side_free;
+constexpr size_t KIT_KEEP = 16;
+std::mutex g_kit_mu;
+std::vector<RunnerKit *> g_kit_free;
 
-SideStreams *take_side(int device) {
+RunnerKit *take_kit(int device) {
     {
-        std::lock_guard<std::mutex> lock(g_side_mu);
-        for (size_t k = 0; k < g_side_free.size(); k++) {
-            if (g_side_free[k]->device != device) continue;
-            SideStreams *x = g_side_free[k];
-            g_side_free.erase(g_side_free.begin() + k);
+        std::lock_guard<std::mutex> lock(g_kit_mu);
+        for (size_t k = 0; k < g_kit_free.size(); k++) {
+            if (g_kit_free[k]->device != device) continue;
+            RunnerKit *x = g_kit_free[k];
+            g_kit_free.erase(g_kit_free.begin() + k);
             return x;
         }
     }
-    std::unique_ptr<SideStreams> x(new SideStreams());
+    std::unique_ptr<RunnerKit> x(new RunnerKit());
     x->device = device;
     ck(cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming), "cudaEventCreate");
+    ck(cudaEventCreate(&x->begin), "cudaEventCreate");
+    ck(cudaEventCreate(&x->end), "cudaEventCreate");
     for (int q = 0; q < N_BINS - 1; q++) {
         ck(cudaStreamCreateWithFlags(&x->s[q], cudaStreamNonBlocking), "cudaStreamCreate");
         ck(cudaEventCreateWithFlags(&x->join[q], cudaEventDisableTiming), "cudaEventCreate");
@@ -391,17 +420,36 @@ SideStreams *take_side(int device) {
     return x.release();
 }
 
-void give_side(SideStreams *x) {
+void give_kit(RunnerKit *x) {
     if (!x) return;
-    {
-        std::lock_guard<std::mutex> lock(g_side_mu);
-        if (g_side_free.size() < SIDE_KEEP) {
-            g_side_free.push_back(x);
+    // (large blocks are not kept)
+    const bool small = x->tables.n + x->readout.n <= (16u << 20);
+    if (small) {
+        std::lock_guard<std::mutex> lock(g_kit_mu);
+        if (g_kit_free.size() < KIT_KEEP) {
+            g_kit_free.push_back(x);
             return;
         }
     }
     delete x;
 }
+
+template <class T>
+struct View {             // a table inside the runner's device block
+    T *p = nullptr;
+};
+
+// Everything a captured iteration depends on: the launches' arguments.  A
+// graph captured with the same ones does the same work, whatever the tables
+// behind the pointers hold by then.
+struct GraphKey {
+    SlotTab S;
+    ProdTab P;
+    InstTab I;
+    WorkBufs W;
+    Tuning T;
+    uint32_t n_slots, n_inst, max_n, growth;
+};
 
 // The closure-loop driver over one or more contexts (a batch).  Every
 // context's non-terminals get global slot ids; work items name slots, so
@@ -416,43 +464,54 @@ struct Runner {
     uint32_t n_slots = 0, n_prods = 0;
     uint32_t max_n = 0;
     std::vector<uint32_t> slot_ctx;    // slot -> context index
-    // device tables
-    DevArr<uint4 *> d_desc;
-    DevArr<uint2 *> d_dn;
-    DevArr<uint32_t *> d_pool;
-    DevArr<uint32_t> d_n, d_inst, d_occw, d_local;
-    DevArr<uint32_t *> d_occ;
-    DevArr<unsigned long long *> d_htab;
-    DevArr<uint2 *> d_hval;
+    // Device tables: views into one block, laid out by bind() as the grammar's
+    // part (productions, uses), the graphs' part (pointers, sizes), the state
+    // (uploaded by bind, read back by read_status) and counters that stay on
+    // the device.  The host's mirror has the same layout up to the state's end.
+    DevArr<char> d_block;
+    size_t off_graphs = 0, off_htab = 0, off_pool = 0, off_state = 0, off_end = 0;
+    View<uint4 *> d_desc;
+    View<uint2 *> d_dn;
+    View<uint32_t *> d_pool;
+    View<uint32_t> d_n, d_inst, d_occw, d_local;
+    View<uint32_t *> d_occ;
+    View<unsigned long long *> d_htab;
+    View<uint2 *> d_hval;
     DevArr<uint2> d_cand_wit;
     bool wit = false;                  // some context of the batch records witnesses
-    DevArr<unsigned long long> d_hmask, d_cand, d_delta, d_nnz;
-    DevArr<unsigned long long> d_pool_top, d_pool_cap, d_inst_delta;
-    DevArr<uint32_t> d_inst_active, d_inst_iters, d_inst_base;
+    View<unsigned long long> d_hmask, d_cand, d_delta, d_nnz;
+    View<unsigned long long> d_pool_top, d_pool_cap, d_inst_delta;
+    View<uint32_t> d_inst_active, d_inst_iters;
+    DevArr<uint32_t> d_inst_base;
     DevArr<unsigned long long> d_inst_cnt;
     DevArr<uint2 *> d_inst_out;
-    DevArr<uint4> d_prod;
-    DevArr<uint4> d_fam;
-    DevArr<uint32_t> d_fam_prod;
-    DevArr<uint32_t> d_use_off;
-    DevArr<uint4> d_use_rec;
+    View<uint4> d_prod;
+    View<uint4> d_fam;
+    View<uint32_t> d_fam_prod;
+    View<uint32_t> d_use_off;
+    View<uint4> d_use_rec;
+    View<unsigned long long> d_touched_n;     // [2]
+    View<Counters> d_cnt;
+    View<LoopCtl> d_ctl;
+    View<int> d_parity;
+    // the grammar's part in the block: of the owner's grammar alone (its
+    // version, the execution form and the size class bind() looks at), or 0
+    uint64_t grammar_key[3] = {0, 0, 0};
     // work buffers
     DevArr<uint2> d_touched[2];
-    DevArr<unsigned long long> d_touched_n;   // [2]
     DevArr<uint2> d_groups[N_BINS];
     DevArr<unsigned long long> d_cand_key;
     DevArr<uint32_t> d_cand_slot;
     DevArr<uint2> d_cand_pos;
     DevArr<uint32_t> d_bitmap;
     DevArr<uint2> d_big;                      // long delta rows for the symbolic CTA pass
-    DevArr<Counters> d_cnt;
-    DevArr<LoopCtl> d_ctl;
-    DevArr<int> d_parity;
-    Counters *h_cnt = nullptr;                // pinned
-    LoopCtl *h_ctl = nullptr;                 // pinned
-    int *h_parity = nullptr;                  // pinned
-    unsigned long long *h_small = nullptr;    // pinned scratch for small reads
-    size_t h_small_n = 0;
+    // in the mirror: the state as last read
+    Counters *h_cnt = nullptr;
+    LoopCtl *h_ctl = nullptr;
+    int *h_parity = nullptr;
+    unsigned long long *h_touched_n = nullptr, *h_pool_top = nullptr, *h_nnz = nullptr,
+                       *h_cand = nullptr;
+    uint32_t *h_iters = nullptr, *h_active = nullptr;
     uint64_t cand_cap = 0, touched_cap = 0;
     uint64_t group_cap[N_BINS] = {};
     uint64_t regrows = 0;
@@ -461,34 +520,27 @@ struct Runner {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     cudaGraphConditionalHandle handle = 0;
-    bool graph_valid = false;
-    SideStreams *side = nullptr;       // for the product bins
-    bool side_broken = false;          // a capture on them failed
+    GraphKey graph_key{};              // what `gexec` was captured with
+    RunnerKit *kit = nullptr;
+    bool kit_broken = false;           // a capture on its streams failed
 
     explicit Runner(cflr_ctx *owner) : own(owner), st(owner->stream), sms(owner->sms) {
         prof.owner = own;
         prof.on = own->cfg.profile != 0;
         prof.st = st;
-        ck(cudaMallocHost(&h_cnt, sizeof(Counters)), "cudaMallocHost");
-        ck(cudaMallocHost(&h_ctl, sizeof(LoopCtl)), "cudaMallocHost");
-        ck(cudaMallocHost(&h_parity, sizeof(int)), "cudaMallocHost");
-        side = take_side(own->device);
+        kit = take_kit(own->device);
     }
     ~Runner() {
         drop_graph();
-        if (side_broken) delete side;
-        else give_side(side);
-        if (h_cnt) cudaFreeHost(h_cnt);
-        if (h_ctl) cudaFreeHost(h_ctl);
-        if (h_parity) cudaFreeHost(h_parity);
-        if (h_small) cudaFreeHost(h_small);
+        cudaStreamSynchronize(st);     // nothing uses the kit any more
+        if (kit_broken) delete kit;
+        else give_kit(kit);
     }
     void drop_graph() {
         if (gexec) cudaGraphExecDestroy(gexec);
         if (graph) cudaGraphDestroy(graph);
         gexec = nullptr;
         graph = nullptr;
-        graph_valid = false;
     }
 
     // A context's allocation (stream-ordered on the context's stream) made
@@ -499,60 +551,22 @@ struct Runner {
         return p;
     }
 
-    unsigned long long *small(size_t n) {
-        if (n > h_small_n) {
-            if (h_small) cudaFreeHost(h_small);
-            h_small = nullptr;
-            h_small_n = std::max<size_t>(n, 64);
-            ck(cudaMallocHost(&h_small, h_small_n * 8), "cudaMallocHost");
-        }
-        return h_small;
-    }
     void sync(const char *what) { ck(cudaStreamSynchronize(st), what); }
 
     // ---- tables ---------------------------------------------------------
-    // Point the runner at a batch of contexts (their matrices are loaded):
-    // global slot ids, production and use tables, pair counts.
-    void bind(std::vector<cflr_ctx *> ctxs) {
-        cx = std::move(ctxs);
-        regrows = 0;
-        regrow_kind[0] = regrow_kind[1] = regrow_kind[2] = 0;
-        drop_graph();
-        wit = false;
-        for (auto *c : cx) wit |= c->cfg.witness != 0;
-        if (wit && cand_cap && d_cand_wit.n < cand_cap) d_cand_wit.alloc(own, cand_cap);
-        base.clear();
-        slot_ctx.clear();
-        n_slots = 0;
-        max_n = 0;
-        for (size_t k = 0; k < cx.size(); k++) {
-            base.push_back(n_slots);
-            uint32_t nt = (uint32_t)cx[k]->g.nts.size();
-            for (uint32_t x = 0; x < nt; x++) slot_ctx.push_back((uint32_t)k);
-            n_slots += nt;
-            max_n = std::max(max_n, cx[k]->n);
-        }
-        std::vector<uint4 *> hd(n_slots);
-        std::vector<uint2 *> hdn(n_slots);
-        std::vector<uint32_t *> hoc(n_slots);
-        std::vector<uint32_t> hn(n_slots), hi(n_slots), how(n_slots), hl(n_slots);
-        std::vector<unsigned long long> hz(n_slots);
-        std::vector<uint4> prods, fams;
-        std::vector<uint32_t> fam_prod;
+    // The production and use tables of the batch (the grammar's part).
+    struct GrammarTables {
+        std::vector<uint4> prods, fams, recs;
+        std::vector<uint32_t> fam_prod, off;
+    };
+    GrammarTables grammar_tables() const {
+        GrammarTables out;
+        std::vector<uint4> &prods = out.prods, &fams = out.fams;
+        std::vector<uint32_t> &fam_prod = out.fam_prod;
         std::vector<std::vector<uint32_t>> uses((size_t)n_slots * 2);
         for (size_t k = 0; k < cx.size(); k++) {
-            cflr_ctx *c = cx[k];
-            uint32_t nt = (uint32_t)c->g.nts.size(), b0 = base[k];
-            for (uint32_t x = 0; x < nt; x++) {
-                hd[b0 + x] = c->desc + (size_t)x * 2 * c->n;
-                hdn[b0 + x] = c->dn + (size_t)x * 2 * c->n;
-                hoc[b0 + x] = c->occ;
-                how[b0 + x] = c->occ_w;
-                hl[b0 + x] = x;
-                hn[b0 + x] = c->n;
-                hi[b0 + x] = (uint32_t)k;
-                hz[b0 + x] = c->nnz[x];
-            }
+            const cflr_ctx *c = cx[k];
+            const uint32_t b0 = base[k];
             const Grammar &g = c->g;
             std::vector<uint32_t> pid(g.bin_c.size());
             for (size_t p = 0; p < g.bin_c.size(); p++) {
@@ -628,9 +642,7 @@ struct Runner {
                 uses[(size_t)(b0 + g.unit_a[p]) * 2 + 0].push_back(id << 2 | PART_U);
             }
         }
-        n_prods = (uint32_t)prods.size();
-        std::vector<uint32_t> off(1, 0);
-        std::vector<uint4> recs;
+        out.off.assign(1, 0);
         for (auto &u : uses) {
             for (uint32_t code : u) {
                 const uint32_t part = code & 3;
@@ -640,78 +652,181 @@ struct Runner {
                 uint32_t w = fm.y;
                 if (fm.z & FAM_CSHARED) w |= USE_SHARED;
                 if ((fm.z & FAM_CONSEC) && fm.y <= 64) w |= USE_NARROW;
-                recs.push_back(make_uint4(code, pr.x, fm.w == PART_A ? pr.z : pr.y, w));
+                out.recs.push_back(make_uint4(code, pr.x, fm.w == PART_A ? pr.z : pr.y, w));
             }
-            off.push_back((uint32_t)recs.size());
+            out.off.push_back((uint32_t)out.recs.size());
         }
-        const size_t ni = cx.size();
-        d_desc.ensure(own, n_slots);
-        d_dn.ensure(own, n_slots);
-        d_occ.ensure(own, n_slots);
-        d_occw.ensure(own, n_slots);
-        d_local.ensure(own, n_slots);
-        d_pool.ensure(own, n_slots);
-        d_n.ensure(own, n_slots);
-        d_inst.ensure(own, n_slots);
-        d_htab.ensure(own, n_slots);
-        d_hval.ensure(own, n_slots);
-        d_hmask.ensure(own, n_slots);
-        d_cand.ensure(own, n_slots);
-        d_delta.ensure(own, n_slots);
-        d_nnz.ensure(own, n_slots);
-        d_prod.ensure(own, prods.size());
-        d_fam.ensure(own, std::max<size_t>(fams.size(), 1));
-        d_fam_prod.ensure(own, std::max<size_t>(fam_prod.size(), 1));
-        d_use_off.ensure(own, off.size());
-        d_use_rec.ensure(own, recs.size());
-        d_pool_top.ensure(own, ni);
-        d_pool_cap.ensure(own, ni);
-        d_inst_delta.ensure(own, ni);
-        d_inst_active.ensure(own, ni);
-        d_inst_iters.ensure(own, ni);
-        d_touched_n.ensure(own, 2);
-        d_cnt.ensure(own, 1);
-        d_ctl.ensure(own, 1);
-        d_parity.ensure(own, 1);
-        ck(cudaMemcpyAsync(d_desc.p, hd.data(), n_slots * sizeof(uint4 *), cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_dn.p, hdn.data(), n_slots * sizeof(uint2 *), cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_occ.p, hoc.data(), n_slots * sizeof(uint32_t *), cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_occw.p, how.data(), n_slots * 4, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_local.p, hl.data(), n_slots * 4, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_n.p, hn.data(), n_slots * 4, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_inst.p, hi.data(), n_slots * 4, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_nnz.p, hz.data(), n_slots * 8, cudaMemcpyHostToDevice, st), "H2D");
-        if (!prods.empty())
-            ck(cudaMemcpyAsync(d_prod.p, prods.data(), prods.size() * sizeof(uint4), cudaMemcpyHostToDevice, st), "H2D");
-        if (!fams.empty()) {
-            ck(cudaMemcpyAsync(d_fam.p, fams.data(), fams.size() * sizeof(uint4), cudaMemcpyHostToDevice, st), "H2D");
-            ck(cudaMemcpyAsync(d_fam_prod.p, fam_prod.data(), fam_prod.size() * 4, cudaMemcpyHostToDevice, st), "H2D");
-        }
-        ck(cudaMemcpyAsync(d_use_off.p, off.data(), off.size() * 4, cudaMemcpyHostToDevice, st), "H2D");
-        if (!recs.empty())
-            ck(cudaMemcpyAsync(d_use_rec.p, recs.data(), recs.size() * sizeof(uint4),
-                               cudaMemcpyHostToDevice, st), "H2D");
-        // loop state: parity 0, no touched rows, iteration count 0
-        std::vector<uint32_t> act(ni);
-        for (size_t k = 0; k < ni; k++) act[k] = cx[k]->touched_n ? 1u : 0u;
-        ck(cudaMemcpyAsync(d_inst_active.p, act.data(), ni * 4, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemsetAsync(d_inst_iters.p, 0, ni * 4, st), "memset");
-        ck(cudaMemsetAsync(d_touched_n.p, 0, 16, st), "memset");
-        ck(cudaMemsetAsync(d_parity.p, 0, sizeof(int), st), "memset");
-        LoopCtl ctl{};
-        ctl.limit = own->cfg.max_iterations ? own->cfg.max_iterations : 0xFFFFFFFFu;
-        ctl.stop_on_converge = own->cfg.stop_on_first_converged ? 1u : 0u;
-        *h_ctl = ctl;
-        ck(cudaMemcpyAsync(d_ctl.p, h_ctl, sizeof(LoopCtl), cudaMemcpyHostToDevice, st), "H2D");
-        upload_htabs();
-        upload_pools();
-        sync("bind");
+        return out;
     }
 
-    void upload_htabs() {
-        std::vector<unsigned long long *> ht(n_slots);
-        std::vector<uint2 *> hv(n_slots);
-        std::vector<unsigned long long> hm(n_slots);
+    // Point the runner at a batch of contexts (their matrices are loaded):
+    // global slot ids, the tables and the loop's first state, in one copy to
+    // the device.  (A copy and partly a wait per table, about thirty of them,
+    // took most of the 0.2 ms that a reset or a solve of a small graph spent
+    // on the host.)  A runner bound to its owner alone keeps the grammar's
+    // part while the owner keeps its grammar.
+    void bind(std::vector<cflr_ctx *> ctxs) {
+        cx = std::move(ctxs);
+        regrows = 0;
+        regrow_kind[0] = regrow_kind[1] = regrow_kind[2] = 0;
+        wit = false;
+        for (auto *c : cx) wit |= c->cfg.witness != 0;
+        if (wit && cand_cap && d_cand_wit.n < cand_cap) d_cand_wit.alloc(own, cand_cap);
+        base.clear();
+        slot_ctx.clear();
+        n_slots = 0;
+        max_n = 0;
+        for (size_t k = 0; k < cx.size(); k++) {
+            base.push_back(n_slots);
+            uint32_t nt = (uint32_t)cx[k]->g.nts.size();
+            for (uint32_t x = 0; x < nt; x++) slot_ctx.push_back((uint32_t)k);
+            n_slots += nt;
+            max_n = std::max(max_n, cx[k]->n);
+        }
+        const size_t ni = cx.size(), ns = n_slots;
+        // (families of several output non-terminals need words below 2^21)
+        const uint64_t key[3] = {ni == 1 && cx[0] == own ? own->grammar_version : 0,
+                                 (uint64_t)own->cfg.form + 1, max_n > (1u << 26) ? 2ull : 1ull};
+        const bool keep = key[0] && std::equal(key, key + 3, grammar_key);
+        GrammarTables g;
+        if (!keep) g = grammar_tables();
+        size_t at = keep ? off_graphs : 0;
+        auto take = [&](size_t bytes) {
+            const size_t o = at;
+            at = (at + bytes + 15) & ~(size_t)15;
+            return o;
+        };
+        size_t o_prod = 0, o_fam = 0, o_fp = 0, o_off = 0, o_rec = 0;
+        if (!keep) {
+            o_prod = take(g.prods.size() * sizeof(uint4));
+            o_fam = take(g.fams.size() * sizeof(uint4));
+            o_fp = take(g.fam_prod.size() * 4);
+            o_off = take(g.off.size() * 4);
+            o_rec = take(g.recs.size() * sizeof(uint4));
+            off_graphs = at;
+        }
+        const size_t o_desc = take(ns * 8), o_dn = take(ns * 8), o_occ = take(ns * 8);
+        const size_t o_n = take(ns * 4), o_inst = take(ns * 4), o_occw = take(ns * 4),
+                     o_local = take(ns * 4);
+        off_htab = at;
+        const size_t o_htab = take(ns * 8), o_hval = take(ns * 8), o_hmask = take(ns * 8);
+        off_pool = at;
+        const size_t o_pool = take(ns * 8), o_pcap = take(ni * 8);
+        off_state = at;
+        const size_t o_ctl = take(sizeof(LoopCtl)), o_cnt = take(sizeof(Counters)),
+                     o_tn = take(16), o_par = take(sizeof(int)), o_ptop = take(ni * 8),
+                     o_nnz = take(ns * 8), o_cand = take(ns * 8), o_iters = take(ni * 4),
+                     o_act = take(ni * 4);
+        off_end = at;
+        const size_t o_delta = take(ns * 8), o_idelta = take(ni * 8);
+        sync("bind");                     // the mirror's last copy is done with
+        if (keep && (at > d_block.n || off_end > kit->tables.n)) {
+            // the block moves: the grammar's part goes with it
+            std::fill(grammar_key, grammar_key + 3, 0);
+            return bind(std::vector<cflr_ctx *>(cx));
+        }
+        d_block.ensure(own, at);
+        kit->tables.ensure(off_end);
+        char *d = d_block.p, *h = kit->tables.p;
+        auto put = [&](size_t o, const void *from, size_t bytes) {
+            if (bytes) std::memcpy(h + o, from, bytes);
+        };
+        if (!keep) {
+            put(o_prod, g.prods.data(), g.prods.size() * sizeof(uint4));
+            put(o_fam, g.fams.data(), g.fams.size() * sizeof(uint4));
+            put(o_fp, g.fam_prod.data(), g.fam_prod.size() * 4);
+            put(o_off, g.off.data(), g.off.size() * 4);
+            put(o_rec, g.recs.data(), g.recs.size() * sizeof(uint4));
+            n_prods = (uint32_t)g.prods.size();
+            d_prod.p = (uint4 *)(d + o_prod);
+            d_fam.p = (uint4 *)(d + o_fam);
+            d_fam_prod.p = (uint32_t *)(d + o_fp);
+            d_use_off.p = (uint32_t *)(d + o_off);
+            d_use_rec.p = (uint4 *)(d + o_rec);
+            std::copy(key, key + 3, grammar_key);
+        }
+        d_desc.p = (uint4 **)(d + o_desc);
+        d_dn.p = (uint2 **)(d + o_dn);
+        d_occ.p = (uint32_t **)(d + o_occ);
+        d_n.p = (uint32_t *)(d + o_n);
+        d_inst.p = (uint32_t *)(d + o_inst);
+        d_occw.p = (uint32_t *)(d + o_occw);
+        d_local.p = (uint32_t *)(d + o_local);
+        d_htab.p = (unsigned long long **)(d + o_htab);
+        d_hval.p = (uint2 **)(d + o_hval);
+        d_hmask.p = (unsigned long long *)(d + o_hmask);
+        d_pool.p = (uint32_t **)(d + o_pool);
+        d_pool_cap.p = (unsigned long long *)(d + o_pcap);
+        d_ctl.p = (LoopCtl *)(d + o_ctl);
+        d_cnt.p = (Counters *)(d + o_cnt);
+        d_touched_n.p = (unsigned long long *)(d + o_tn);
+        d_parity.p = (int *)(d + o_par);
+        d_pool_top.p = (unsigned long long *)(d + o_ptop);
+        d_nnz.p = (unsigned long long *)(d + o_nnz);
+        d_cand.p = (unsigned long long *)(d + o_cand);
+        d_inst_iters.p = (uint32_t *)(d + o_iters);
+        d_inst_active.p = (uint32_t *)(d + o_act);
+        d_delta.p = (unsigned long long *)(d + o_delta);
+        d_inst_delta.p = (unsigned long long *)(d + o_idelta);
+        h_ctl = (LoopCtl *)(h + o_ctl);
+        h_cnt = (Counters *)(h + o_cnt);
+        h_touched_n = (unsigned long long *)(h + o_tn);
+        h_parity = (int *)(h + o_par);
+        h_pool_top = (unsigned long long *)(h + o_ptop);
+        h_nnz = (unsigned long long *)(h + o_nnz);
+        h_cand = (unsigned long long *)(h + o_cand);
+        h_iters = (uint32_t *)(h + o_iters);
+        h_active = (uint32_t *)(h + o_act);
+        // the graphs' part
+        uint4 **hd = (uint4 **)(h + o_desc);
+        uint2 **hdn = (uint2 **)(h + o_dn);
+        uint32_t **hoc = (uint32_t **)(h + o_occ);
+        uint32_t *hn = (uint32_t *)(h + o_n), *hi = (uint32_t *)(h + o_inst);
+        uint32_t *how = (uint32_t *)(h + o_occw), *hl = (uint32_t *)(h + o_local);
+        uint64_t touched = 0;
+        for (size_t k = 0; k < ni; k++) {
+            cflr_ctx *c = cx[k];
+            const uint32_t nt = (uint32_t)c->g.nts.size(), b0 = base[k];
+            for (uint32_t x = 0; x < nt; x++) {
+                hd[b0 + x] = c->desc + (size_t)x * 2 * c->n;
+                hdn[b0 + x] = c->dn + (size_t)x * 2 * c->n;
+                hoc[b0 + x] = c->occ;
+                how[b0 + x] = c->occ_w;
+                hl[b0 + x] = x;
+                hn[b0 + x] = c->n;
+                hi[b0 + x] = (uint32_t)k;
+                h_nnz[b0 + x] = c->nnz[x];
+                h_cand[b0 + x] = 0;
+            }
+            h_pool_top[k] = c->pool_top;
+            h_iters[k] = 0;
+            h_active[k] = c->touched_n ? 1u : 0u;
+            touched += c->touched_n;
+        }
+        fill_htabs();
+        fill_pools();
+        // loop state: parity 0, the pending delta rows (import_touched brings
+        // them), iteration count 0
+        *h_ctl = LoopCtl{};
+        h_ctl->limit = own->cfg.max_iterations ? own->cfg.max_iterations : 0xFFFFFFFFu;
+        h_ctl->stop_on_converge = own->cfg.stop_on_first_converged ? 1u : 0u;
+        *h_cnt = Counters{};
+        h_touched_n[0] = touched;
+        h_touched_n[1] = 0;
+        *h_parity = 0;
+        upload(keep ? off_graphs : 0, off_end);
+    }
+
+    // Bytes [from, to) of the mirror to the device block.
+    void upload(size_t from, size_t to) {
+        ck(cudaMemcpyAsync(d_block.p + from, kit->tables.p + from, to - from,
+                           cudaMemcpyHostToDevice, st), "H2D tables");
+    }
+    void fill_htabs() {
+        char *h = kit->tables.p;
+        auto **ht = (unsigned long long **)(h + ((char *)d_htab.p - d_block.p));
+        auto **hv = (uint2 **)(h + ((char *)d_hval.p - d_block.p));
+        auto *hm = (unsigned long long *)(h + ((char *)d_hmask.p - d_block.p));
         for (uint32_t s = 0; s < n_slots; s++) {
             cflr_ctx *c = cx[slot_ctx[s]];
             uint32_t x = s - base[slot_ctx[s]];
@@ -719,44 +834,34 @@ struct Runner {
             hv[s] = x < c->hval.size() ? c->hval[x] : nullptr;
             hm[s] = c->hcap[x] - 1;
         }
-        ck(cudaMemcpyAsync(d_htab.p, ht.data(), n_slots * 8, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_hval.p, hv.data(), n_slots * sizeof(uint2 *), cudaMemcpyHostToDevice,
-                           st), "H2D");
-        ck(cudaMemcpyAsync(d_hmask.p, hm.data(), n_slots * 8, cudaMemcpyHostToDevice, st), "H2D");
-        sync("upload htabs");
     }
-
-    // Pool pointers, capacities and (at bind only) the bump counters.
-    void upload_pools(bool tops = true) {
-        std::vector<unsigned long long> top(cx.size()), cap(cx.size());
-        std::vector<uint32_t *> hp(n_slots);
-        for (size_t k = 0; k < cx.size(); k++) {
-            top[k] = cx[k]->pool_top;
-            cap[k] = cx[k]->pool_cap;
-        }
+    void fill_pools() {
+        char *h = kit->tables.p;
+        auto **hp = (uint32_t **)(h + ((char *)d_pool.p - d_block.p));
+        auto *cap = (unsigned long long *)(h + ((char *)d_pool_cap.p - d_block.p));
+        for (size_t k = 0; k < cx.size(); k++) cap[k] = cx[k]->pool_cap;
         for (uint32_t s = 0; s < n_slots; s++) hp[s] = cx[slot_ctx[s]]->pool;
-        if (tops)
-            ck(cudaMemcpyAsync(d_pool_top.p, top.data(), cx.size() * 8, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_pool_cap.p, cap.data(), cx.size() * 8, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemcpyAsync(d_pool.p, hp.data(), n_slots * sizeof(uint32_t *), cudaMemcpyHostToDevice, st), "H2D");
-        sync("upload pools");
+    }
+    // After growths, whose sets or pools moved (the stream has been waited for
+    // since the mirror was last copied: the growth was decided on a read state).
+    void upload_htabs() {
+        fill_htabs();
+        upload(off_htab, off_pool);
+    }
+    void upload_pools() {
+        fill_pools();
+        upload(off_pool, off_state);
     }
 
-    // After a solve: pool counters, pair counts and iteration counts back to
-    // the contexts.
+    // After a solve, from the state as last read: pool counters, pair counts
+    // and iteration counts back to the contexts.
     void download_state(bool add_iterations) {
-        const size_t ni = cx.size();
-        std::vector<unsigned long long> top(ni), nz(n_slots);
-        std::vector<uint32_t> it(ni);
-        ck(cudaMemcpyAsync(top.data(), d_pool_top.p, ni * 8, cudaMemcpyDeviceToHost, st), "D2H");
-        ck(cudaMemcpyAsync(nz.data(), d_nnz.p, n_slots * 8, cudaMemcpyDeviceToHost, st), "D2H");
-        ck(cudaMemcpyAsync(it.data(), d_inst_iters.p, ni * 4, cudaMemcpyDeviceToHost, st), "D2H");
-        sync("download state");
-        for (size_t k = 0; k < ni; k++) {
-            cx[k]->pool_top = top[k];
-            if (add_iterations) cx[k]->iterations += it[k];
+        for (size_t k = 0; k < cx.size(); k++) {
+            cx[k]->pool_top = h_pool_top[k];
+            if (add_iterations) cx[k]->iterations += h_iters[k];
         }
-        for (uint32_t s = 0; s < n_slots; s++) cx[slot_ctx[s]]->nnz[s - base[slot_ctx[s]]] = nz[s];
+        for (uint32_t s = 0; s < n_slots; s++)
+            cx[slot_ctx[s]]->nnz[s - base[slot_ctx[s]]] = h_nnz[s];
     }
 
     SlotTab slots() {
@@ -817,7 +922,6 @@ struct Runner {
         d_cand_slot.alloc(own, cap);
         if (wit) d_cand_wit.alloc(own, cap);
         d_cand_pos.alloc(own, cap);
-        graph_valid = false;
     }
     // Both touched lists; the list touched[parity] keeps its rows.  Each must
     // hold two rows per new pair (row and column form).
@@ -841,14 +945,12 @@ struct Runner {
         // a listed row has more than 64 delta entries, and the deltas of
         // one iteration hold at most touched_cap entries
         d_big.ensure(own, cap / 64 + 1024);
-        graph_valid = false;
     }
     void size_groups(int b, uint64_t cap) {
         cap = std::max<uint64_t>(cap, min_cap(1 << 14));
         if (cap <= group_cap[b]) return;
         group_cap[b] = cap;
         d_groups[b].alloc(own, cap);
-        graph_valid = false;
     }
     void init_buffers(uint64_t cand_hint, uint64_t touched_in) {
         const uint64_t ic = own->cfg.initial_capacity;
@@ -864,8 +966,7 @@ struct Runner {
         if (max_n > 200 * 1024 * 8) {   // bitmaps do not fit shared memory
             uint64_t words = (max_n + 31) / 32;
             d_bitmap.ensure(own, words * (uint64_t)sms * 8);
-            graph_valid = false;
-        }
+            }
     }
 
     void grow_htab(uint32_t s, uint64_t need) {
@@ -891,7 +992,8 @@ struct Runner {
         // points-to solve grows hundreds of sets, and one wait each had cost
         // about 30 % of its first solve)
         if (c->stream != st) sync("rehash");
-        c->dfree(c->htab[x], c->hcap[x] * 8);
+        if (c->hown[x]) c->dfree(c->htab[x], c->hcap[x] * 8);
+        c->hown[x] = 1;
         if (c->hval[x]) c->dfree(c->hval[x], c->hcap[x] * 8);
         c->htab[x] = nt;
         c->hval[x] = nv;
@@ -949,17 +1051,17 @@ struct Runner {
             // leave.  The heaviest kind of group (bin 3) starts first.  (200k
             // alias solve 53.5 -> 48.9 ms, 500k points-to 108 -> 98.5, Dyck-1
             // of 1000 vertices 2.1 -> 1.7, with two launches less a turn.)
-            ck(cudaEventRecord(side->fork, st), "fork");
+            ck(cudaEventRecord(kit->fork, st), "fork");
             for (int b = N_BINS - 1; b >= 0; b--) {
                 const int q = b - 1;          // bin 0 stays on the solve stream
-                cudaStream_t on = b ? side->s[q] : st;
-                if (b) ck(cudaStreamWaitEvent(on, side->fork, 0), "fork");
+                cudaStream_t on = b ? kit->s[q] : st;
+                if (b) ck(cudaStreamWaitEvent(on, kit->fork, 0), "fork");
                 launch_spgemm(b, S, P, W, max_n, tuning(), sms, on);
                 ck(cudaGetLastError(), kKernelNames[KID_BIN0 + b]);
-                if (b) ck(cudaEventRecord(side->join[q], on), "join");
+                if (b) ck(cudaEventRecord(kit->join[q], on), "join");
             }
             for (int q = 0; q < N_BINS - 1; q++)
-                ck(cudaStreamWaitEvent(st, side->join[q], 0), "join");
+                ck(cudaStreamWaitEvent(st, kit->join[q], 0), "join");
         }
     }
     // Commit and union, from the dedupe (stage 0), the capacity pass
@@ -999,8 +1101,29 @@ struct Runner {
         ck(cudaGetLastError(), "k_iter_begin");
     }
 
+    GraphKey current_key() {
+        GraphKey k;
+        std::memset(&k, 0, sizeof k);
+        k.S = slots();
+        k.P = prodtab();
+        k.I = insttab();
+        k.W = work();
+        k.T = tuning();
+        k.n_slots = n_slots;
+        k.n_inst = (uint32_t)cx.size();
+        k.max_n = max_n;
+        k.growth = 1;
+        for (auto *c : cx) k.growth &= c->cfg.test_fixed_pair_sets == 0 ? 1u : 0u;
+        return k;
+    }
+    // A graph captured with the same arguments serves again: a context that
+    // solves the same or another graph with the buffers it has keeps it.
+    bool graph_fits() {
+        const GraphKey k = current_key();
+        return gexec && !std::memcmp(&k, &graph_key, sizeof k);
+    }
     void ensure_graph() {
-        if (graph_valid) return;
+        if (graph_fits()) return;
         drop_graph();
         prepare_launch_attributes();
         ck(cudaGraphCreate(&graph, 0), "cudaGraphCreate");
@@ -1023,18 +1146,18 @@ struct Runner {
         } catch (...) {
             // end the capture; side streams caught in it go to nobody else
             cudaStreamEndCapture(st, &captured);
-            side_broken = true;
+            kit_broken = true;
             throw;
         }
         ck(cudaStreamEndCapture(st, &captured), "cudaStreamEndCapture");
         ck(cudaGraphInstantiate(&gexec, graph, 0), "cudaGraphInstantiate");
-        graph_valid = true;
+        graph_key = current_key();
     }
 
+    // The state into the mirror (one copy, one wait).
     void read_status() {
-        ck(cudaMemcpyAsync(h_cnt, d_cnt.p, sizeof(Counters), cudaMemcpyDeviceToHost, st), "D2H");
-        ck(cudaMemcpyAsync(h_ctl, d_ctl.p, sizeof(LoopCtl), cudaMemcpyDeviceToHost, st), "D2H");
-        ck(cudaMemcpyAsync(h_parity, d_parity.p, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H");
+        ck(cudaMemcpyAsync(kit->tables.p + off_state, d_block.p + off_state, off_end - off_state,
+                           cudaMemcpyDeviceToHost, st), "D2H");
         sync("status");
     }
     void clear_overflow() {            // and the list of rows to move beside it
@@ -1078,14 +1201,11 @@ struct Runner {
         const InstTab I = insttab();
         const WorkBufs W = work();
         if (st_bits & OVF_HASH) {                      // grow pair sets, then commit
-            std::vector<unsigned long long> nz(n_slots), cd(n_slots);
-            ck(cudaMemcpyAsync(nz.data(), d_nnz.p, n_slots * 8, cudaMemcpyDeviceToHost, st), "D2H");
-            ck(cudaMemcpyAsync(cd.data(), d_cand.p, n_slots * 8, cudaMemcpyDeviceToHost, st), "D2H");
-            sync("hash sizes");
             for (uint32_t s = 0; s < n_slots; s++) {
                 cflr_ctx *c = cx[slot_ctx[s]];
                 uint32_t x = s - base[slot_ctx[s]];
-                if (2 * (nz[s] + cd[s]) > c->hcap[x]) grow_htab(s, nz[s] + cd[s]);
+                const uint64_t need = h_nnz[s] + h_cand[s];
+                if (2 * need > c->hcap[x]) grow_htab(s, need);
             }
             upload_htabs();
             clear_overflow();
@@ -1094,12 +1214,9 @@ struct Runner {
         }
         for (int guard = 0; h_ctl->status & OVF_POOL; guard++) {   // grow pools, redo the union
             if (guard > 8) throw Status{CFLR_ENOMEM, "pool growth did not converge"};
-            std::vector<unsigned long long> top(cx.size());
-            ck(cudaMemcpyAsync(top.data(), d_pool_top.p, cx.size() * 8, cudaMemcpyDeviceToHost, st), "D2H");
-            sync("pool tops");
             for (size_t k = 0; k < cx.size(); k++)
-                if (top[k] > cx[k]->pool_cap) grow_pool(k, top[k]);
-            upload_pools(false);
+                if (h_pool_top[k] > cx[k]->pool_cap) grow_pool(k, h_pool_top[k]);
+            upload_pools();
             clear_overflow();
             launch_merge(S, I, W, 1, true, false, true, false);
             read_status();
@@ -1121,7 +1238,7 @@ struct Runner {
         // so after one the loop runs host-launched iterations until one of
         // them needs no growth, and only then captures the graph again (a
         // fresh context grows several buffers in its first iterations).
-        bool settled = graph_valid;
+        bool settled = use_graph && graph_fits();
         zero_counters();
         for (;;) {
             if (use_graph && settled) {
@@ -1147,16 +1264,14 @@ struct Runner {
     }
 
     // True when some instance of the batch reached its fixpoint.
-    bool first_converged() {
-        std::vector<uint32_t> act(cx.size());
-        ck(cudaMemcpyAsync(act.data(), d_inst_active.p, cx.size() * 4, cudaMemcpyDeviceToHost, st), "D2H");
-        sync("active");
-        for (uint32_t a : act)
-            if (!a) return true;
+    bool first_converged() const {
+        for (size_t k = 0; k < cx.size(); k++)
+            if (!h_active[k]) return true;
         return false;
     }
 
-    // Pending delta rows of each context into the "in" touched list.
+    // Pending delta rows of each context into the "in" touched list (bind set
+    // their number).
     void import_touched() {
         uint64_t total = 0;
         for (auto *c : cx) total += c->touched_n;
@@ -1169,23 +1284,13 @@ struct Runner {
             ck(cudaGetLastError(), "remap");
             at += c->touched_n;
         }
-        unsigned long long *h = small(2);
-        h[0] = at;
-        h[1] = 0;
-        ck(cudaMemcpyAsync(d_touched_n.p, h, 16, cudaMemcpyHostToDevice, st), "H2D");
-        ck(cudaMemsetAsync(d_parity.p, 0, sizeof(int), st), "memset");
-        sync("import");
     }
 
     // Save the pending delta rows of each context (local slot ids), split
-    // on the device.
+    // on the device; their number is in the state as last read.
     void export_touched() {
-        unsigned long long *h = small(2);
-        ck(cudaMemcpyAsync(h, d_touched_n.p, 16, cudaMemcpyDeviceToHost, st), "D2H");
-        ck(cudaMemcpyAsync(h_parity, d_parity.p, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H");
-        sync("export");
         const int par = *h_parity;
-        const uint64_t n_in = h[par];
+        const uint64_t n_in = h_touched_n[par];
         const size_t ni = cx.size();
         if (n_in == 0) {
             for (auto *c : cx) c->touched_n = 0;
@@ -1204,7 +1309,7 @@ struct Runner {
             c->touched_n = n_in;
             ck(cudaMemcpyAsync(c->touched, d_touched[par].p, n_in * sizeof(uint2),
                                cudaMemcpyDeviceToDevice, st), "D2D touched");
-            sync("export copy");
+            if (c->stream != st) sync("export copy");   // (else ordered with what follows)
             return;
         }
         d_inst_cnt.ensure(own, ni);
@@ -1239,9 +1344,9 @@ struct Runner {
         sync("export split");
     }
 
-    // Byte and work totals of the finished solve, from the loop control.
+    // Byte and work totals of the finished solve, from the loop control as
+    // last read.
     void account() {
-        read_status();
         own->k_bytes[KID_SYMBOLIC] += h_ctl->bytes_sym;
         for (int b = 0; b < N_BINS; b++) own->k_bytes[KID_BIN0 + b] += h_ctl->bytes_bin[b];
         own->k_bytes[KID_COMMIT] += 24 * h_ctl->total_cand + 12 * h_ctl->total_delta +
@@ -1584,11 +1689,33 @@ void upload_graph(cflr_ctx *c, uint32_t n, uint64_t m, const uint32_t *src, cons
     c->hval.assign(nt, nullptr);
     c->hcap.assign(nt, 0);
     c->nnz.assign(nt, 0);
+    // First capacities.  Without a budget or a test's sizes the named
+    // non-terminals share 64 MB (at most 512 KB each): clearing that costs
+    // 10 us, and a set that starts at 1024 entries grows two or three times,
+    // each a wait of the solve (618 growths of the 61k-vertex points-to
+    // solve).  One allocation then holds all first tables; one that grows
+    // leaves its place in it unused (an eighth of its new size at most).
+    const bool roomy =
+        !c->cfg.mem_budget_bytes && !c->cfg.initial_capacity && !c->cfg.test_fixed_pair_sets;
+    uint64_t least = 1024;
+    if (roomy && g.n_named)
+        while (least < (1u << 16) && 2 * least * 8 * g.n_named <= (64ull << 20)) least *= 2;
+    uint64_t all = 0;
     for (uint32_t A = 0; A < nt; A++) {
         uint64_t want = std::max<uint64_t>(4 * c->init_cnt[A], 1024);
-        if (A < g.n_named) want = std::max<uint64_t>(want, 3 * share);
+        if (A < g.n_named) want = std::max<uint64_t>({want, least, 3 * share});
         c->hcap[A] = next_pow2(want);
-        c->htab[A] = (unsigned long long *)c->dalloc(c->hcap[A] * 8);
+        all += c->hcap[A];
+    }
+    c->hown.assign(nt, roomy ? 0 : 1);
+    if (roomy) {
+        c->hblock = (unsigned long long *)c->dalloc(all * 8);
+        c->hblock_n = all;
+    }
+    uint64_t at = 0;
+    for (uint32_t A = 0; A < nt; A++) {
+        c->htab[A] = roomy ? c->hblock + at : (unsigned long long *)c->dalloc(c->hcap[A] * 8);
+        at += c->hcap[A];
         if (c->cfg.witness) c->hval[A] = (uint2 *)c->dalloc(c->hcap[A] * 8);
     }
 }
@@ -1658,19 +1785,16 @@ int cuda_status(cflr_ctx *c, const CudaError &e) {
 int solve_many(std::vector<cflr_ctx *> cx, cflr_stats *stats) {
     Range range("cflr_solve");
     cflr_ctx *own = cx[0];
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     ck(cudaSetDevice(own->device), "cudaSetDevice");
     std::vector<cflr_ctx *> active;
     for (auto *c : cx)
         if (c->touched_n) active.push_back(c);
-    ck(cudaEventCreate(&ev0), "event");
-    ck(cudaEventCreate(&ev1), "event");
-    ck(cudaEventRecord(ev0, own->stream), "event");
+    Runner &r = runner_of(own);
+    ck(cudaEventRecord(r.kit->begin, own->stream), "event");
     int rc = CFLR_OK;
     uint64_t flops = 0, cand = 0, regrows = 0, groups[4] = {0, 0, 0, 0}, kinds[3] = {0, 0, 0};
     uint64_t tiles3[2] = {0, 0};
     if (!active.empty()) {
-        Runner &r = runner_of(own);
         r.bind(active);
         uint64_t hint = 0;
         for (auto *c : active) hint += c->touched_n;
@@ -1693,12 +1817,10 @@ int solve_many(std::vector<cflr_ctx *> cx, cflr_stats *stats) {
         regrows = r.regrows;
         for (int q = 0; q < 3; q++) kinds[q] = r.regrow_kind[q];
     }
-    ck(cudaEventRecord(ev1, own->stream), "event");
-    ck(cudaEventSynchronize(ev1), "event");
+    ck(cudaEventRecord(r.kit->end, own->stream), "event");
+    ck(cudaEventSynchronize(r.kit->end), "event");
     float ms = 0;
-    cudaEventElapsedTime(&ms, ev0, ev1);
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
+    cudaEventElapsedTime(&ms, r.kit->begin, r.kit->end);
     for (size_t k = 0; k < cx.size(); k++) {
         cflr_ctx *c = cx[k];
         cflr_stats s{};
@@ -1791,6 +1913,7 @@ int cflr_load_grammar(cflr_ctx *c, const char *text, size_t len) {
         if (g.nts.size() >= (1u << 20)) return c->fail(CFLR_EGRAMMAR, "too many non-terminals");
         c->free_graph();
         c->g = std::move(g);
+        c->grammar_version = ++g_grammar_versions;
         c->grammar_text.assign(text, len);
         c->state = ST_GRAMMAR;
         c->err.clear();
@@ -1977,30 +2100,35 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
     const uint32_t E = (uint32_t)tab.size();
     uint64_t total = 0;
     for (uint64_t p : pairs) total += p;
-    tab.resize(2 * (size_t)E);
-    std::vector<unsigned long long> first(E + 1);
-    extract_plan(E, n, pairs.data(), c->sms, tab.data() + E, first.data());
+    // the call's tables, in one copy to the device: cursors, error flag and
+    // total (four words, zero), first units, listed ids, rows per unit
+    PinnedBlock &pin = runner_of(c).kit->readout;
+    const size_t tab_n = 32 + 8 * ((size_t)E + 1) + 8 * (size_t)E;
+    pin.ensure(tab_n);
+    c->scratch(c->x_tab, c->x_tab_n, tab_n);
+    unsigned long long *misc = (unsigned long long *)pin.p;
+    unsigned long long *first = misc + 4;
+    uint32_t *ids = (uint32_t *)(first + E + 1);
+    std::fill(misc, misc + 4, 0ull);
+    std::copy(tab.begin(), tab.end(), ids);
+    extract_plan(E, n, pairs.data(), c->sms, ids + E, first);
     const uint64_t U = first[E];
-    c->scratch(c->x_nts, c->x_nts_n, 2 * (size_t)E);
-    c->scratch(c->x_first, c->x_first_n, (size_t)E + 1);
+    unsigned long long *d_misc = (unsigned long long *)c->x_tab;
+    uint32_t *d_ids = (uint32_t *)(d_misc + 4 + E + 1);
     c->scratch(c->x_unit, c->x_unit_n, U + 1);
     c->scratch(c->x_bsum, c->x_bsum_n, U / 1024 + 2);
-    c->scratch(c->x_misc, c->x_misc_n, 4);       // cursors, error flag, total
     const size_t words = ((size_t)n + 31) / 32;
     if (words * 4 > 200 * 1024) c->scratch(c->x_bm, c->x_bm_n, words * (size_t)c->sms * 4);
-    ck(cudaMemcpyAsync(c->x_nts, tab.data(), tab.size() * 4, cudaMemcpyHostToDevice, st), "H2D");
-    ck(cudaMemcpyAsync(c->x_first, first.data(), first.size() * 8, cudaMemcpyHostToDevice, st),
-       "H2D");
-    ck(cudaMemsetAsync(c->x_misc + 2, 0, 8, st), "memset");
-    unsigned *err = (unsigned *)(c->x_misc + 2);
+    ck(cudaMemcpyAsync(c->x_tab, pin.p, tab_n, cudaMemcpyHostToDevice, st), "H2D");
+    unsigned *err = (unsigned *)(d_misc + 2);
     ExtractList L{};
     L.desc = c->desc;
     L.pool = c->pool;
     L.perm = c->perm;
     L.iperm = c->iperm;
-    L.nts = c->x_nts;
-    L.rows_per = c->x_nts + E;
-    L.unit_first = c->x_first;
+    L.nts = d_ids;
+    L.rows_per = d_ids + E;
+    L.unit_first = d_misc + 4;
     L.n = n;
     L.count = E;
     L.units = U;
@@ -2022,11 +2150,10 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
         ck(cudaGetLastError(), "row map");
         L.map = c->x_map;
     }
-    launch_extract_count(L, c->x_unit, c->x_bsum, c->x_misc + 3, c->sms, st);
+    launch_extract_count(L, c->x_unit, c->x_bsum, d_misc + 3, c->sms, st);
     ck(cudaGetLastError(), "extract count");
-    unsigned long long misc[4] = {0, 0, 0, 0};
     auto check = [&]() {
-        ck(cudaMemcpyAsync(misc, c->x_misc, sizeof(misc), cudaMemcpyDeviceToHost, st), "D2H");
+        ck(cudaMemcpyAsync(misc, d_misc, 32, cudaMemcpyDeviceToHost, st), "D2H");
         ck(cudaStreamSynchronize(st), "sync extract");
         if (misc[2] & 1)
             throw Status{CFLR_ECUDA, "internal: the long-row list of the extraction overflowed"};
@@ -2043,7 +2170,7 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
         L.u_end = U;
         L.base = 0;
         L.limit = total;
-        launch_extract_write(L, ws, wd, c->x_unit, c->x_bigl, c->x_bigl_n, c->x_misc, c->x_bm,
+        launch_extract_write(L, ws, wd, c->x_unit, c->x_bigl, c->x_bigl_n, d_misc, c->x_bm,
                              err, c->sms, st);
         ck(cudaGetLastError(), "extract");
         check();
@@ -2082,7 +2209,9 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
         L.base = uoff[cut[r]];
         L.limit = uoff[cut[r + 1]];
         uint32_t *bs = c->x_src + b * cap, *bd = c->x_dst + b * cap;
-        launch_extract_write(L, bs, bd, c->x_unit, c->x_bigl, c->x_bigl_n, c->x_misc, c->x_bm,
+        // (the cursors start at zero; each further range starts them again)
+        if (r) ck(cudaMemsetAsync(d_misc, 0, 16, st), "memset");
+        launch_extract_write(L, bs, bd, c->x_unit, c->x_bigl, c->x_bigl_n, d_misc, c->x_bm,
                              err, c->sms, st);
         ck(cudaGetLastError(), "extract");
         ck(cudaStreamWaitEvent(lane.s, lane.record(st), 0), "cudaStreamWaitEvent");
@@ -2267,7 +2396,6 @@ int cflr_set_tuning(cflr_ctx *c, const cflr_tuning *t) {
     for (int b = 0; b < 3; b++) n.limit[b] = t->bin_limit[b];
     for (int b = 0; b < 4; b++) n.ctas_per_sm[b] = t->ctas_per_sm[b];
     c->tuning = n;
-    if (c->runner) c->runner->drop_graph();   // the graph holds the old grids
     return CFLR_OK;
 }
 
@@ -2322,7 +2450,6 @@ int cflr_autotune(cflr_ctx *c, uint32_t max_trials, cflr_tuning *best) {
     Tuning found;
     if (cache && cache_lookup(cache, key, found)) {
         c->tuning = found;
-        if (c->runner) c->runner->drop_graph();
         // the schedule does not change the initial matrices: a context that
         // has not run an iteration since its graph was loaded stays as it is
         int rc = c->iterations == 0 ? CFLR_OK : cflr_reset(c);
@@ -2332,7 +2459,6 @@ int cflr_autotune(cflr_ctx *c, uint32_t max_trials, cflr_tuning *best) {
     if (!max_trials) max_trials = 24;
     auto trial = [&](const Tuning &t, double &ms) -> int {
         c->tuning = t;
-        if (c->runner) c->runner->drop_graph();
         int rc = cflr_reset(c);
         if (rc != CFLR_OK) return rc;
         cflr_stats st;
@@ -2385,7 +2511,6 @@ int cflr_autotune(cflr_ctx *c, uint32_t max_trials, cflr_tuning *best) {
         }
     }
     c->tuning = cur;
-    if (c->runner) c->runner->drop_graph();
     rc = cflr_reset(c);
     if (rc != CFLR_OK) return rc;
     if (cache) cache_store(cache, key, cur);
