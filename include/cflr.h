@@ -106,7 +106,7 @@ typedef struct {
                                    graph (it stays usable)                          */
     int order_on_device;        /* where the breadth-first vertex order is found
                                    (unless keep_vertex_order): 0 (default) on the
-                                   GPU for graphs of at least 2^18 edges, on the
+                                   GPU for graphs of at least 2^17 edges, on the
                                    host below that; 1 on the GPU; -1 on the host.
                                    Both give the same order.  The GPU search needs
                                    fewer than 2^32 edges and no vertex with more

@@ -359,7 +359,8 @@ void launch_extract_write(const ExtractList &L, uint32_t *out_src, uint32_t *out
 // scans of cnt (component offsets) and is_root (root offsets, the root count
 // as total), launch_rn_roots (level 0), then per level launch_rn_claim, a
 // scan of won into woff[0..fsize], launch_rn_write (the next frontier into
-// F2, the next segment tables, perm and iperm), until the frontier is empty;
+// F2, the next segment tables, perm and iperm), or launch_rn_levels for a run
+// of levels with small frontiers, until the frontier is empty;
 // launch_rn_check sets *bad unless perm and iperm are inverse permutations.
 constexpr uint32_t RENUM_LIST_MAX = 8192;
 void launch_rn_adjacency(const uint32_t *src, const uint32_t *dst, unsigned long long m,
@@ -388,6 +389,22 @@ void launch_rn_write(const uint32_t *F, uint32_t fsize, const unsigned long long
                      const uint32_t *sf, const uint32_t *se, const uint32_t *pc, uint32_t *sf2,
                      uint32_t *se2, uint32_t *pc2, uint32_t *perm, uint32_t *iperm, uint32_t n,
                      int sms, cudaStream_t st);
+// The same levels while the frontier holds 1 .. limit vertices, on the device
+// (loop: where to start, and afterwards where it stopped).
+struct RnLoop {
+    uint32_t fsize, level, which, placed;   // frontier F[which]; vertices placed by the kernel
+};
+struct RnTables {
+    uint32_t *F[2], *sf[2], *se[2], *pc[2];
+    const unsigned long long *off, *adj;
+    uint32_t *lvl;
+    unsigned long long *key, *woff;
+    const uint32_t *parent;
+    const unsigned long long *comp_off;
+    uint32_t *perm, *iperm;
+};
+void launch_rn_levels(RnLoop *loop, const RnTables &T, uint32_t n, uint32_t limit,
+                      cudaStream_t st);
 void launch_rn_check(const uint32_t *perm, const uint32_t *iperm, uint32_t n, unsigned *bad,
                      int sms, cudaStream_t st);
 

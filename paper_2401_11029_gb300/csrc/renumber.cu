@@ -24,6 +24,8 @@
 // both without a pass of their own.
 #include "kernels.cuh"
 
+#include <cooperative_groups.h>
+
 #include <mutex>
 
 namespace cflr {
@@ -285,6 +287,179 @@ __global__ void __launch_bounds__(256) k_rn_write(
     }
 }
 
+// The levels of a small frontier by one cluster of RN_CTAS CTAs, without the
+// host: claim, count and write as above, with cluster barriers between them.
+// A level of a few thousand vertices is all latency: seven launches and a
+// read of the next size by the host took 28 us of it, and a program-shaped
+// graph has about a hundred levels.  Eight lanes take a frontier vertex (the
+// lists hold about eleven entries; those of more than RN_LONG take the warp),
+// each group a contiguous run of them, so the offsets are a scan of the
+// groups' counts: over the CTA in shared memory, over the cluster through the
+// other CTAs' totals.  Larger frontiers, where
+// eight SMs are too few, go back to the host's launches.
+// The loop ends when the frontier is empty or larger than `limit`, at the
+// latest after n levels (each places a vertex); the barriers are the
+// hardware's.
+constexpr uint32_t RN_CTAS = 8, RN_THREADS = 1024, RN_GROUPS = RN_THREADS / 8;
+constexpr uint32_t RN_LONG = 64;
+
+__global__ void __cluster_dims__(RN_CTAS, 1, 1) __launch_bounds__(RN_THREADS, 1)
+    k_rn_levels(RnLoop *loop, RnTables T, uint32_t n, uint32_t limit) {
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    auto cluster_sync = [&]() {
+        __syncwarp();                          // (the groups of a warp meet again)
+        cl.sync();
+    };
+    __shared__ uint32_t run_sum[RN_GROUPS];    // won by each group's run, then their scan
+    __shared__ uint32_t warp_sum[RN_GROUPS / 32];
+    __shared__ uint32_t cta_won;
+    const uint32_t rank = cl.block_rank();
+    const uint32_t g = threadIdx.x >> 3, gl = threadIdx.x & 7, lane = threadIdx.x & 31;
+    const uint32_t gsh = lane & ~7u, gmask = 0xFFu << gsh;
+    uint32_t fsize = loop->fsize, level = loop->level, b = loop->which, placed = 0;
+    while (fsize && fsize <= limit && level <= n) {
+        const uint32_t *F = T.F[b];
+        uint32_t *F2 = T.F[b ^ 1];
+        const unsigned long long gid = (unsigned long long)rank * RN_GROUPS + g;
+        const uint32_t q0 = (uint32_t)(fsize * gid / (RN_CTAS * RN_GROUPS));
+        const uint32_t q1 = (uint32_t)(fsize * (gid + 1) / (RN_CTAS * RN_GROUPS));
+        // work(q, u, a, e, first lane, lanes, mask) for every vertex of the
+        // run: short lists by the group, then the long ones of the warp's four
+        // runs by the whole warp
+        auto each = [&](auto &&work) {
+            bool any_long = false;
+            for (uint32_t q = q0; q < q1; q++) {
+                const uint32_t u = F[q];
+                const unsigned long long a = T.off[u], e = T.off[u + 1];
+                if (e - a > RN_LONG) any_long = true;
+                else work(q, u, a, e, gl, 8u, gmask);
+            }
+            if (!__any_sync(0xFFFFFFFFu, any_long)) return;
+            for (uint32_t w = 0; w < 32; w += 8) {
+                const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, q0, w);
+                const uint32_t w1 = __shfl_sync(0xFFFFFFFFu, q1, w);
+                for (uint32_t q = w0; q < w1; q++) {
+                    const uint32_t u = F[q];
+                    const unsigned long long a = T.off[u], e = T.off[u + 1];
+                    if (e - a > RN_LONG) work(q, u, a, e, lane, 32u, 0xFFFFFFFFu);
+                }
+            }
+            __syncwarp();
+        };
+        each([&](uint32_t q, uint32_t, unsigned long long a, unsigned long long e, uint32_t l0,
+                 uint32_t lanes, uint32_t) {
+#pragma unroll 4
+            for (unsigned long long j = a + l0; j < e; j += lanes) {
+                const uint32_t v = (uint32_t)T.adj[j];
+                if (T.lvl[v] == RN_UNSEEN)
+                    atomicMin(&T.key[v], ((unsigned long long)q << 32) | (uint32_t)(j - a));
+            }
+        });
+        cluster_sync();
+        each([&](uint32_t q, uint32_t, unsigned long long a, unsigned long long e, uint32_t l0,
+                 uint32_t lanes, uint32_t mask) {
+            uint32_t c = 0;
+#pragma unroll 4
+            for (unsigned long long j = a + l0; j < e; j += lanes) {
+                const uint32_t v = (uint32_t)T.adj[j];
+                c += T.lvl[v] == RN_UNSEEN &&
+                     T.key[v] == (((unsigned long long)q << 32) | (uint32_t)(j - a));
+            }
+            for (uint32_t d = lanes / 2; d > 0; d >>= 1) c += __shfl_xor_sync(mask, c, d);
+            if (l0 == 0) T.woff[q] = c;
+        });
+        // the run's counts into positions from its start
+        uint32_t sum = 0;
+        if (gl == 0) {
+            for (uint32_t q = q0; q < q1; q++) {
+                const uint32_t c = (uint32_t)T.woff[q];
+                T.woff[q] = sum;
+                sum += c;
+            }
+        }
+        if (gl == 0) run_sum[g] = sum;
+        __syncthreads();
+        if (threadIdx.x < RN_GROUPS) {         // four whole warps
+            uint32_t x = run_sum[threadIdx.x];
+            const uint32_t own = x;
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+                if (lane >= (uint32_t)d) x += y;
+            }
+            if (lane == 31) warp_sum[threadIdx.x >> 5] = x;
+            run_sum[threadIdx.x] = x - own;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t t = 0;
+            for (uint32_t w = 0; w < RN_GROUPS / 32; w++) {
+                const uint32_t x = warp_sum[w];
+                warp_sum[w] = t;
+                t += x;
+            }
+            cta_won = t;
+        }
+        cluster_sync();                        // (orders the CTA's threads too)
+        uint32_t before = 0, won = 0;
+        for (uint32_t r = 0; r < RN_CTAS; r++) {
+            const uint32_t x = *cl.map_shared_rank(&cta_won, r);
+            if (r < rank) before += x;
+            won += x;
+        }
+        before += warp_sum[g >> 5] + run_sum[g];
+        if (gl == 0)
+            for (uint32_t q = q0; q < q1; q++) T.woff[q] += before;
+        if (rank == 0 && threadIdx.x == 0) T.woff[fsize] = won;
+        cluster_sync();
+        each([&](uint32_t q, uint32_t u, unsigned long long a, unsigned long long e, uint32_t l0,
+                 uint32_t lanes, uint32_t mask) {
+            const uint32_t r = T.parent[u], sh = lanes == 8 ? gsh : 0u;
+            const uint32_t s0 = T.sf[b][r], s1 = T.se[b][r], p0 = T.pc[b][r];
+            const unsigned long long wbase = T.woff[s0];
+            if (q == s0 && l0 == 0) {
+                T.sf[b ^ 1][r] = (uint32_t)wbase;
+                T.se[b ^ 1][r] = (uint32_t)T.woff[s1];
+                T.pc[b ^ 1][r] = p0 + (s1 - s0);
+            }
+            const unsigned long long pos0 = T.comp_off[r] + p0 + (s1 - s0);
+            unsigned long long t = T.woff[q];
+            for (unsigned long long jb = a; jb < e; jb += lanes) {
+                const unsigned long long j = jb + l0;
+                uint32_t v = 0;
+                bool w = false;
+                if (j < e) {
+                    v = (uint32_t)T.adj[j];
+                    w = T.lvl[v] == RN_UNSEEN &&
+                        T.key[v] == (((unsigned long long)q << 32) | (uint32_t)(j - a));
+                }
+                const unsigned m = (__ballot_sync(mask, w) & mask) >> sh;
+                if (w) {
+                    const unsigned long long tt = t + __popc(m & ((1u << l0) - 1));
+                    const unsigned long long pos = pos0 + (tt - wbase);
+                    T.lvl[v] = level + 1;
+                    if (tt < n) F2[tt] = v;
+                    if (pos < n) {
+                        T.iperm[pos] = v;
+                        T.perm[v] = (uint32_t)pos;
+                    }
+                }
+                t += __popc(m);
+            }
+        });
+        cluster_sync();
+        placed += fsize;
+        fsize = won;
+        level++;
+        b ^= 1;
+    }
+    if (rank == 0 && threadIdx.x == 0) {
+        loop->fsize = fsize;
+        loop->level = level;
+        loop->which = b;
+        loop->placed += placed;
+    }
+}
+
 // *bad = 1 unless perm and iperm are inverse permutations of 0..n-1.
 __global__ void k_rn_check(const uint32_t *perm, const uint32_t *iperm, uint32_t n,
                            unsigned *bad) {
@@ -379,6 +554,11 @@ void launch_rn_write(const uint32_t *F, uint32_t fsize, const unsigned long long
     k_rn_write<<<rn_grid(fsize, 8, sms, 16), 256, 0, st>>>(F, fsize, off, adj, lvl, key, woff, F2,
                                                           level, parent, comp_off, sf, se, pc,
                                                           sf2, se2, pc2, perm, iperm, n);
+}
+
+void launch_rn_levels(RnLoop *loop, const RnTables &T, uint32_t n, uint32_t limit,
+                      cudaStream_t st) {
+    k_rn_levels<<<RN_CTAS, RN_THREADS, 0, st>>>(loop, T, n, limit);
 }
 
 void launch_rn_check(const uint32_t *perm, const uint32_t *iperm, uint32_t n, unsigned *bad,

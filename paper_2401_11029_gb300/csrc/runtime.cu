@@ -1462,6 +1462,12 @@ struct TempArrays {
 // settle in 128 passes, or scratch beyond the context's memory budget.
 bool device_order_steps(cflr_ctx *c, uint32_t n, uint64_t m);
 
+// Frontiers up to which the search's levels run on the device in a row: about
+// where a level takes the cluster as long as the launches and the wait.  Load
+// of the 100k-vertex alias graph 5.3 -> 4.2 ms, 61k points-to 7.4 -> 5.5, 20k
+// alias 3.5 -> 2.0.
+constexpr uint32_t RN_LOOP_MAX = 8192;
+
 bool device_order(cflr_ctx *c, uint32_t n, uint64_t m) {
     if (m >= (1ull << 32)) return false;
     try {
@@ -1529,22 +1535,50 @@ bool device_order_steps(cflr_ctx *c, uint32_t n, uint64_t m) {
     ck(cudaGetLastError(), "renumbering: roots");
     unsigned long long fsize = 0;
     read_word(tot, 8, &fsize);
+    RnTables T{};
+    T.F[0] = F;
+    T.F[1] = F2;
+    for (int q = 0; q < 2; q++) {
+        T.sf[q] = seg[q][0];
+        T.se[q] = seg[q][1];
+        T.pc[q] = seg[q][2];
+    }
+    T.off = off;
+    T.adj = adj;
+    T.lvl = lvl;
+    T.key = key;
+    T.woff = woff;
+    T.parent = parent;
+    T.comp_off = comp_off;
+    T.perm = c->perm;
+    T.iperm = c->iperm;
+    RnLoop *d_loop = tmp.get<RnLoop>(1);
     uint64_t placed = 0;
     int b = 0;
-    for (uint32_t level = 0; fsize; level++) {
+    for (uint32_t level = 0; fsize;) {
         if (level > n) throw Status{CFLR_ECUDA, "internal: the device search did not end"};
+        if (fsize <= RN_LOOP_MAX) {       // a run of small levels on the device
+            RnLoop loop{(uint32_t)fsize, level, (uint32_t)b, 0};
+            ck(cudaMemcpyAsync(d_loop, &loop, sizeof loop, cudaMemcpyHostToDevice, st), "H2D");
+            launch_rn_levels(d_loop, T, n, RN_LOOP_MAX, st);
+            ck(cudaGetLastError(), "renumbering: levels");
+            read_word(d_loop, sizeof loop, &loop);
+            placed += loop.placed;
+            fsize = loop.fsize;
+            level = loop.level;
+            b = (int)loop.which;
+            continue;
+        }
         placed += fsize;
-        launch_rn_claim(F, (uint32_t)fsize, off, adj, lvl, key, won, sms, st);
+        launch_rn_claim(T.F[b], (uint32_t)fsize, off, adj, lvl, key, won, sms, st);
         launch_exclusive_scan(won, (uint32_t)fsize, woff, bsum, woff + fsize, st);
-        launch_rn_write(F, (uint32_t)fsize, off, adj, lvl, key, woff, F2, level, parent, comp_off,
-                        seg[b][0], seg[b][1], seg[b][2], seg[b ^ 1][0], seg[b ^ 1][1],
-                        seg[b ^ 1][2], c->perm, c->iperm, n, sms, st);
+        launch_rn_write(T.F[b], (uint32_t)fsize, off, adj, lvl, key, woff, T.F[b ^ 1], level,
+                        parent, comp_off, seg[b][0], seg[b][1], seg[b][2], seg[b ^ 1][0],
+                        seg[b ^ 1][1], seg[b ^ 1][2], c->perm, c->iperm, n, sms, st);
         ck(cudaGetLastError(), "renumbering: level");
-        unsigned long long next = 0;
-        read_word(woff + fsize, 8, &next);
-        std::swap(F, F2);
+        read_word(woff + fsize, 8, &fsize);
+        level++;
         b ^= 1;
-        fsize = next;
     }
     if (placed != n)
         throw Status{CFLR_ECUDA, "internal: the device search placed " + std::to_string(placed) +
@@ -1635,7 +1669,10 @@ void upload_graph(cflr_ctx *c, uint32_t n, uint64_t m, const uint32_t *src, cons
         c->perm = (uint32_t *)c->dalloc((size_t)n * 4);
         c->iperm = (uint32_t *)c->dalloc((size_t)n * 4);
         const int where = c->cfg.order_on_device;
-        const bool on_device = where > 0 || (where == 0 && m >= (1u << 18));
+        // (about where both take as long: 20k-vertex alias graph, 110k edges, 1.93
+        // ms host and 2.01 device; 41k-vertex field-sensitive one, 112k edges, 3.1
+        // and 2.3; 40k-vertex alias graph, 220k edges, 3.8 and 2.5)
+        const bool on_device = where > 0 || (where == 0 && m >= (1u << 17));
         if (!on_device || !device_order(c, n, m)) {
             Range range("cflr: vertex renumbering (host)");
             const std::vector<uint32_t> order = locality_order(n, m, src, dst);
