@@ -106,6 +106,7 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
 // one 16-byte store clears two slots (clear_table); the caller keeps the
 // load <= 1/2.
 struct HashAcc {
+    static constexpr bool PEEK = false;
     uint32_t *tab;
     int lg;
     unsigned *err;     // gets OVF_FULL if a probe sequence finds the table full
@@ -144,6 +145,7 @@ __device__ __forceinline__ void clear_table(uint32_t *tab, uint32_t lg, uint32_t
 
 // n-bit bitmap of the row (bin 3).
 struct BitmapAcc {
+    static constexpr bool PEEK = true;   // a word's bits can be read without a search
     uint32_t *bm;
 #if defined(CFLR_CHECKED)
     uint32_t words;     // the row's words (checked builds)
@@ -163,6 +165,17 @@ struct BitmapAcc {
         if (!CFLR_CHECK(w < words, err)) return;
 #endif
         atomicOr(&bm[w], b);
+    }
+    // the bits of word w seen now (bits are only ever added), and the bits of
+    // b that this call adds
+    __device__ __forceinline__ uint32_t peek(uint32_t w) const {
+#if defined(CFLR_CHECKED)
+        if (!CFLR_CHECK(w < words, err)) return ~0u;
+#endif
+        return ((volatile uint32_t *)bm)[w];
+    }
+    __device__ __forceinline__ uint32_t add(uint32_t w, uint32_t b) const {
+        return b & ~atomicOr(&bm[w], b);
     }
 };
 
@@ -1114,21 +1127,20 @@ __device__ __forceinline__ unsigned long long group_key(const GroupInfo &gi, uin
 // only when its occupancy bit is set.  Tagged families key the accumulator
 // by member and word, and emit to each member's non-terminal.
 // The 32 tile lists the lanes hold are walked together as one packed
-// sequence of 16-byte tile pairs (see `walk`).  Returns the emitted count.
+// sequence (see `walk_packed`) or list by list.  Returns the emitted count.
 
 // TAGS false: the caller never gets a tagged family group (the bitmap bin:
 // a tagged family stays within bin 2's limit or splits into its members), so
 // the member tags are not carried through the walk.  PACKED: walk the lanes'
 // tile lists as one packed sequence (walk_packed) rather than list by list
-// (walk_lists); WALK_U: 16-byte tile-pair loads each lane of the packed walk
-// has in flight.
+// (walk_lists); WALK_U: 16-byte loads each lane of the packed walk has in
+// flight (two a quad).
 template <bool WIT, bool TAGS, bool PACKED, int WALK_U, class Acc>
 __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab &P,
                                                 const WorkBufs &W, const GroupInfo &gi,
                                                 uint2 own, uint32_t warp_id, uint32_t nwarps,
                                                 int lane, const Acc &acc, CandChunk &ck) {
-    // the packed walk emits two windows' tiles per reservation
-    static_assert(!PACKED || WALK_U % 2 == 0, "the packed walk needs an even depth");
+    static_assert(!PACKED || WALK_U % 2 == 0, "the packed walk loads 32-byte quads");
     const uint32_t dstart = own.x, d = own.y;
     const uint32_t *pool = S.pool[gi.c];
     const size_t oo = (size_t)gi.o * gi.n;
@@ -1293,17 +1305,24 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
         }
     };
     // The tile lists held by the lanes (toff, tn; member tag; delta entry k),
-    // walked as one sequence of 16-byte tile pairs: the lists with tiles are
-    // moved to the front lanes, list l owns the pairs [excl_l, incl_l) of the
-    // sequence, and each lane loads the pair at its position in WALK_U
-    // windows of 32 positions at a time (all loads in flight before any is
-    // used).  The owner of position p is the number of lists that end at or
-    // before p: the lists that end before the window (a ballot) plus those
-    // that end inside it (one bit each, OR-reduced over the warp).  Segments
-    // start on 16-byte boundaries and a tile section holds an even number of
-    // tiles, so a pair never leaves its segment; the second tile of a list's
-    // last pair is ignored when the list has an odd count.
+    // walked as one sequence of 32-byte quads (four tiles): the lists with
+    // tiles are moved to the front lanes, list l owns the quads [excl_l,
+    // incl_l) of the sequence, and each lane loads the quad at its position in
+    // WALK_U / 2 windows of 32 positions at a time (all loads in flight before
+    // any is used).  The owner of position p is the number of lists that end
+    // at or before p: the lists that end before the window (a ballot) plus
+    // those that end inside it (one bit each, OR-reduced over the warp).
+    // Segments start on 16-byte boundaries and a tile section holds an even
+    // number of tiles, so a 16-byte half of a quad that holds a tile never
+    // leaves its section; what a list does not fill of its last quad is zeroed.
+    // The bitmap accumulator is read for all of a lane's tiles before any is
+    // added: nearly every product is already present, so the reads overlap and
+    // one vote decides whether anything follows.  (Finding a list's owner for
+    // every 16-byte pair and testing a tile at a time, 38 instructions per
+    // warp and 32 tiles, bin 3 took 19.5 ms of the 200k alias solve; now
+    // 14.8.)
     auto walk_packed = [&](uint32_t toff, uint32_t tn, uint32_t tag, uint32_t k) {
+        constexpr int U = WALK_U / 2;
         const unsigned nz = __ballot_sync(FULL_MASK, tn != 0);
         if (!nz) return;
         const uint32_t cnt = __popc(nz);
@@ -1313,18 +1332,18 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
         if (TAGS || WIT) tag = __shfl_sync(FULL_MASK, tag, src);
         if (WIT) k = __shfl_sync(FULL_MASK, k, src);
         if ((uint32_t)lane >= cnt) tn = 0;
-        const uint32_t np = (tn + 1) >> 1;
-        const uint32_t incl = warp_incl_scan(np, lane);
-        const uint32_t excl = incl - np;
+        const uint32_t nq = (tn + 3) >> 2;
+        const uint32_t incl = warp_incl_scan(nq, lane);
+        const uint32_t excl = incl - nq;
         const uint32_t total = __shfl_sync(FULL_MASK, incl, 31);
         const uint32_t le = FULL_MASK >> (31 - lane);
-        for (uint32_t b = 0; b < total; b += 32 * WALK_U) {
-            uint4 w[WALK_U];
-            uint32_t nv[WALK_U], tg[WALK_U], kk[WALK_U];
+        for (uint32_t b = 0; b < total; b += 32 * U) {
+            uint4 w[2 * U];
+            uint32_t tg[U], kk[U];
 #pragma unroll
-            for (int u = 0; u < WALK_U; u++) {
-                w[u] = make_uint4(0, 0, 0, 0);
-                nv[u] = tg[u] = kk[u] = 0;
+            for (int u = 0; u < U; u++) {
+                w[2 * u] = w[2 * u + 1] = make_uint4(0, 0, 0, 0);
+                tg[u] = kk[u] = 0;
                 const uint32_t bu = b + 32 * u, p = bu + lane;
                 if (bu >= total) continue;          // uniform: the last windows may be empty
                 const uint32_t first = __popc(__ballot_sync(FULL_MASK, incl <= bu));
@@ -1337,34 +1356,44 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
                 tg[u] = (TAGS || WIT) ? __shfl_sync(FULL_MASK, tag, own) : 0u;
                 kk[u] = WIT ? __shfl_sync(FULL_MASK, k, own) : 0u;
                 if (p < total) {
-                    const uint32_t rel = p - o_excl;
-                    nv[u] = min(2u, o_tn - 2 * rel);
-                    w[u] = *reinterpret_cast<const uint4 *>(pool + o_toff + 4 * rel);
+                    const uint32_t rel = p - o_excl, nv = o_tn - 4 * rel;
+                    const uint4 *q4 = reinterpret_cast<const uint4 *>(pool + o_toff + 8 * rel);
+                    w[2 * u] = q4[0];
+                    if (nv > 2) w[2 * u + 1] = q4[1];
+                    if (nv == 1) w[2 * u].z = w[2 * u].w = 0;
+                    if (nv == 3) w[2 * u + 1].z = w[2 * u + 1].w = 0;
                 }
             }
-            uint32_t nb[2 * WALK_U], any = 0;
+            uint32_t nb[4 * U], any = 0;
+            if constexpr (Acc::PEEK) {
 #pragma unroll
-            for (int u = 0; u < WALK_U; u++) {
-                nb[2 * u] = nv[u] > 0 ? acc.ins(key_of(w[u].x, tg[u]), w[u].y) : 0u;
-                nb[2 * u + 1] = nv[u] > 1 ? acc.ins(key_of(w[u].z, tg[u]), w[u].w) : 0u;
-                any |= nb[2 * u] | nb[2 * u + 1];
-            }
-            // nearly every product is already present: one vote, then the
-            // new bits go out four tiles per reservation (with tags or
-            // witnesses, one window's pair at a time)
-            if (__any_sync(FULL_MASK, any != 0)) {
-                if constexpr (!TAGS && !WIT) {
-#pragma unroll
-                    for (int u = 0; u < WALK_U; u += 2)
-                        emit_bits(nb[2 * u], w[u].x, nb[2 * u + 1], w[u].z, nb[2 * u + 2],
-                                  w[u + 1].x, nb[2 * u + 3], w[u + 1].z, 0u, 0u);
-                } else {
-#pragma unroll
-                    for (int u = 0; u < WALK_U; u++)
-                        emit_bits(nb[2 * u], w[u].x, nb[2 * u + 1], w[u].z, 0u, 0u, 0u, 0u, tg[u],
-                                  kk[u]);
+                for (int i = 0; i < 2 * U; i++) {
+                    nb[2 * i] = w[i].y & ~acc.peek(w[i].x);
+                    nb[2 * i + 1] = w[i].w & ~acc.peek(w[i].z);
+                    any |= nb[2 * i] | nb[2 * i + 1];
                 }
+                if (!__any_sync(FULL_MASK, any != 0)) continue;
+#pragma unroll
+                for (int i = 0; i < 2 * U; i++) {
+                    if (nb[2 * i]) nb[2 * i] = acc.add(w[i].x, nb[2 * i]);
+                    if (nb[2 * i + 1]) nb[2 * i + 1] = acc.add(w[i].z, nb[2 * i + 1]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 2 * U; i++) {
+                    nb[2 * i] = w[i].y ? acc.ins(key_of(w[i].x, tg[i / 2]), w[i].y) : 0u;
+                    nb[2 * i + 1] = w[i].w ? acc.ins(key_of(w[i].z, tg[i / 2]), w[i].w) : 0u;
+                    any |= nb[2 * i] | nb[2 * i + 1];
+                }
+                if (!__any_sync(FULL_MASK, any != 0)) continue;
             }
+            // the new bits go out a quad per reservation
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (__any_sync(FULL_MASK, (nb[4 * u] | nb[4 * u + 1] | nb[4 * u + 2] |
+                                           nb[4 * u + 3]) != 0))
+                    emit_bits(nb[4 * u], w[2 * u].x, nb[4 * u + 1], w[2 * u].z, nb[4 * u + 2],
+                              w[2 * u + 1].x, nb[4 * u + 3], w[2 * u + 1].z, tg[u], kk[u]);
         }
     };
     auto walk = [&](uint32_t toff, uint32_t tn, uint32_t tag, uint32_t k) {
