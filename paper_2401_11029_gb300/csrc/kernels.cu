@@ -1107,6 +1107,75 @@ __device__ __forceinline__ uint2 owner_delta(const SlotTab &S, const GroupInfo &
     return make_uint2(dsc.x + tile_words(dsc.z), d);
 }
 
+// What a group's product needs before its first tile, decoded ahead by bin 0:
+// a warp takes a few neighbouring groups and a lane each follows the chain
+// group -> production -> descriptors for all of them at once (48 bytes a
+// group in shared memory).  Decoding a group when its turn came put seven
+// dependent loads before its first tile, and these groups hold a few dozen
+// tiles (bin 0 of the 500k points-to solve 12.7 -> 11.4 ms).  Neighbours, not
+// groups at a stride: they often share a row, and a stride cost bins 1 and 3
+// more than the chain (200k alias pass 48.5 -> 50.5 ms).
+struct GroupMeta {
+    uint32_t bits, idx, c, a, b, n, first, F;
+    uint32_t mask_off, mask_n;      // mask row: pool offset and tiles
+    uint32_t dstart, d;             // delta entries: pool offset and count
+};
+
+__device__ __forceinline__ GroupMeta group_meta(const ProdTab &P, const SlotTab &S, uint2 g,
+                                                unsigned *err) {
+    const GroupInfo gi = decode_group(P, S, g);
+    GroupMeta m;
+    m.bits = gi.part | (gi.probe ? 4u : 0u) | (gi.fam ? 8u : 0u) | (gi.tagged ? 16u : 0u) |
+             (gi.consec ? 32u : 0u) | gi.lg << 8;
+    m.idx = gi.idx;
+    m.c = gi.c;
+    m.a = gi.a;
+    m.b = gi.b;
+    m.n = gi.n;
+    m.first = gi.first;
+    m.F = gi.F;
+    m.mask_off = m.mask_n = 0;
+    if (!gi.probe) {
+        const uint4 md = S.desc[gi.c][(size_t)gi.o * gi.n + gi.idx];
+        if (row_in_pool(S, gi.c, md, err)) {
+            m.mask_off = md.x;
+            m.mask_n = md.y;
+        }
+    }
+    const uint2 own = owner_delta(S, gi, err);
+    m.dstart = own.x;
+    m.d = own.y;
+    return m;
+}
+
+__device__ __forceinline__ GroupInfo group_info(const GroupMeta &m) {
+    GroupInfo gi;
+    gi.part = m.bits & 3;
+    gi.probe = m.bits & 4;
+    gi.fam = m.bits & 8;
+    gi.tagged = m.bits & 16;
+    gi.consec = m.bits & 32;
+    gi.lg = m.bits >> 8;
+    gi.o = gi.part == PART_B ? 1u : 0u;
+    gi.idx = m.idx;
+    gi.c = m.c;
+    gi.a = m.a;
+    gi.b = m.b;
+    gi.n = m.n;
+    gi.first = m.first;
+    gi.F = m.F;
+    return gi;
+}
+
+// Groups of a batch (few: the 48 bytes of each are taken from the L1 cache).
+constexpr uint32_t BATCH_MAX = 8;
+
+// log2 of the groups of a batch when `takers` warps share n groups: at least
+// four batches each, and single groups when there are few.
+__device__ __forceinline__ uint32_t batch_log2(unsigned long long n, unsigned long long takers) {
+    return n >= 32 * takers ? 3u : n >= 16 * takers ? 2u : n >= 8 * takers ? 1u : 0u;
+}
+
 __device__ __forceinline__ unsigned long long group_key(const GroupInfo &gi, uint32_t v) {
     // row groups produce (idx, v); column groups produce (v, idx)
     return gi.o ? (((unsigned long long)v << 32) | gi.idx)
@@ -1597,21 +1666,39 @@ __device__ __forceinline__ void preload_mask(const SlotTab &S, const GroupInfo &
     }
 }
 
+// The same for a group decoded ahead.
+template <class Acc>
+__device__ __forceinline__ void preload_mask_ahead(const SlotTab &S, const GroupMeta &m, const Acc &acc,
+                                             uint32_t tid, uint32_t nth) {
+    const uint32_t *tl = S.pool[m.c] + m.mask_off;
+    for (uint32_t q = tid; 2 * q < m.mask_n; q += nth) {
+        const uint4 t = *reinterpret_cast<const uint4 *>(tl + 4 * q);
+        acc.set(t.x, t.y);
+        if (2 * q + 1 < m.mask_n) acc.set(t.z, t.w);
+    }
+}
+
 // Bin 0: one warp per group, a private shared-memory table per warp (2^LG
 // words and their bits).
 template <int LG, int WARPS, bool WIT>
 __global__ void __launch_bounds__(WARPS * 32, 4) k_spgemm_warp(SlotTab S, ProdTab P, WorkBufs W,
                                                                int bin) {
     extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ GroupMeta meta_sh[WARPS][BATCH_MAX];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     uint32_t *tab = smem + (size_t)wib * (2u << LG);
     const unsigned long long n_groups =
         min(W.cnt->groups[bin], W.group_cap[bin]);
     const unsigned long long nw = (unsigned long long)gridDim.x * WARPS;
+    const uint32_t lgb = batch_log2(n_groups, nw);
+    const unsigned long long nb = (n_groups + (1u << lgb) - 1) >> lgb;
     CandChunk ck{0, 0};
     unsigned long long bytes = 0;
-    for (unsigned long long g = (unsigned long long)blockIdx.x * WARPS + wib; g < n_groups;
-         g += nw) {
+    // Fewer than eight groups a warp: one at a time, at a stride.  Handing the
+    // group's data through shared memory and claims on one address would cost
+    // each launch 2 to 3 us (100k value-flow pass 2.32 -> 2.38 ms).
+    for (unsigned long long g = lgb ? n_groups : (unsigned long long)blockIdx.x * WARPS + wib;
+         g < n_groups; g += nw) {
         const GroupInfo gi = decode_group(P, S, W.groups[bin][g]);
         const int lg = min((int)gi.lg, LG);
         clear_table(tab, lg, lane, 32);
@@ -1622,13 +1709,45 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_spgemm_warp(SlotTab S, ProdTa
             __syncwarp();
         }
         const uint2 own = owner_delta(S, gi, &W.cnt->overflow);
-        const uint32_t e =
+        const uint32_t em =
             expand_rows<WIT, true, false, 2>(S, P, W, gi, own, 0, 1, lane, acc, ck);
-        if (lane == 0 && e) {
-            if (!gi.tagged) atomicAdd(&S.cand[gi.c], (unsigned long long)e);
-            bytes += 12ull * e;
+        if (lane == 0 && em) {
+            if (!gi.tagged) atomicAdd(&S.cand[gi.c], (unsigned long long)em);
+            bytes += 12ull * em;
         }
         __syncwarp();
+    }
+    // More: batches decoded ahead, the first by the warp's number, the others
+    // claimed from a cursor (the next one while this one runs)
+    unsigned long long c = lgb ? (unsigned long long)blockIdx.x * WARPS + wib : nb;
+    while (c < nb) {
+        unsigned long long c_next = nb;
+        if (lane == 0) c_next = nw + atomicAdd(&W.cnt->claim[bin], 1ull);
+        const unsigned long long e = (c << lgb) + lane;
+        const bool has = lane < (1 << lgb) && e < n_groups;
+        if (has) meta_sh[wib][lane] = group_meta(P, S, W.groups[bin][e], &W.cnt->overflow);
+        const int cnt = __popc(__ballot_sync(FULL_MASK, has));   // the first lanes
+        __syncwarp();
+        for (int l = 0; l < cnt; l++) {
+            const GroupMeta &m = meta_sh[wib][l];
+            const GroupInfo gi = group_info(m);
+            const int lg = min((int)gi.lg, LG);
+            clear_table(tab, lg, lane, 32);
+            __syncwarp();
+            const HashAcc acc{tab, lg, &W.cnt->overflow};
+            if (!gi.probe) {
+                preload_mask_ahead(S, m, acc, lane, 32);
+                __syncwarp();
+            }
+            const uint32_t em = expand_rows<WIT, true, false, 2>(
+                S, P, W, gi, make_uint2(m.dstart, m.d), 0, 1, lane, acc, ck);
+            if (lane == 0 && em) {
+                if (!gi.tagged) atomicAdd(&S.cand[gi.c], (unsigned long long)em);
+                bytes += 12ull * em;
+            }
+            __syncwarp();
+        }
+        c = __shfl_sync(FULL_MASK, c_next, 0);
     }
     release_chunk(W, ck, lane);
     if (lane == 0 && bytes) atomicAdd(&W.cnt->bytes_bin[bin], bytes);
