@@ -106,13 +106,21 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
 // one 16-byte store clears two slots (clear_table); the caller keeps the
 // load <= 1/2.
 struct HashAcc {
-    static constexpr bool PEEK = false;
     uint32_t *tab;
     int lg;
     unsigned *err;     // gets OVF_FULL if a probe sequence finds the table full
+    __device__ __forceinline__ uint32_t home(uint32_t w) const {
+        return (w * 2654435761u) >> (32 - lg);
+    }
+    // a slot's word and bits in one 8-byte read (one after the other, the 200k
+    // alias solve took 39.4 ms instead of 38.9)
+    __device__ __forceinline__ uint2 slot(uint32_t s) const {
+        const unsigned long long v = ((volatile unsigned long long *)tab)[s];
+        return make_uint2((uint32_t)v, (uint32_t)(v >> 32));
+    }
     __device__ __forceinline__ uint32_t ins(uint32_t w, uint32_t b) const {
         const uint32_t m = (1u << lg) - 1;
-        uint32_t s = (w * 2654435761u) >> (32 - lg);
+        uint32_t s = home(w), have = 0;
         // at most one pass over the table (the callers keep it at most half
         // full, so the pass always ends early)
         for (uint32_t p = 0;; p++) {
@@ -120,19 +128,26 @@ struct HashAcc {
                 atomicOr(err, OVF_FULL);
                 return 0;
             }
-            const uint32_t cur = ((volatile uint32_t *)tab)[2 * s];
-            if (cur == w) break;
-            if (cur == EMPTY32) {
+            const uint2 cur = slot(s);
+            have = cur.y;
+            if (cur.x == w) break;
+            if (cur.x == EMPTY32) {
                 const uint32_t old = atomicCAS(&tab[2 * s], EMPTY32, w);
                 if (old == EMPTY32 || old == w) break;
             }
             s = (s + 1) & m;
         }
-        const uint32_t ob = ((volatile uint32_t *)tab)[2 * s + 1];
-        if ((ob & b) == b) return 0;
+        if ((have & b) == b) return 0;
         return b & ~atomicOr(&tab[2 * s + 1], b);
     }
     __device__ __forceinline__ void set(uint32_t w, uint32_t b) const { ins(w, b); }
+    // bits of word w known to be present (those of its first slot, if that is
+    // the word's), and the bits of b that this call adds
+    __device__ __forceinline__ uint32_t peek(uint32_t w) const {
+        const uint2 cur = slot(home(w));
+        return cur.x == w ? cur.y : 0u;
+    }
+    __device__ __forceinline__ uint32_t add(uint32_t w, uint32_t b) const { return ins(w, b); }
 };
 
 // Empty all 2^lg slots of a table (16-byte aligned, lg >= 1); thread tid of nth.
@@ -145,7 +160,6 @@ __device__ __forceinline__ void clear_table(uint32_t *tab, uint32_t lg, uint32_t
 
 // n-bit bitmap of the row (bin 3).
 struct BitmapAcc {
-    static constexpr bool PEEK = true;   // a word's bits can be read without a search
     uint32_t *bm;
 #if defined(CFLR_CHECKED)
     uint32_t words;     // the row's words (checked builds)
@@ -1384,8 +1398,7 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
     // Segments start on 16-byte boundaries and a tile section holds an even
     // number of tiles, so a 16-byte half of a quad that holds a tile never
     // leaves its section; what a list does not fill of its last quad is zeroed.
-    // The bitmap accumulator is read for all of a lane's tiles before any is
-    // added: nearly every product is already present, so the reads overlap and
+    // The accumulator is read for all of a lane's tiles before any is added: nearly every product is already present, so the reads overlap and
     // one vote decides whether anything follows.  (Finding a list's owner for
     // every 16-byte pair and testing a tile at a time, 38 instructions per
     // warp and 32 tiles, bin 3 took 19.5 ms of the 200k alias solve; now
@@ -1434,27 +1447,18 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
                 }
             }
             uint32_t nb[4 * U], any = 0;
-            if constexpr (Acc::PEEK) {
 #pragma unroll
-                for (int i = 0; i < 2 * U; i++) {
-                    nb[2 * i] = w[i].y & ~acc.peek(w[i].x);
-                    nb[2 * i + 1] = w[i].w & ~acc.peek(w[i].z);
-                    any |= nb[2 * i] | nb[2 * i + 1];
-                }
-                if (!__any_sync(FULL_MASK, any != 0)) continue;
+            for (int i = 0; i < 2 * U; i++) {
+                nb[2 * i] = w[i].y & ~acc.peek(key_of(w[i].x, tg[i / 2]));
+                nb[2 * i + 1] = w[i].w & ~acc.peek(key_of(w[i].z, tg[i / 2]));
+                any |= nb[2 * i] | nb[2 * i + 1];
+            }
+            if (!__any_sync(FULL_MASK, any != 0)) continue;
 #pragma unroll
-                for (int i = 0; i < 2 * U; i++) {
-                    if (nb[2 * i]) nb[2 * i] = acc.add(w[i].x, nb[2 * i]);
-                    if (nb[2 * i + 1]) nb[2 * i + 1] = acc.add(w[i].z, nb[2 * i + 1]);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 2 * U; i++) {
-                    nb[2 * i] = w[i].y ? acc.ins(key_of(w[i].x, tg[i / 2]), w[i].y) : 0u;
-                    nb[2 * i + 1] = w[i].w ? acc.ins(key_of(w[i].z, tg[i / 2]), w[i].w) : 0u;
-                    any |= nb[2 * i] | nb[2 * i + 1];
-                }
-                if (!__any_sync(FULL_MASK, any != 0)) continue;
+            for (int i = 0; i < 2 * U; i++) {
+                if (nb[2 * i]) nb[2 * i] = acc.add(key_of(w[i].x, tg[i / 2]), nb[2 * i]);
+                if (nb[2 * i + 1])
+                    nb[2 * i + 1] = acc.add(key_of(w[i].z, tg[i / 2]), nb[2 * i + 1]);
             }
             // the new bits go out a quad per reservation
 #pragma unroll
@@ -3457,8 +3461,9 @@ constexpr size_t BIN1S_SMEM = 4 * 2 * 1024 * 4;  // 4 parts x 1024 slots (limit 
 constexpr size_t BIN2_SMEM = 2 * 8192 * 4;
 constexpr size_t BIN2S_SMEM = 2 * 4096 * 4;       // limit <= 2048
 constexpr size_t SMEM_BITMAP_MAX = 200 * 1024;
-// Bin 1 walks list by list: the packed walk took 93.3 ms for the 500k-vertex
-// points-to solve against 91.9, and 44.5 against 44.8 for the 200k alias solve.
+// Bin 1 walks list by list: packed it took 4.4 ms of the 200k alias solve's sum
+// instead of 4.8, but 12.9 instead of 12.4 of the 500k points-to solve's and
+// 4.1 instead of 3.6 of the 61k one's.
 constexpr bool BIN1_PACKED = false;
 
 static void set_smem_attrs();
