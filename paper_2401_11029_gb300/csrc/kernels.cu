@@ -3601,6 +3601,7 @@ void launch_capacity_big(const SlotTab &S, const InstTab &I, const WorkBufs &W, 
     const bool sm = bm_bytes <= SMEM_BITMAP_MAX;
     int per_sm = sm ? (int)((220 * 1024) / (bm_bytes + 3072)) : 8;
     per_sm = per_sm < 1 ? 1 : (per_sm > 8 ? 8 : per_sm);
+    per_sm = per_sm > 2 ? 2 : per_sm;      // few rows are that long
     k_capacity_big<<<sms * per_sm, 256, sm ? bm_bytes : 0, st>>>(S, I, W, sm ? 1 : 0);
 }
 

@@ -466,10 +466,10 @@ struct Runner {
     std::vector<uint32_t> slot_ctx;    // slot -> context index
     // Device tables: views into one block, laid out by bind() as the grammar's
     // part (productions, uses), the graphs' part (pointers, sizes), the state
-    // (uploaded by bind, read back by read_status) and counters that stay on
-    // the device.  The host's mirror has the same layout up to the state's end.
+    // (uploaded by bind, read back by read_status) and counters that are only
+    // uploaded (zero).  The host's mirror has the same layout.
     DevArr<char> d_block;
-    size_t off_graphs = 0, off_htab = 0, off_pool = 0, off_state = 0, off_end = 0;
+    size_t off_graphs = 0, off_htab = 0, off_pool = 0, off_state = 0, off_read = 0, off_end = 0;
     View<uint4 *> d_desc;
     View<uint2 *> d_dn;
     View<uint32_t *> d_pool;
@@ -717,8 +717,9 @@ struct Runner {
                      o_tn = take(16), o_par = take(sizeof(int)), o_ptop = take(ni * 8),
                      o_nnz = take(ns * 8), o_cand = take(ns * 8), o_iters = take(ni * 4),
                      o_act = take(ni * 4);
-        off_end = at;
+        off_read = at;
         const size_t o_delta = take(ns * 8), o_idelta = take(ni * 8);
+        off_end = at;
         sync("bind");                     // the mirror's last copy is done with
         if (keep && (at > d_block.n || off_end > kit->tables.n)) {
             // the block moves: the grammar's part goes with it
@@ -803,9 +804,10 @@ struct Runner {
             h_active[k] = c->touched_n ? 1u : 0u;
             touched += c->touched_n;
         }
+        std::memset(h + o_delta, 0, off_end - o_delta);
         fill_htabs();
         fill_pools();
-        // loop state: parity 0, the pending delta rows (import_touched brings
+        // loop state, with every counter zero: parity 0, the pending delta rows (import_touched brings
         // them), iteration count 0
         *h_ctl = LoopCtl{};
         h_ctl->limit = own->cfg.max_iterations ? own->cfg.max_iterations : 0xFFFFFFFFu;
@@ -1064,19 +1066,23 @@ struct Runner {
                 ck(cudaStreamWaitEvent(st, kit->join[q], 0), "join");
         }
     }
-    // Commit and union, from the dedupe (stage 0), the capacity pass
-    // (stage 1) or the scatter (stage 2), then the end of the iteration.
+    // Commit and union, from the dedupe (stage 0, or -1 for the terminal
+    // initialisation), the capacity pass (stage 1) or the scatter (stage 2), then the end of the iteration.
     void launch_merge(const SlotTab &S, const InstTab &I, const WorkBufs &W, int stage,
                       bool count_iteration, bool in_graph, bool timed, bool check) {
         auto run = [&](int kid, auto f) { if (timed) prof.run(kid, f); else f(); };
         if (stage <= 0) {
             // the previous deltas end before the commit counts the new ones
-            run(KID_RESET, [&] { launch_check_reset(S, W, n_slots, check, sms, st); });
+            // (stage -1, the terminal initialisation, has none)
+            if (stage == 0)
+                run(KID_RESET, [&] { launch_check_reset(S, W, n_slots, check, sms, st); });
             run(KID_COMMIT, [&] { launch_commit(S, W, n_slots, sms, st); });
         }
         if (stage <= 1) {
             run(KID_CAPACITY, [&] { launch_capacity(S, I, W, sms, st); });
-            run(KID_CAPACITY_BIG, [&] { launch_capacity_big(S, I, W, max_n, sms, st); });
+            // (at the terminal initialisation no row holds tiles yet)
+            if (stage >= 0)
+                run(KID_CAPACITY_BIG, [&] { launch_capacity_big(S, I, W, max_n, sms, st); });
         }
         run(KID_SCATTER, [&] { launch_scatter(S, W, sms, st); });
         run(KID_PACK, [&] { launch_pack(S, W, sms, st); });
@@ -1156,7 +1162,7 @@ struct Runner {
 
     // The state into the mirror (one copy, one wait).
     void read_status() {
-        ck(cudaMemcpyAsync(kit->tables.p + off_state, d_block.p + off_state, off_end - off_state,
+        ck(cudaMemcpyAsync(kit->tables.p + off_state, d_block.p + off_state, off_read - off_state,
                            cudaMemcpyDeviceToHost, st), "D2H");
         sync("status");
     }
@@ -1239,7 +1245,6 @@ struct Runner {
         // them needs no growth, and only then captures the graph again (a
         // fresh context grows several buffers in its first iterations).
         bool settled = use_graph && graph_fits();
-        zero_counters();
         for (;;) {
             if (use_graph && settled) {
                 Range range("cflr: closure loop (CUDA graph)");
@@ -1794,7 +1799,6 @@ void reset_matrices(cflr_ctx *c) {
     const SlotTab S = r.slots();
     const InstTab I = r.insttab();
     const WorkBufs W = r.work();
-    launch_iter_begin(S, I, W, r.n_slots, 1, st);
     r.prof.run(KID_INIT, [&] {
         launch_init_edges(c->e_src, c->e_lab, c->e_dst, c->m_edges, c->t_off, c->t_slot, nterm, W,
                           c->sms, st);
@@ -1803,7 +1807,7 @@ void reset_matrices(cflr_ctx *c) {
     c->k_bytes[KID_INIT] += 12 * c->m_edges + 12 * c->n_init;
     // the pair sets were sized from the exact initial counts, so the commit
     // needs no capacity check; the pool may still grow
-    r.launch_merge(S, I, W, 0, false, false, true, false);
+    r.launch_merge(S, I, W, -1, false, false, true, false);
     r.read_status();
     if (r.h_cnt->overflow & OVF_CAND) throw Status{CFLR_ECUDA, "internal: init overflow"};
     if (r.h_ctl->status) r.recover();
