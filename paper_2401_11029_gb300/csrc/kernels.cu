@@ -1910,24 +1910,33 @@ __global__ void __launch_bounds__(256) k_commit(SlotTab S, WorkBufs W, uint32_t 
     __shared__ unsigned stop;
     // one read for the CTA (this kernel's own threads may set OVF_FULL, and
     // every thread must take the same path to the barriers below)
-    if (threadIdx.x == 0) stop = W.cnt->overflow & OVF_STOP;
-    __syncthreads();
-    if (stop) return;                          // the iteration is re-run after a growth
+    if (threadIdx.x == 0) {
+        stop = W.cnt->overflow & OVF_STOP;
+        n_new = n_touch = 0;
+    }
     const int lane = threadIdx.x & 31;
     const int par = *W.parity;
     unsigned long long *out_n = &W.touched_n[par ^ 1];
     uint2 *t_out = W.touched[par ^ 1];
     const unsigned long long nc = min(W.cnt->cand, W.cand_cap);
-    if ((unsigned long long)blockIdx.x * COMMIT_ROUND >= nc) return;   // no round for this CTA
     const bool hist = n_slots <= COMMIT_SLOTS;
     if (hist)
         for (uint32_t s = threadIdx.x; s < n_slots; s += blockDim.x) slot_new[s] = 0;
-    if (threadIdx.x == 0) n_new = n_touch = 0;
     __syncthreads();
+    if (stop) return;                          // the iteration is re-run after a growth
+    // A candidate per thread when the grid holds them all: a small launch is
+    // then one chain of probe and atomics long instead of two (24 us a launch
+    // on the 613-vertex alias graph, whose one-shot solve went from 1.80 to
+    // 1.75 ms, Dyck-1 of 1000 vertices from 1.48 to 1.44).  A larger one is
+    // bound by the reservations, which rounds of 512 halve (200k alias solve:
+    // commit 5.9 ms, 6.3 at 256).
+    const uint32_t round =
+        nc > (unsigned long long)gridDim.x * blockDim.x ? COMMIT_ROUND : blockDim.x;
+    if ((unsigned long long)blockIdx.x * round >= nc) return;   // no round for this CTA
     uint32_t mine = 0;                         // new pairs of this warp (lane 0)
-    for (unsigned long long r0 = (unsigned long long)blockIdx.x * COMMIT_ROUND; r0 < nc;
-         r0 += (unsigned long long)gridDim.x * COMMIT_ROUND) {
-        for (uint32_t q = 0; q < COMMIT_ROUND; q += blockDim.x) {
+    for (unsigned long long r0 = (unsigned long long)blockIdx.x * round; r0 < nc;
+         r0 += (unsigned long long)gridDim.x * round) {
+        for (uint32_t q = 0; q < round; q += blockDim.x) {
             const unsigned long long t = r0 + q + threadIdx.x;
             bool isnew = false;
             unsigned long long key = 0;
