@@ -2681,6 +2681,64 @@ __global__ void k_rehash(const unsigned long long *old_tab, const uint2 *old_val
     }
 }
 
+// Entries of a pair set a CTA clears at a time.
+constexpr uint32_t CLEAR_CHUNK = 4096;   // 32 KB: 128 bytes a thread
+
+// Move many small pair sets into larger tables, in one launch per phase for
+// all of them (phase 0 empties the new tables, phase 1 moves the keys): a fill
+// and a move per set cost the host 5 us a set, and a fresh points-to solve
+// grows hundreds (61k points-to graph, load to read-out: 27.0 -> 25.5 ms).  A table is
+// cut into chunks numbered over all sets (first[k]: set k's first chunk, of the
+// new tables in phase 0, of the old ones in phase 1).  The chunks of the move
+// are short, so that a few hundred thousand entries spread over the chip: a
+// thread's keys are loaded together, but their probes are a chain of atomics.
+constexpr uint32_t MOVE_CHUNK = 1024;    // four entries a thread
+
+__global__ void __launch_bounds__(256) k_rehash_many(const GrownSet *sets, uint32_t count,
+                                                     int phase, unsigned *err) {
+    const unsigned long long chunks = sets[count].first[phase];
+    for (unsigned long long k = blockIdx.x; k < chunks; k += gridDim.x) {
+        uint32_t lo = 0, hi = count;              // first[lo] <= k < first[hi]
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (sets[mid].first[phase] <= k) lo = mid;
+            else hi = mid;
+        }
+        const GrownSet g = sets[lo];
+        if (phase == 0) {
+            const unsigned long long e0 = (k - g.first[0]) * CLEAR_CHUNK;
+            const uint32_t n2 =
+                (uint32_t)(min((unsigned long long)CLEAR_CHUNK, g.new_cap - e0) / 2);
+            uint4 *p = reinterpret_cast<uint4 *>(g.new_tab + e0);
+            for (uint32_t q = threadIdx.x; q < n2; q += 256)
+                p[q] = make_uint4(EMPTY32, EMPTY32, EMPTY32, EMPTY32);
+            continue;
+        }
+        const unsigned long long e0 = (k - g.first[1]) * MOVE_CHUNK;
+        const unsigned long long e1 = min(e0 + MOVE_CHUNK, g.old_cap), m = g.new_cap - 1;
+        unsigned long long keys[MOVE_CHUNK / 256];
+#pragma unroll
+        for (uint32_t q = 0; q < MOVE_CHUNK / 256; q++) {
+            const unsigned long long s = e0 + threadIdx.x + 256 * q;
+            keys[q] = s < e1 ? g.old_tab[s] : EMPTY_KEY;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < MOVE_CHUNK / 256; q++) {
+            const unsigned long long key = keys[q], s = e0 + threadIdx.x + 256 * q;
+            if (key == EMPTY_KEY) continue;
+            unsigned long long h = pair_home(key, m);
+            unsigned long long p = 0;     // one pass at most (the new set is at most 1/4 full)
+            while (atomicCAS(&g.new_tab[h], EMPTY_KEY, key) != EMPTY_KEY && ++p <= m)
+                h = (h + 1) & m;
+            if (p > m) {
+                atomicOr(err, OVF_FULL);
+                continue;
+            }
+            if (g.new_val) g.new_val[h] = g.old_val[s];
+        }
+    }
+}
+
 // The recorded derivation step of one pair (single thread): {~0, ~0} when
 // the pair is not in the set.
 __global__ void k_witness_lookup(const unsigned long long *tab, const uint2 *val,
@@ -2712,7 +2770,6 @@ __global__ void k_fill_u64(unsigned long long *p, unsigned long long count,
 // field-sensitive alias pass from 13.7 to 12.2 ms).  The sets are cut into chunks of CLEAR_CHUNK entries, numbered over
 // all sets; every block finds the sets of its chunks itself, from a scan of
 // CLEAR_SEG slots' chunk counts at a time, so the host prepares no table.
-constexpr uint32_t CLEAR_CHUNK = 4096;   // 32 KB: 128 bytes a thread
 constexpr uint32_t CLEAR_SEG = 2048;     // slots scanned at a time, 8 a thread
 
 __global__ void __launch_bounds__(256) k_clear_sets(SlotTab S, uint32_t n_slots) {
@@ -3678,6 +3735,18 @@ void launch_rehash(const unsigned long long *old_tab, const uint2 *old_val,
                    unsigned long long new_cap, unsigned *err, int sms, cudaStream_t st) {
     k_rehash<<<grid_for(old_cap, 256, sms, 8), 256, 0, st>>>(old_tab, old_val, old_cap, new_tab,
                                                               new_val, new_cap, err);
+}
+
+unsigned long long set_chunks(unsigned long long cap, int phase) {
+    const uint32_t c = phase ? MOVE_CHUNK : CLEAR_CHUNK;
+    return (cap + c - 1) / c;
+}
+
+void launch_rehash_many(const GrownSet *sets, uint32_t count, unsigned long long new_chunks,
+                        unsigned long long old_chunks, unsigned *err, int sms, cudaStream_t st) {
+    if (!count) return;
+    k_rehash_many<<<grid_for(new_chunks, 1, sms, 8), 256, 0, st>>>(sets, count, 0, err);
+    k_rehash_many<<<grid_for(old_chunks, 1, sms, 8), 256, 0, st>>>(sets, count, 1, err);
 }
 
 void launch_witness_lookup(const unsigned long long *tab, const uint2 *val,

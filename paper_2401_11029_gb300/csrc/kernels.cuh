@@ -258,6 +258,21 @@ void launch_init_eps(uint32_t slot, uint32_t n, const WorkBufs &W, int sms, cuda
 void launch_rehash(const unsigned long long *old_tab, const uint2 *old_val,
                    unsigned long long old_cap, unsigned long long *new_tab, uint2 *new_val,
                    unsigned long long new_cap, unsigned *err, int sms, cudaStream_t st);
+// The same for many sets.  sets (on the device): one record per set and one
+// past the end that holds only the chunk totals, first[0] counting the new
+// tables' chunks (set_chunks of their capacities, phase 0), first[1] the old
+// ones' (phase 1).
+struct GrownSet {
+    const unsigned long long *old_tab;
+    const uint2 *old_val;
+    unsigned long long *new_tab;
+    uint2 *new_val;
+    unsigned long long old_cap, new_cap;
+    unsigned long long first[2];
+};
+unsigned long long set_chunks(unsigned long long cap, int phase);
+void launch_rehash_many(const GrownSet *sets, uint32_t count, unsigned long long new_chunks,
+                        unsigned long long old_chunks, unsigned *err, int sms, cudaStream_t st);
 // The witness of pair `key` in a pair set of capacity mask + 1, written to
 // *out ({~0, ~0} when the pair is absent).
 void launch_witness_lookup(const unsigned long long *tab, const uint2 *val,

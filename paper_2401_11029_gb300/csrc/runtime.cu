@@ -504,6 +504,7 @@ struct Runner {
     DevArr<uint32_t> d_cand_slot;
     DevArr<uint2> d_cand_pos;
     DevArr<uint32_t> d_bitmap;
+    DevArr<GrownSet> d_grown;                 // sets of a growth (grow_htabs)
     DevArr<uint2> d_big;                      // long delta rows for the symbolic CTA pass
     // in the mirror: the state as last read
     Counters *h_cnt = nullptr;
@@ -971,15 +972,19 @@ struct Runner {
             }
     }
 
+    static constexpr uint64_t GROWN_TOGETHER = 1ull << 21;   // entries: 16 MB
+    // Room for eight times the need (the set is at most an eighth full
+    // afterwards): a fresh solve's sets grow through several iterations,
+    // and every growth costs a host round trip and a re-run of the commit
+    // (58.5 -> 51.4 ms for the first solve of the 200k alias graph, with
+    // the pool quadrupling instead of doubling).
+    static uint64_t grown_cap(uint64_t need) {
+        return next_pow2(std::max<uint64_t>(8 * need, 1024));
+    }
     void grow_htab(uint32_t s, uint64_t need) {
         cflr_ctx *c = cx[slot_ctx[s]];
         uint32_t x = s - base[slot_ctx[s]];
-        // room for eight times the need (the set is at most an eighth full
-        // afterwards): a fresh solve's sets grow through several iterations,
-        // and every growth costs a host round trip and a re-run of the commit
-        // (58.5 -> 51.4 ms for the first solve of the 200k alias graph, with
-        // the pool quadrupling instead of doubling)
-        uint64_t cap = next_pow2(std::max<uint64_t>(8 * need, 1024));
+        const uint64_t cap = grown_cap(need);
         unsigned long long *nt = (unsigned long long *)alloc_for(c, cap * 8);
         ck(cudaMemsetAsync(nt, 0xFF, cap * 8, st), "memset");
         uint2 *nv = c->hval[x] ? (uint2 *)alloc_for(c, cap * 8) : nullptr;
@@ -1002,6 +1007,98 @@ struct Runner {
         c->hcap[x] = cap;
         regrows++;
         regrow_kind[1]++;
+    }
+    // Larger tables for the listed slots {slot, pairs to hold}: all new tables
+    // are allocated, filled by two launches per part of the list (a part's
+    // tables stay in the L2 cache between the two), then put in place of the
+    // old ones.  Throws before anything is in place when one cannot be had.
+    void grow_htabs(const std::vector<std::pair<uint32_t, uint64_t>> &list) {
+        if (list.empty()) return;
+        struct Pending {                // freed on the way out unless put in place
+            Runner *r;
+            const std::vector<std::pair<uint32_t, uint64_t>> &list;
+            std::vector<GrownSet> sets;
+            ~Pending() {
+                for (size_t q = 0; q < sets.size(); q++) {
+                    cflr_ctx *c = r->cx[r->slot_ctx[list[q].first]];
+                    if (sets[q].new_tab) c->dfree(sets[q].new_tab, sets[q].new_cap * 8);
+                    if (sets[q].new_val) c->dfree(sets[q].new_val, sets[q].new_cap * 8);
+                }
+            }
+        } pend{this, list, {}};
+        std::vector<GrownSet> &sets = pend.sets;
+        sets.reserve(list.size() + 1);
+        bool other_stream = false;
+        for (const auto &e : list) {
+            cflr_ctx *c = cx[slot_ctx[e.first]];
+            const uint32_t x = e.first - base[slot_ctx[e.first]];
+            const uint64_t cap = grown_cap(e.second);
+            sets.push_back(GrownSet{});
+            GrownSet &g = sets.back();
+            g.old_tab = c->htab[x];
+            g.old_val = c->hval[x];
+            g.old_cap = c->hcap[x];
+            g.new_cap = cap;
+            g.new_tab = (unsigned long long *)alloc_for(c, cap * 8);
+            if (c->hval[x]) g.new_val = (uint2 *)alloc_for(c, cap * 8);
+            other_stream |= c->stream != st;
+        }
+        struct Part {
+            size_t at;                      // in table: `count` sets, then their chunk totals
+            uint32_t count;
+        };
+        constexpr uint64_t PART_BYTES = 32ull << 20;
+        std::vector<GrownSet> table;
+        std::vector<Part> parts;
+        GrownSet total{};
+        uint64_t bytes = 0;
+        for (const GrownSet &g : sets) {
+            const uint64_t b = g.new_cap * (g.new_val ? 16 : 8);
+            if (parts.empty() || bytes + b > PART_BYTES) {
+                if (!parts.empty()) table.push_back(total);
+                parts.push_back({table.size(), 0});
+                total = GrownSet{};
+                bytes = 0;
+            }
+            bytes += b;
+            parts.back().count++;
+            table.push_back(g);
+            for (int ph = 0; ph < 2; ph++) {
+                table.back().first[ph] = total.first[ph];
+                total.first[ph] += set_chunks(ph ? g.old_cap : g.new_cap, ph);
+            }
+        }
+        table.push_back(total);
+        d_grown.ensure(own, table.size());
+        ck(cudaMemcpyAsync(d_grown.p, table.data(), table.size() * sizeof(GrownSet),
+                           cudaMemcpyHostToDevice, st), "H2D");
+        prof.run(KID_REHASH, [&] {
+            for (const Part &p : parts) {
+                const GrownSet &end = table[p.at + p.count];
+                launch_rehash_many(d_grown.p + p.at, p.count, end.first[0], end.first[1],
+                                   &d_cnt.p->overflow, sms, st);
+            }
+        });
+        // an old table is freed on its context's stream: when that is the
+        // batch stream the free is ordered after the move and no wait is
+        // needed (the move reports through the loop status read next)
+        if (other_stream) sync("rehash");
+        for (size_t q = 0; q < sets.size(); q++) {
+            cflr_ctx *c = cx[slot_ctx[list[q].first]];
+            const uint32_t x = list[q].first - base[slot_ctx[list[q].first]];
+            GrownSet &g = sets[q];
+            own->k_bytes[KID_REHASH] += g.old_cap * 8 + list[q].second * 8;
+            if (c->hown[x]) c->dfree(c->htab[x], c->hcap[x] * 8);
+            c->hown[x] = 1;
+            if (c->hval[x]) c->dfree(c->hval[x], c->hcap[x] * 8);
+            c->htab[x] = g.new_tab;
+            c->hval[x] = g.new_val;
+            c->hcap[x] = g.new_cap;
+            g.new_tab = nullptr;
+            g.new_val = nullptr;
+            regrows++;
+            regrow_kind[1]++;
+        }
     }
 
     void grow_pool(size_t k, uint64_t top) {
@@ -1207,12 +1304,31 @@ struct Runner {
         const InstTab I = insttab();
         const WorkBufs W = work();
         if (st_bits & OVF_HASH) {                      // grow pair sets, then commit
+            std::vector<std::pair<uint32_t, uint64_t>> small;
             for (uint32_t s = 0; s < n_slots; s++) {
                 cflr_ctx *c = cx[slot_ctx[s]];
-                uint32_t x = s - base[slot_ctx[s]];
                 const uint64_t need = h_nnz[s] + h_cand[s];
-                if (2 * need > c->hcap[x]) grow_htab(s, need);
+                if (2 * need <= c->hcap[s - base[slot_ctx[s]]]) continue;
+                // Many small sets move together; one at a time under a budget
+                // and above 16 MB, where the fill of one set and its move
+                // outlast the launches (20k alias solve 14.8 ms one at a time,
+                // 15.1 together).
+                if (c->cfg.mem_budget_bytes || grown_cap(need) > GROWN_TOGETHER)
+                    grow_htab(s, need);
+                else
+                    small.push_back({s, need});
             }
+            bool together = small.size() > 1;
+            if (together) {
+                try {
+                    grow_htabs(small);
+                } catch (const Status &e) {       // no room for old and new at once
+                    if (e.code != CFLR_ENOMEM) throw;
+                    together = false;
+                }
+            }
+            if (!together)
+                for (const auto &e : small) grow_htab(e.first, e.second);
             upload_htabs();
             clear_overflow();
             launch_merge(S, I, W, 0, true, false, true, false);
