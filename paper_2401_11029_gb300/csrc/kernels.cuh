@@ -45,9 +45,9 @@ constexpr int N_BINS = 4;
 // Bin limits on a group's smem need (mask entries + products); a bin's table
 // holds twice its limit so the load factor stays <= 1/2.
 constexpr uint32_t BIN0_LIMIT = 128;    // warp per group, 256-slot table
-constexpr uint32_t BIN1_LIMIT = 1024;   // warp per group, 2048-slot table
+constexpr uint32_t BIN1_LIMIT = 1024;   // two warps per group, 2048-slot table
 constexpr uint32_t BIN2_LIMIT = 4096;   // CTA per group, 8192-slot table
-                                        // bin 3: CTA per group, n-bit bitmap
+                                        // bin 3: half a CTA per group, n-bit bitmap
 constexpr uint32_t PROBE_RATIO = 4;     // probe when mask_len > PROBE_RATIO*flops
 
 // Run-time schedule of the product kernels (picked by cflr_autotune).
