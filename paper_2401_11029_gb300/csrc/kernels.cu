@@ -283,9 +283,10 @@ __device__ __forceinline__ unsigned long long block_excl_scan256(unsigned long l
 // k_symbolic: groups of this iteration, binned by shared-memory need
 // ---------------------------------------------------------------------------
 
-// The kernels of the merge and the second work-list launch start while the one
-// before them ends (launch_after) and wait here, before their first access, for
-// everything it wrote; then the next one may start.
+// The kernels of the merge, the second work-list launch and those of the
+// terminal initialisation and the read-out start while the one before them ends
+// (launch_after) and wait here, before their first access, for everything it
+// wrote; then the next one may start.
 __device__ __forceinline__ void wait_before() {
     cudaGridDependencySynchronize();
     cudaTriggerProgrammaticLaunchCompletion();
@@ -2627,6 +2628,7 @@ __global__ void __launch_bounds__(256) k_init_edges(const uint32_t *src, const u
                                                     const uint32_t *term_off,
                                                     const uint32_t *term_slot,
                                                     uint32_t n_terms, WorkBufs W) {
+    wait_before();
     const int lane = threadIdx.x & 31;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x +
@@ -2652,6 +2654,7 @@ __global__ void __launch_bounds__(256) k_init_edges(const uint32_t *src, const u
 }
 
 __global__ void k_init_eps(uint32_t slot, uint32_t n, WorkBufs W) {
+    wait_before();
     const int lane = threadIdx.x & 31;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x +
@@ -2773,6 +2776,7 @@ __global__ void k_fill_u64(unsigned long long *p, unsigned long long count,
 constexpr uint32_t CLEAR_SEG = 2048;     // slots scanned at a time, 8 a thread
 
 __global__ void __launch_bounds__(256) k_clear_sets(SlotTab S, uint32_t n_slots) {
+    wait_before();
     __shared__ unsigned long long first[CLEAR_SEG + 1];   // first chunk of each slot
     __shared__ unsigned long long sh[16];
     const uint4 empty = make_uint4(EMPTY32, EMPTY32, EMPTY32, EMPTY32);
@@ -3163,6 +3167,7 @@ __device__ __forceinline__ uint32_t row_words(uint32_t n) { return (n + 31) / 32
 
 __global__ void __launch_bounds__(256) k_row_map(ExtractList L, const uint32_t *occ,
                                                  uint32_t occ_w, uint32_t *map) {
+    wait_before();
     const int lane = threadIdx.x & 31;
     const uint32_t words = row_words(L.n);
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
@@ -3239,6 +3244,7 @@ __device__ __forceinline__ uint32_t warp_row_len(const uint32_t *tl, uint32_t nt
 // longer ones by the warp.
 __global__ void __launch_bounds__(256) k_unit_lengths(ExtractList L,
                                                       unsigned long long *unit_len) {
+    wait_before();
     const int lane = threadIdx.x & 31;
     const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
     for (unsigned long long u = (unsigned long long)blockIdx.x * (blockDim.x >> 5) +
@@ -3282,6 +3288,7 @@ __global__ void __launch_bounds__(256) k_extract_units(ExtractList L,
                                                        uint4 *big, unsigned long long big_cap,
                                                        unsigned long long *cursor,
                                                        unsigned *err) {
+    cudaGridDependencySynchronize();
     __shared__ uint32_t sbuf[8][EXTRACT_WARP_MAX];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     uint32_t *s = sbuf[wib];
@@ -3428,6 +3435,7 @@ constexpr uint32_t SCAN_TILE = 1024;   // 256 threads x 4 elements
 template <typename T>
 __global__ void __launch_bounds__(256) k_scan_reduce(const T *in, unsigned long long n,
                                                      unsigned long long *bsum) {
+    wait_before();
     __shared__ unsigned long long sh[16];
     const unsigned long long base = (unsigned long long)blockIdx.x * SCAN_TILE + threadIdx.x * 4;
     unsigned long long v = 0;
@@ -3441,6 +3449,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(const T *in, unsigned long 
 
 __global__ void __launch_bounds__(256) k_scan_top(unsigned long long *bsum, uint32_t nb,
                                                   unsigned long long *grand) {
+    wait_before();
     __shared__ unsigned long long sh[16];
     unsigned long long carry = 0;
     for (uint32_t b0 = 0; b0 < nb; b0 += 256) {
@@ -3458,6 +3467,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_scan_down(const T *in, unsigned long long n,
                                                    const unsigned long long *bsum,
                                                    unsigned long long *out) {
+    wait_before();
     __shared__ unsigned long long sh[16];
     const unsigned long long base = (unsigned long long)blockIdx.x * SCAN_TILE + threadIdx.x * 4;
     T x[4];
@@ -3491,6 +3501,7 @@ constexpr unsigned long long SCAN_ONE = 8192;
 
 __global__ void __launch_bounds__(256) k_scan_one(unsigned long long *v, uint32_t n,
                                                   unsigned long long *grand) {
+    wait_before();
     __shared__ unsigned long long sh[16];
     unsigned long long carry = 0;
     for (uint32_t b0 = 0; b0 < n; b0 += SCAN_TILE) {
@@ -3512,18 +3523,39 @@ __global__ void __launch_bounds__(256) k_scan_one(unsigned long long *v, uint32_
     if (threadIdx.x == 0 && grand) *grand = carry;
 }
 
+// Launch a kernel of 256-thread CTAs that may start before the one ahead of it
+// in the stream has ended (it calls wait_before): the gaps between ten kernels
+// in a row are a large part of a small iteration (one-shot solve of the
+// 613-vertex alias graph 1.79 -> 1.72 ms, 100k value-flow pass 2.32 -> 2.27,
+// 64 batched Dyck-3 instances 16.1 -> 15.4, 200k alias unchanged), and of the
+// short launches of a reset and a read-out (the Dyck-3 batch 15.5 -> 15.0).
+template <class... Ps, class... As>
+static void launch_after(void (*k)(Ps...), int grid, size_t smem, cudaStream_t st, As... as) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, static_cast<Ps>(as)...);
+}
+
 void launch_exclusive_scan64(unsigned long long *in_out, unsigned long long n,
                              unsigned long long *bsum, unsigned long long *grand,
                              cudaStream_t st) {
     if (!n) return;
     if (n <= SCAN_ONE) {
-        k_scan_one<<<1, 256, 0, st>>>(in_out, (uint32_t)n, grand);
+        launch_after(k_scan_one, 1, 0, st, in_out, (uint32_t)n, grand);
         return;
     }
     const unsigned long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    k_scan_reduce<unsigned long long><<<(unsigned)nb, 256, 0, st>>>(in_out, n, bsum);
-    k_scan_top<<<1, 256, 0, st>>>(bsum, (uint32_t)nb, grand);
-    k_scan_down<unsigned long long><<<(unsigned)nb, 256, 0, st>>>(in_out, n, bsum, in_out);
+    launch_after(k_scan_reduce<unsigned long long>, (unsigned)nb, 0, st, in_out, n, bsum);
+    launch_after(k_scan_top, 1, 0, st, bsum, (uint32_t)nb, grand);
+    launch_after(k_scan_down<unsigned long long>, (unsigned)nb, 0, st, in_out, n, bsum, in_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -3583,26 +3615,6 @@ static void set_smem_attrs() {
                          (int)SMEM_BITMAP_MAX);
     cudaFuncSetAttribute(k_capacity_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)SMEM_BITMAP_MAX);
-}
-
-// Launch a kernel of 256-thread CTAs that may start before the one ahead of it
-// in the stream has ended (it calls wait_before): the gaps between ten kernels
-// in a row are a large part of a small iteration (one-shot solve of the
-// 613-vertex alias graph 1.79 -> 1.72 ms, 100k value-flow pass 2.32 -> 2.27,
-// 64 batched Dyck-3 instances 16.1 -> 15.4, 200k alias unchanged).
-template <class... Ps, class... As>
-static void launch_after(void (*k)(Ps...), int grid, size_t smem, cudaStream_t st, As... as) {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k, static_cast<Ps>(as)...);
 }
 
 void launch_symbolic(const SlotTab &S, const ProdTab &P, const WorkBufs &W, int prod_only,
@@ -3721,13 +3733,13 @@ void launch_init_edges(const uint32_t *src, const uint32_t *lab, const uint32_t 
                        const uint32_t *term_slot, uint32_t n_terms, const WorkBufs &W,
                        int sms, cudaStream_t st) {
     if (!n_edges) return;
-    k_init_edges<<<grid_for(n_edges, 256, sms, 8), 256, 0, st>>>(src, lab, dst, n_edges,
-                                                                  term_off, term_slot, n_terms, W);
+    launch_after(k_init_edges, grid_for(n_edges, 256, sms, 8), 0, st, src, lab, dst, n_edges,
+                 term_off, term_slot, n_terms, W);
 }
 
 void launch_init_eps(uint32_t slot, uint32_t n, const WorkBufs &W, int sms, cudaStream_t st) {
     if (!n) return;
-    k_init_eps<<<grid_for(n, 256, sms, 8), 256, 0, st>>>(slot, n, W);
+    launch_after(k_init_eps, grid_for(n, 256, sms, 8), 0, st, slot, n, W);
 }
 
 void launch_rehash(const unsigned long long *old_tab, const uint2 *old_val,
@@ -3830,7 +3842,7 @@ void launch_extract_count(const ExtractList &L, unsigned long long *units,
                           cudaStream_t st) {
     const unsigned long long nu = L.units;
     if (!nu || !L.n) return;
-    k_unit_lengths<<<grid_for(nu, 8, sms, 8), 256, 0, st>>>(L, units);
+    launch_after(k_unit_lengths, grid_for(nu, 8, sms, 8), 0, st, L, units);
     launch_exclusive_scan64(units, nu, bsum, total, st);
 }
 
@@ -3847,10 +3859,11 @@ void launch_extract_write(const ExtractList &L, uint32_t *out_src, uint32_t *out
     const unsigned long long nu = L.u_end > L.u_begin ? L.u_end - L.u_begin : 0;
     if (!nu || !L.n) return;
     set_smem_attrs();
-    k_extract_units<<<grid_for(nu, 8, sms, 8), 256, 0, st>>>(L, units, out_src, out_dst, big,
-                                                             big_cap, cursor, err);
+    launch_after(k_extract_units, grid_for(nu, 8, sms, 8), 0, st, L, units, out_src, out_dst, big,
+                 big_cap, cursor, err);
     const size_t bm_bytes = (size_t)((L.n + 31) / 32) * 4;
     const bool sm = bm_bytes <= SMEM_BITMAP_MAX;
+    // (not early: its CTAs would hold their bitmaps while the short rows are written)
     k_extract_units_big<<<sms * 4, 256, sm ? bm_bytes : 0, st>>>(L, out_src, out_dst, big,
                                                                  big_cap, cursor, bitmap,
                                                                  sm ? 1 : 0);
