@@ -1164,7 +1164,7 @@ struct Runner {
         }
     }
     // Commit and union, from the dedupe (stage 0, or -1 for the terminal
-    // initialisation), the capacity pass (stage 1) or the scatter (stage 2), then the end of the iteration.
+    // initialisation) or the capacity pass (stage 1) to the end of the iteration.
     void launch_merge(const SlotTab &S, const InstTab &I, const WorkBufs &W, int stage,
                       bool count_iteration, bool in_graph, bool timed, bool check) {
         auto run = [&](int kid, auto f) { if (timed) prof.run(kid, f); else f(); };
