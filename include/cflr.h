@@ -311,8 +311,11 @@ int cflr_reset(cflr_ctx *c);
 
 /* Solve n independent contexts together: each closure iteration runs the
  * products of all unfinished contexts in one launch sequence.  Every
- * context must hold a loaded graph and use the same device and stream as
- * ctxs[0].  stats (nullable) is an array of n.  Results are identical to
+ * context must hold a loaded graph and use the same device as ctxs[0].  The
+ * work runs on ctxs[0]'s stream; the contexts may have streams of their own
+ * (private ones, or the caller's), and what a load or a reset left queued on
+ * them is ordered before the batch.  stats (nullable) is an array of n.
+ * Results are identical to
  * solving each context alone.  The iteration limit and the work buffers are
  * those of ctxs[0], which may be a context whose solve has already finished
  * (it then only lends its buffers): with max_iterations = 1 every call

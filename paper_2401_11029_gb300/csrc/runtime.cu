@@ -136,6 +136,9 @@ struct cflr_ctx {
     std::vector<uint64_t> nnz;
     uint2 *touched = nullptr;           // rows with dnew > 0 (local slot ids)
     uint64_t touched_n = 0;
+    // after the last copy into `touched` that the host did not wait for (on
+    // `stream`): a batch led from another stream waits for it
+    cudaEvent_t touched_ev = nullptr;
     uint64_t touched_cap = 0;
     uint32_t iterations = 0;
     // the graph as loaded (device copies, kept for cflr_reset)
@@ -1392,7 +1395,9 @@ struct Runner {
     }
 
     // Pending delta rows of each context into the "in" touched list (bind set
-    // their number).
+    // their number).  A load or a reset returns with the copy of its context's
+    // rows still queued on the context's stream; everything else there the
+    // host has waited for.
     void import_touched() {
         uint64_t total = 0;
         for (auto *c : cx) total += c->touched_n;
@@ -1400,8 +1405,11 @@ struct Runner {
         uint64_t at = 0;
         for (size_t k = 0; k < cx.size(); k++) {
             cflr_ctx *c = cx[k];
-            if (c->touched_n)
+            if (c->touched_n) {
+                if (c->stream != st && c->touched_ev)
+                    ck(cudaStreamWaitEvent(st, c->touched_ev, 0), "touched event");
                 launch_remap_touched(c->touched, c->touched_n, base[k], d_touched[0].p + at, st);
+            }
             ck(cudaGetLastError(), "remap");
             at += c->touched_n;
         }
@@ -1430,7 +1438,15 @@ struct Runner {
             c->touched_n = n_in;
             ck(cudaMemcpyAsync(c->touched, d_touched[par].p, n_in * sizeof(uint2),
                                cudaMemcpyDeviceToDevice, st), "D2D touched");
-            if (c->stream != st) sync("export copy");   // (else ordered with what follows)
+            if (c->stream != st) {
+                sync("export copy");
+            } else {        // no wait here: what follows on this stream is ordered, and
+                            // import_touched orders another stream's read
+                if (!c->touched_ev)
+                    ck(cudaEventCreateWithFlags(&c->touched_ev, cudaEventDisableTiming),
+                       "cudaEventCreate");
+                ck(cudaEventRecord(c->touched_ev, st), "touched event");
+            }
             return;
         }
         d_inst_cnt.ensure(own, ni);
@@ -2702,6 +2718,7 @@ void cflr_destroy(cflr_ctx *c) {
     c->runner = nullptr;
     c->free_graph();
     if (c->stream) cudaStreamSynchronize(c->stream);   // the frees above are stream-ordered
+    if (c->touched_ev) cudaEventDestroy(c->touched_ev);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }

@@ -104,7 +104,8 @@ class Server:
 
     def _admit(self, graph):
         # a private stream: the load overlaps the tick running on the
-        # leader's stream (the load ends synchronised with the host)
+        # leader's stream (what it leaves queued there is ordered before the
+        # tick that the context first takes part in)
         ctx = cflr.cflr_create(device=self.device, form=self.form, size_hint=self.size_hint)
         cflr.cflr_load_grammar(ctx, self.text)
         ids = self._label_ids(ctx, graph.labels)
