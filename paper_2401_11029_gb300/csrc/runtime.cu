@@ -2247,6 +2247,16 @@ struct CopyLane {
     }
 };
 
+// A call that ends by an exception waits for what it has queued: pinned memory
+// that outlives it is not written or freed while a copy of it is under way.
+struct WaitOnFailure {
+    cudaStream_t st;
+    bool armed = true;
+    ~WaitOnFailure() {
+        if (armed) cudaStreamSynchronize(st);
+    }
+};
+
 // Write the pairs of the listed non-terminals (nts[0..count), output
 // positions offsets[0..count]) one after another, each non-terminal's
 // sorted by (src, dst): into the device arrays ws/wd, or into the host
@@ -2275,6 +2285,7 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
     for (uint64_t p : pairs) total += p;
     // the call's tables, in one copy to the device: cursors, error flag and
     // total (four words, zero), first units, listed ids, rows per unit
+    WaitOnFailure wait{st};
     PinnedBlock &pin = runner_of(c).kit->readout;
     const size_t tab_n = 32 + 8 * ((size_t)E + 1) + 8 * (size_t)E;
     pin.ensure(tab_n);
@@ -2347,6 +2358,7 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
                              err, c->sms, st);
         ck(cudaGetLastError(), "extract");
         check();
+        wait.armed = false;
         return;
     }
     // ranges of units that fit a staging buffer (a unit larger than that
@@ -2395,6 +2407,7 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
     }
     ck(cudaStreamSynchronize(lane.s), "sync copy");
     check();
+    wait.armed = false;
 }
 
 int get_pairs_common(cflr_ctx *c, uint32_t nonterminal, uint32_t *src, uint32_t *dst,

@@ -403,8 +403,50 @@ void batch_across_streams() {
     expect(cflr_reset(a.c) == CFLR_OK && batch({lead.c, a.c}) == CFLR_OK, "one of a batch");
 }
 
+cudaStream_t new_stream() {
+    cudaStream_t s;
+    cudaStreamCreateWithFlags(&s, 0);
+    return s;
+}
+// fails the k-th device allocation from now on (k = 1, 2, ...)
+std::function<bool(size_t)> nth(uint64_t k) {
+    return [k](size_t) mutable { return k && --k == 0; };
+}
+
+// Read-outs in which each device allocation in turn fails: the call's tables
+// are copied from memory that the next call writes, so nothing may be pending
+// on return.
+void failed_readouts() {
+    const uint32_t ids[2] = {0, 1};
+    for (int host = 0; host < 2; host++) {
+        int failed = 0, rc = CFLR_ENOMEM;
+        for (uint64_t k = 1; rc != CFLR_OK && k < 50; k++) {
+            const cudaStream_t st = new_stream();
+            Context x([&](cflr_config &c) { c.stream = st; });
+            expect(x.load() == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "solve");
+            std::vector<uint32_t> s(2 * g_pairs), d(2 * g_pairs);
+            // (stands for device arrays too: no kernel writes them here)
+            uint64_t off[3];
+            auto read = [&]() {
+                return host ? cflr_get_pairs_many(x.c, 2, ids, s.data(), d.data(), s.size(), off)
+                            : cflr_get_pairs_device_many(x.c, 2, ids, s.data(), d.data(), s.size(),
+                                                         off);
+            };
+            g_fail_alloc = nth(k);
+            rc = read();
+            g_fail_alloc = nullptr;
+            failed += rc == CFLR_ENOMEM;
+            expect(rc == CFLR_OK || rc == CFLR_ENOMEM, "read-out: code");
+            expect(idle(st), "read-out: work pending after the call");
+            expect(read() == CFLR_OK, "read-out after a failed one");
+        }
+        expect(rc == CFLR_OK && failed >= 4, "read-out: allocations reached");
+    }
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
     {"batch_across_streams", batch_across_streams},
+    {"failed_readouts", failed_readouts},
 };
 
 }  // namespace
