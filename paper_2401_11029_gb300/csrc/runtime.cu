@@ -526,7 +526,8 @@ struct Runner {
     cudaGraphConditionalHandle handle = 0;
     GraphKey graph_key{};              // what `gexec` was captured with
     RunnerKit *kit = nullptr;
-    bool kit_broken = false;           // a capture on its streams failed
+    bool kit_broken = false;           // a launch or capture on its streams failed
+    bool capturing = false;            // the launches go into a graph
 
     explicit Runner(cflr_ctx *owner) : own(owner), st(owner->stream), sms(owner->sms) {
         prof.owner = own;
@@ -1153,17 +1154,29 @@ struct Runner {
             // leave.  The heaviest kind of group (bin 3) starts first.  (200k
             // alias solve 53.5 -> 48.9 ms, 500k points-to 108 -> 98.5, Dyck-1
             // of 1000 vertices 2.1 -> 1.7, with two launches less a turn.)
-            ck(cudaEventRecord(kit->fork, st), "fork");
-            for (int b = N_BINS - 1; b >= 0; b--) {
-                const int q = b - 1;          // bin 0 stays on the solve stream
-                cudaStream_t on = b ? kit->s[q] : st;
-                if (b) ck(cudaStreamWaitEvent(on, kit->fork, 0), "fork");
-                launch_spgemm(b, S, P, W, max_n, tuning(), sms, on);
-                ck(cudaGetLastError(), kKernelNames[KID_BIN0 + b]);
-                if (b) ck(cudaEventRecord(kit->join[q], on), "join");
+            try {
+                ck(cudaEventRecord(kit->fork, st), "fork");
+                for (int b = N_BINS - 1; b >= 0; b--) {
+                    const int q = b - 1;          // bin 0 stays on the solve stream
+                    cudaStream_t on = b ? kit->s[q] : st;
+                    if (b) ck(cudaStreamWaitEvent(on, kit->fork, 0), "fork");
+                    launch_spgemm(b, S, P, W, max_n, tuning(), sms, on);
+                    ck(cudaGetLastError(), kKernelNames[KID_BIN0 + b]);
+                    if (b) ck(cudaEventRecord(kit->join[q], on), "join");
+                }
+                for (int q = 0; q < N_BINS - 1; q++)
+                    ck(cudaStreamWaitEvent(st, kit->join[q], 0), "join");
+            } catch (...) {
+                // what runs on the side streams is not joined: wait for it
+                // here (a capture has nothing running, and must not be waited
+                // for), and let no other runner have the streams
+                kit_broken = true;
+                if (!capturing) {
+                    for (cudaStream_t x : kit->s) cudaStreamSynchronize(x);
+                    cudaStreamSynchronize(st);
+                }
+                throw;
             }
-            for (int q = 0; q < N_BINS - 1; q++)
-                ck(cudaStreamWaitEvent(st, kit->join[q], 0), "join");
         }
     }
     // Commit and union, from the dedupe (stage 0, or -1 for the terminal
@@ -1247,14 +1260,17 @@ struct Runner {
                                          cudaStreamCaptureModeThreadLocal),
            "cudaStreamBeginCaptureToGraph");
         cudaGraph_t captured = nullptr;
+        capturing = true;
         try {
             launch_iteration(true, false);
         } catch (...) {
             // end the capture; side streams caught in it go to nobody else
+            capturing = false;
             cudaStreamEndCapture(st, &captured);
             kit_broken = true;
             throw;
         }
+        capturing = false;
         ck(cudaStreamEndCapture(st, &captured), "cudaStreamEndCapture");
         ck(cudaGraphInstantiate(&gexec, graph, 0), "cudaGraphInstantiate");
         graph_key = current_key();

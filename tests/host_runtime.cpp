@@ -61,6 +61,9 @@ uint64_t g_rows = 1000, g_pairs = 10;           // of an initialisation
 uint64_t g_maps = 0;                            // launches of the row map
 std::function<bool(size_t)> g_fail_alloc;       // device allocation of so many bytes
 std::string g_fail_launch;                      // name of the launch that fails next
+bool g_fail_captured = false;                   // ... when it is captured into a graph
+uint32_t g_iters = 1;                           // iterations of a closure
+bool g_capturing = false;
 cudaError_t g_last = cudaSuccess;
 
 void bad(const std::string &what) {
@@ -98,7 +101,7 @@ Block *block_of(const void *p) {
 }
 // work `m` on stream st uses [p, p + n)
 void use(const char *what, const void *p, size_t n, cudaStream_t st, Mark m, bool writes) {
-    if (!n) return;
+    if (!n || g_capturing) return;
     Block *b = block_of(p);
     if (!b) {
         if (p == nullptr || writes) bad(std::string(what) + ": not an allocation");
@@ -118,8 +121,8 @@ void use(const char *what, const void *p, size_t n, cudaStream_t st, Mark m, boo
     b->uses.push_back(m);
 }
 void launch(const char *name, cudaStream_t st) {
-    enqueue(st);
-    if (g_fail_launch == name) {
+    if (!g_capturing) enqueue(st);
+    if (g_fail_launch == name && g_fail_captured == g_capturing) {
         g_fail_launch.clear();
         g_last = cudaErrorLaunchOutOfResources;
     }
@@ -198,9 +201,13 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {
     g_streams[of(s)->id] = nullptr;
     return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { return merge(g_host, of(s)->seen), cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    expect(!g_capturing, "a wait inside a capture");
+    return merge(g_host, of(s)->seen), cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
-    return merge(of(s)->seen, ((Event *)e)->at), cudaSuccess;
+    if (!g_capturing) merge(of(s)->seen, ((Event *)e)->at);
+    return cudaSuccess;
 }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) {
     return *e = (cudaEvent_t) new Event(), cudaSuccess;
@@ -208,6 +215,7 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) {
 cudaError_t cudaEventCreate(cudaEvent_t *e) { return cudaEventCreateWithFlags(e, 0); }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+    if (g_capturing) return cudaSuccess;
     enqueue(s);
     return ((Event *)e)->at = of(s)->seen, cudaSuccess;
 }
@@ -230,6 +238,26 @@ cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t st) {
     use("memset", p, n, st, enqueue(st), true);
     std::memset(p, v, n);
     return cudaSuccess;
+}
+// (a graph is captured but never launched here)
+cudaError_t cudaGraphCreate(cudaGraph_t *g, unsigned) { return *g = (cudaGraph_t)1, cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphConditionalHandleCreate(cudaGraphConditionalHandle *h, cudaGraph_t, unsigned,
+                                             unsigned) {
+    return *h = 1, cudaSuccess;
+}
+cudaError_t cudaGraphAddNode(cudaGraphNode_t *, cudaGraph_t, const cudaGraphNode_t *,
+                             const cudaGraphEdgeData *, size_t, cudaGraphNodeParams *p) {
+    static cudaGraph_t body = (cudaGraph_t)2;
+    return p->conditional.phGraph_out = &body, cudaSuccess;
+}
+cudaError_t cudaStreamBeginCaptureToGraph(cudaStream_t, cudaGraph_t, const cudaGraphNode_t *,
+                                          const cudaGraphEdgeData *, size_t,
+                                          cudaStreamCaptureMode) {
+    return g_capturing = true, cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) {
+    return g_capturing = false, cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void **, const void *) { return cudaErrorNotSupported; }
 
@@ -279,8 +307,10 @@ void launch_iter_end(const SlotTab &S, const InstTab &I, const WorkBufs &W, Loop
                      uint32_t n_slots, uint32_t n_inst, bool count, cudaGraphConditionalHandle,
                      bool, cudaStream_t st) {
     launch("iter_end", st);
+    if (g_capturing) return;
     const int par = *W.parity;
-    const uint64_t rows = count ? 0 : std::min<uint64_t>(g_rows, W.touched_cap);
+    const uint64_t rows =
+        count && ctl->iter + 1 >= g_iters ? 0 : std::min<uint64_t>(g_rows, W.touched_cap);
     W.touched_n[par] = 0;
     W.touched_n[par ^ 1] = rows;
     for (uint64_t q = 0; q < rows; q++) W.touched[par ^ 1][q] = make_uint2(0, 0);
@@ -444,7 +474,40 @@ void failed_readouts() {
     }
 }
 
+// A launch that fails while the product bins run on several streams, or while
+// they are captured: nothing may be running when the call returns, and the
+// streams do not go to another context.
+void failed_products() {
+    for (int captured = 0; captured < 2; captured++) {
+        for (const char *at : {"bin3", "bin2", "bin1", "bin0"}) {
+            const std::string what = std::string(at) + (captured ? " (captured)" : "");
+            const cudaStream_t st = new_stream();
+            const size_t first = g_streams.size();
+            {
+                Context x([&](cflr_config &c) {
+                    c.stream = st;
+                    c.form = CFLR_FORM_GRAPH;
+                });
+                expect(x.load() == CFLR_OK, "load");
+                expect(g_streams.size() > first, "streams of its own");
+                g_iters = 3;                    // the second iteration is captured
+                g_fail_launch = at;
+                g_fail_captured = captured;
+                expect(cflr_solve(x.c, nullptr) == CFLR_ECUDA, what + ": code");
+                expect(g_fail_launch.empty() && !g_capturing, what + ": launch reached");
+                g_fail_captured = false;
+                g_iters = 1;
+                for (Stream *s : g_streams)
+                    if (s) expect(idle((cudaStream_t)s), what + ": work pending");
+            }
+            for (size_t k = first; k < g_streams.size(); k++)
+                expect(!g_streams[k], what + ": a stream is kept for another context");
+        }
+    }
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"failed_products", failed_products},
     {"batch_across_streams", batch_across_streams},
     {"failed_readouts", failed_readouts},
 };

@@ -31,7 +31,8 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["batch_across_streams", "failed_readouts"])
+@pytest.mark.parametrize("scenario", ["batch_across_streams", "failed_readouts",
+                                      "failed_products"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout[-4000:] + r.stderr[-2000:]
