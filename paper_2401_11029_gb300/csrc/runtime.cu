@@ -343,8 +343,8 @@ struct DevArr {           // device array owned by a context's accounting
     void alloc(cflr_ctx *owner, size_t count) {
         release();
         o = owner;
-        n = count;
         p = (T *)o->dalloc(std::max<size_t>(count, 1) * sizeof(T));
+        n = count;            // (stays 0 when the allocation throws)
     }
     void release() {
         if (p) o->dfree(p, std::max<size_t>(n, 1) * sizeof(T));
@@ -924,11 +924,12 @@ struct Runner {
     void size_cand(uint64_t cap) {
         cap = std::max<uint64_t>(cap, min_cap(1 << 16));
         if (cap <= cand_cap) return;
-        cand_cap = cap;
+        cand_cap = 0;         // a capacity counts once all its arrays are held
         d_cand_key.alloc(own, cap);
         d_cand_slot.alloc(own, cap);
         if (wit) d_cand_wit.alloc(own, cap);
         d_cand_pos.alloc(own, cap);
+        cand_cap = cap;
     }
     // Both touched lists; the list touched[parity] keeps its rows.  Each must
     // hold two rows per new pair (row and column form).
@@ -947,17 +948,19 @@ struct Runner {
         std::swap(d_touched[pin].n, keep.n);
         d_touched[pin].o = own;
         keep.release();
+        touched_cap = 0;
         d_touched[pin ^ 1].alloc(own, cap);
-        touched_cap = cap;
         // a listed row has more than 64 delta entries, and the deltas of
         // one iteration hold at most touched_cap entries
         d_big.ensure(own, cap / 64 + 1024);
+        touched_cap = cap;
     }
     void size_groups(int b, uint64_t cap) {
         cap = std::max<uint64_t>(cap, min_cap(1 << 14));
         if (cap <= group_cap[b]) return;
-        group_cap[b] = cap;
+        group_cap[b] = 0;
         d_groups[b].alloc(own, cap);
+        group_cap[b] = cap;
     }
     void init_buffers(uint64_t cand_hint, uint64_t touched_in) {
         const uint64_t ic = own->cfg.initial_capacity;

@@ -63,6 +63,7 @@ std::function<bool(size_t)> g_fail_alloc;       // device allocation of so many 
 std::string g_fail_launch;                      // name of the launch that fails next
 bool g_fail_captured = false;                   // ... when it is captured into a graph
 uint32_t g_iters = 1;                           // iterations of a closure
+unsigned g_overflow = 0;                        // OVF_* bits that stop the next iteration
 bool g_capturing = false;
 cudaError_t g_last = cudaSuccess;
 
@@ -308,6 +309,13 @@ void launch_iter_end(const SlotTab &S, const InstTab &I, const WorkBufs &W, Loop
                      bool, cudaStream_t st) {
     launch("iter_end", st);
     if (g_capturing) return;
+    if (count && g_overflow) {
+        ctl->status = g_overflow;
+        g_overflow = 0;
+        W.cnt->cand = W.cand_cap + 1;
+        for (int b = 0; b < N_BINS; b++) W.cnt->groups[b] = W.group_cap[b] + 1;
+        return;
+    }
     const int par = *W.parity;
     const uint64_t rows =
         count && ctl->iter + 1 >= g_iters ? 0 : std::min<uint64_t>(g_rows, W.touched_cap);
@@ -506,7 +514,64 @@ void failed_products() {
     }
 }
 
+// A context stays usable after CFLR_ENOMEM, whichever allocation of a load or of
+// a solve whose buffers overflow it was: the next graph's kernels get arrays
+// that hold what they are said to (the launches look at each).
+void failed_buffers() {
+    for (int witness = 0; witness < 2; witness++) {
+        for (int solving = 0; solving < 2; solving++) {
+            int failed = 0, rc = CFLR_ENOMEM;
+            for (uint64_t k = 1; rc != CFLR_OK && k < 100; k++) {
+                Context x([&](cflr_config &c) { c.witness = witness; });
+                expect(x.load() == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "solve");
+                if (solving) {
+                    expect(x.load() == CFLR_OK, "load");
+                    g_overflow = OVF_CAND | OVF_GROUPS;
+                }
+                g_fail_alloc = nth(k);
+                // (100,000 edges: more initial pairs than the first buffers hold)
+                rc = solving ? cflr_solve(x.c, nullptr) : x.load(5000, 100000);
+                g_fail_alloc = nullptr;
+                g_overflow = 0;
+                failed += rc == CFLR_ENOMEM;
+                expect(rc == CFLR_OK || rc == CFLR_ENOMEM, "code");
+                if (rc != CFLR_OK)
+                    expect(cflr_solve(x.c, nullptr) == CFLR_ESTATE, "no graph after a failure");
+                for (int more = 0; more < 2; more++)
+                    expect(x.load() == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "next graph");
+            }
+            expect(rc == CFLR_OK && failed >= 6, "allocations reached");
+        }
+    }
+}
+
+// A batch larger than the leader's tables hold, whose allocations fail in turn:
+// the leader's next solve by itself has its production tables.
+void failed_batch_tables() {
+    int failed = 0, rc = CFLR_ENOMEM;
+    for (uint64_t k = 1; rc != CFLR_OK && k < 50; k++) {
+        Context lead;
+        std::vector<Context> more(8);
+        std::vector<cflr_ctx *> cx(1, lead.c);
+        expect(lead.load() == CFLR_OK, "load");
+        for (auto &x : more) {
+            expect(x.load() == CFLR_OK, "load");
+            cx.push_back(x.c);
+        }
+        g_fail_alloc = nth(k);
+        rc = batch(cx);
+        g_fail_alloc = nullptr;
+        failed += rc == CFLR_ENOMEM;
+        expect(rc == CFLR_OK || rc == CFLR_ENOMEM, "code");
+        for (cflr_ctx *c : cx) expect(rc == CFLR_OK || cflr_reset(c) == CFLR_ESTATE, "dropped");
+        expect(lead.load() == CFLR_OK && cflr_solve(lead.c, nullptr) == CFLR_OK, "leader again");
+    }
+    expect(rc == CFLR_OK && failed >= 1, "allocations reached");
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"failed_batch_tables", failed_batch_tables},
+    {"failed_buffers", failed_buffers},
     {"failed_products", failed_products},
     {"batch_across_streams", batch_across_streams},
     {"failed_readouts", failed_readouts},
