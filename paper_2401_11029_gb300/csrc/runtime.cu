@@ -2283,10 +2283,10 @@ struct WaitOnFailure {
 // For the host, the units' first positions are read back after the count,
 // the units are cut into ranges that fit a buffer, and each range is written
 // into one buffer while the other is copied out on a second stream.
-// Checks the extracted count against the pair sets' counts.
-void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64_t *offsets,
-                  uint32_t *ws, uint32_t *wd, uint32_t *hs, uint32_t *hd) {
-    Range range("cflr: extraction");
+// Checks the extracted count against the pair sets' counts.  with_map: over a
+// map of the non-empty rows.
+void extract_list(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64_t *offsets,
+                  uint32_t *ws, uint32_t *wd, uint32_t *hs, uint32_t *hd, bool with_map) {
     constexpr uint64_t STAGE = 1ull << 24;
     cudaStream_t st = c->stream;
     const uint32_t n = c->n;
@@ -2347,7 +2347,8 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
             if (!keep) c->drop(c->x_map, c->x_map_n);
         }
     } map_guard{c, budget == 0};
-    if (!budget || c->bytes_now + 4 * map_n + 17 * total + (1 << 16) <= budget) {
+    if (with_map &&
+        (!budget || c->bytes_now + 4 * map_n + 17 * total + (1 << 16) <= budget)) {
         c->scratch(c->x_map, c->x_map_n, map_n);
         launch_row_map(L, c->occ, c->occ_w, c->x_map, c->sms, st);
         ck(cudaGetLastError(), "row map");
@@ -2427,6 +2428,20 @@ void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
     ck(cudaStreamSynchronize(lane.s), "sync copy");
     check();
     wait.armed = false;
+}
+
+// The same on a device that has no room for the map, or none beside it: again
+// without one.
+void extract_many(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64_t *offsets,
+                  uint32_t *ws, uint32_t *wd, uint32_t *hs, uint32_t *hd) {
+    Range range("cflr: extraction");
+    try {
+        extract_list(c, count, nts, offsets, ws, wd, hs, hd, true);
+    } catch (const Status &s) {
+        if (s.code != CFLR_ENOMEM) throw;
+        c->drop(c->x_map, c->x_map_n);
+        extract_list(c, count, nts, offsets, ws, wd, hs, hd, false);
+    }
 }
 
 int get_pairs_common(cflr_ctx *c, uint32_t nonterminal, uint32_t *src, uint32_t *dst,

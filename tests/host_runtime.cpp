@@ -446,12 +446,16 @@ cudaStream_t new_stream() {
     cudaStreamCreateWithFlags(&s, 0);
     return s;
 }
-// fails the k-th device allocation from now on (k = 1, 2, ...)
+// fails the k-th device allocation from now on (k = 1, 2, ...), or that and all
+// later ones
 std::function<bool(size_t)> nth(uint64_t k) {
     return [k](size_t) mutable { return k && --k == 0; };
 }
+std::function<bool(size_t)> from(uint64_t k) {
+    return [k](size_t) mutable { return k <= 1 || (--k, false); };
+}
 
-// Read-outs in which each device allocation in turn fails: the call's tables
+// Read-outs that run out of memory at each allocation in turn: the call's tables
 // are copied from memory that the next call writes, so nothing may be pending
 // on return.
 void failed_readouts() {
@@ -470,7 +474,7 @@ void failed_readouts() {
                             : cflr_get_pairs_device_many(x.c, 2, ids, s.data(), d.data(), s.size(),
                                                          off);
             };
-            g_fail_alloc = nth(k);
+            g_fail_alloc = from(k);
             rc = read();
             g_fail_alloc = nullptr;
             failed += rc == CFLR_ENOMEM;
@@ -569,7 +573,38 @@ void failed_batch_tables() {
     expect(rc == CFLR_OK && failed >= 1, "allocations reached");
 }
 
+// A device without room for the map of non-empty rows, which a read-out can do
+// without, or without room for what comes after it beside it.
+void readout_without_map() {
+    const uint32_t n = 10000, ids[2] = {0, 1};
+    const size_t map = 2 * ((n + 31) / 32) * 4;
+    for (int host = 0; host < 2; host++) {
+        for (int beside = 0; beside < 2; beside++) {
+            const cudaStream_t st = new_stream();
+            Context x([&](cflr_config &c) { c.stream = st; });
+            expect(x.load(n, 300) == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "solve");
+            std::vector<uint32_t> s(2 * g_pairs), d(2 * g_pairs);
+            uint64_t off[3];
+            int failed = 0;
+            g_fail_alloc = [&](size_t bytes) {
+                bool fail = bytes == map && !beside;
+                if (beside)                       // whatever it is, while the map is there
+                    for (auto &b : g_blocks) fail |= b.second.n == map && b.second.live;
+                failed += fail;
+                return fail;
+            };
+            expect((host ? cflr_get_pairs_many(x.c, 2, ids, s.data(), d.data(), s.size(), off)
+                         : cflr_get_pairs_device_many(x.c, 2, ids, s.data(), d.data(), s.size(),
+                                                      off)) == CFLR_OK,
+                   "read-out without room for the map");
+            g_fail_alloc = nullptr;
+            expect(failed == 1, "one allocation failed");
+        }
+    }
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"readout_without_map", readout_without_map},
     {"failed_batch_tables", failed_batch_tables},
     {"failed_buffers", failed_buffers},
     {"failed_products", failed_products},
