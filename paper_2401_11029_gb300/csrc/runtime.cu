@@ -160,7 +160,7 @@ struct cflr_ctx {
     uint4 *x_bigl = nullptr;
     size_t x_tab_n = 0, x_bm_n = 0, x_map_n = 0, x_unit_n = 0, x_bsum_n = 0, x_bigl_n = 0;
     uint32_t *x_src = nullptr, *x_dst = nullptr;
-    uint64_t x_out_cap = 0;
+    size_t x_src_n = 0, x_dst_n = 0;
     // accounting
     uint64_t bytes_now = 0, bytes_peak = 0;
     cflr_stats last{};
@@ -230,10 +230,8 @@ struct cflr_ctx {
     }
     // device staging of cflr_get_pairs's host output
     void free_extract_out() {
-        if (x_src) dfree(x_src, x_out_cap * 4);
-        if (x_dst) dfree(x_dst, x_out_cap * 4);
-        x_src = x_dst = nullptr;
-        x_out_cap = 0;
+        drop(x_src, x_src_n);
+        drop(x_dst, x_dst_n);
     }
 
     void free_graph() {
@@ -2396,11 +2394,10 @@ void extract_list(cflr_ctx *c, uint32_t count, const uint32_t *nts, const uint64
     for (size_t r = 0; r + 1 < cut.size(); r++)
         cap = std::max<uint64_t>(cap, uoff[cut[r + 1]] - uoff[cut[r]]);
     cap = std::max<uint64_t>(cap, 1);
-    if (c->x_out_cap < 2 * cap) {
+    if (c->x_src_n < 2 * cap || c->x_dst_n < 2 * cap) {
         c->free_extract_out();
-        c->x_src = (uint32_t *)c->dalloc(2 * cap * 4);
-        c->x_dst = (uint32_t *)c->dalloc(2 * cap * 4);
-        c->x_out_cap = 2 * cap;
+        c->scratch(c->x_src, c->x_src_n, 2 * cap);
+        c->scratch(c->x_dst, c->x_dst_n, 2 * cap);
     }
     c->scratch(c->x_bigl, c->x_bigl_n, cap / 1024 + 1);
     CopyLane lane;

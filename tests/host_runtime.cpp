@@ -603,7 +603,29 @@ void readout_without_map() {
     }
 }
 
+// Read-outs under a memory budget that fail again and again leave what the
+// context is said to hold as it was.
+void budget_after_failed_readouts() {
+    Context x([](cflr_config &c) { c.mem_budget_bytes = 64 << 20; });
+    const uint64_t few = g_pairs;
+    g_pairs = 100000;
+    expect(x.load(1000, 3000) == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "solve");
+    std::vector<uint32_t> s(g_pairs), d(g_pairs);
+    uint64_t got = 0;
+    auto read = [&]() { return cflr_get_pairs(x.c, 0, s.data(), d.data(), s.size(), &got); };
+    const size_t staging = 2 * g_pairs * 4;       // two buffers of sources, two of targets
+    for (int turn = 0; turn < 200; turn++) {
+        int seen = 0;                             // the second array of the pair fails
+        g_fail_alloc = [&](size_t bytes) { return bytes == staging && ++seen % 2 == 0; };
+        expect(read() == CFLR_ENOMEM && seen >= 2, "read-out without room");
+        g_fail_alloc = nullptr;
+    }
+    expect(read() == CFLR_OK && got == g_pairs, "read-out after failed ones");
+    g_pairs = few;
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"budget_after_failed_readouts", budget_after_failed_readouts},
     {"readout_without_map", readout_without_map},
     {"failed_batch_tables", failed_batch_tables},
     {"failed_buffers", failed_buffers},
