@@ -991,8 +991,14 @@ struct Runner {
         uint32_t x = s - base[slot_ctx[s]];
         const uint64_t cap = grown_cap(need);
         unsigned long long *nt = (unsigned long long *)alloc_for(c, cap * 8);
+        uint2 *nv = nullptr;
+        try {
+            if (c->hval[x]) nv = (uint2 *)alloc_for(c, cap * 8);
+        } catch (...) {
+            c->dfree(nt, cap * 8);
+            throw;
+        }
         ck(cudaMemsetAsync(nt, 0xFF, cap * 8, st), "memset");
-        uint2 *nv = c->hval[x] ? (uint2 *)alloc_for(c, cap * 8) : nullptr;
         prof.run(KID_REHASH, [&] {
             launch_rehash(c->htab[x], c->hval[x], c->hcap[x], nt, nv, cap,
                           &d_cnt.p->overflow, sms, st);

@@ -314,6 +314,8 @@ void launch_iter_end(const SlotTab &S, const InstTab &I, const WorkBufs &W, Loop
         g_overflow = 0;
         W.cnt->cand = W.cand_cap + 1;
         for (int b = 0; b < N_BINS; b++) W.cnt->groups[b] = W.group_cap[b] + 1;
+        for (uint32_t s = 0; s < n_slots; s++) S.cand[s] = S.hmask[s];
+        for (uint32_t k = 0; k < n_inst; k++) I.pool_top[k] = I.pool_cap[k] + 1;
         return;
     }
     const int par = *W.parity;
@@ -354,6 +356,24 @@ void launch_clear_sets(const SlotTab &, uint32_t, unsigned long long, int, cudaS
 }
 void launch_clear_rows(uint4 *, uint2 *, uint32_t *, uint32_t, uint32_t, int, cudaStream_t st) {
     launch("clear_rows", st);
+}
+void launch_rehash(const unsigned long long *old_tab, const uint2 *old_val,
+                   unsigned long long old_cap, unsigned long long *new_tab, uint2 *new_val,
+                   unsigned long long new_cap, unsigned *, int, cudaStream_t st) {
+    launch("rehash", st);
+    arg("rehash from", old_tab, old_cap, st);
+    arg("rehash to", new_tab, new_cap, st);
+    expect(!old_val == !new_val, "rehash: witnesses");
+    if (old_val) arg("rehash from", old_val, old_cap, st);
+    if (new_val) arg("rehash to", new_val, new_cap, st);
+}
+unsigned long long set_chunks(unsigned long long cap, int) { return cap / 1024; }
+void launch_rehash_many(const GrownSet *sets, uint32_t count, unsigned long long,
+                        unsigned long long, unsigned *err, int sms, cudaStream_t st) {
+    arg("grown sets", sets, count + 1, st);
+    for (uint32_t k = 0; k < count; k++)
+        launch_rehash(sets[k].old_tab, sets[k].old_val, sets[k].old_cap, sets[k].new_tab,
+                      sets[k].new_val, sets[k].new_cap, err, sms, st);
 }
 void launch_permute_ids(uint32_t *, unsigned long long, const uint32_t *, int, cudaStream_t st) {
     launch("permute_ids", st);
@@ -624,7 +644,39 @@ void budget_after_failed_readouts() {
     g_pairs = few;
 }
 
+// Growths of the pair sets and of the row pool that run out of memory at each
+// allocation in turn (sets one at a time under a budget, together without one):
+// nothing stays allocated once the contexts are gone, and the next graph works.
+void failed_growths() {
+    for (unsigned bits : {OVF_HASH, OVF_POOL}) {
+        for (int witness = 0; witness < 2; witness++) {
+            for (int budget = 0; budget < 2; budget++) {
+                int failed = 0, rc = CFLR_ENOMEM;
+                for (uint64_t k = 1; rc != CFLR_OK && k < 50; k++) {
+                    Context x([&](cflr_config &c) {
+                        c.witness = witness;
+                        c.mem_budget_bytes = budget ? 1ull << 32 : 0;
+                    });
+                    expect(x.load() == CFLR_OK, "load");
+                    g_overflow = bits;
+                    g_fail_alloc = from(k);
+                    rc = cflr_solve(x.c, nullptr);
+                    g_fail_alloc = nullptr;
+                    failed += rc == CFLR_ENOMEM;
+                    expect(rc == CFLR_OK || rc == CFLR_ENOMEM, "code");
+                    expect(x.load() == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK,
+                           "next graph");
+                }
+                expect(rc == CFLR_OK && failed >= 1, "allocations reached");
+            }
+        }
+    }
+    for (auto &b : g_blocks)
+        expect(b.second.pinned || !b.second.live, "device memory left allocated");
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"failed_growths", failed_growths},
     {"budget_after_failed_readouts", budget_after_failed_readouts},
     {"readout_without_map", readout_without_map},
     {"failed_batch_tables", failed_batch_tables},
