@@ -1799,9 +1799,14 @@ EdgeScan scan_edges(const Grammar &g, uint32_t n, uint64_t m, const uint32_t *sr
     return out;
 }
 
+// Whether the first pair sets may be larger than the initial pairs need.
+bool roomy_sets(const cflr_config &cfg) {
+    return !cfg.mem_budget_bytes && !cfg.initial_capacity && !cfg.test_fixed_pair_sets;
+}
+
 // Copy the graph to the device and size the matrices (cflr_load_graph).
 void upload_graph(cflr_ctx *c, uint32_t n, uint64_t m, const uint32_t *src, const uint32_t *lab,
-                  const uint32_t *dst, const EdgeScan &scan) {
+                  const uint32_t *dst, const EdgeScan &scan, bool roomy) {
     const Grammar &g = c->g;
     const uint32_t nt = (uint32_t)g.nts.size(), nterm = (uint32_t)g.terms.size();
     cudaStream_t st = c->stream;
@@ -1886,14 +1891,12 @@ void upload_graph(cflr_ctx *c, uint32_t n, uint64_t m, const uint32_t *src, cons
     c->hval.assign(nt, nullptr);
     c->hcap.assign(nt, 0);
     c->nnz.assign(nt, 0);
-    // First capacities.  Without a budget or a test's sizes the named
-    // non-terminals share 64 MB (at most 512 KB each): clearing that costs
-    // 10 us, and a set that starts at 1024 entries grows two or three times,
-    // each a wait of the solve (618 growths of the 61k-vertex points-to
-    // solve).  One allocation then holds all first tables; one that grows
-    // leaves its place in it unused (an eighth of its new size at most).
-    const bool roomy =
-        !c->cfg.mem_budget_bytes && !c->cfg.initial_capacity && !c->cfg.test_fixed_pair_sets;
+    // First capacities.  Roomy, the named non-terminals share 64 MB (at most
+    // 512 KB each): clearing that costs 10 us, and a set that starts at 1024
+    // entries grows two or three times, each a wait of the solve (618 growths of
+    // the 61k-vertex points-to solve).  One allocation then holds all first
+    // tables; one that grows leaves its place in it unused (an eighth of its
+    // new size at most).
     uint64_t least = 1024;
     if (roomy && g.n_named)
         while (least < (1u << 16) && 2 * least * 8 * g.n_named <= (64ull << 20)) least *= 2;
@@ -2163,10 +2166,20 @@ int cflr_load_graph(cflr_ctx *c, uint32_t n_vertices, uint64_t n_edges, const ui
     try {
         Range range("cflr_load_graph");
         ck(cudaSetDevice(c->device), "cudaSetDevice");
-        c->free_graph();
-        c->state = ST_GRAMMAR;
-        upload_graph(c, n_vertices, n_edges, src, label, dst, scan);
-        reset_matrices(c);
+        auto build = [&](bool roomy) {
+            c->free_graph();
+            c->state = ST_GRAMMAR;
+            upload_graph(c, n_vertices, n_edges, src, label, dst, scan, roomy);
+            reset_matrices(c);
+        };
+        const bool roomy = roomy_sets(c->cfg);
+        try {
+            build(roomy);
+        } catch (const Status &s) {
+            // a device that is nearly full: without the room to grow
+            if (s.code != CFLR_ENOMEM || !roomy) throw;
+            build(false);
+        }
         c->state = ST_GRAPH;
         c->err.clear();
         return CFLR_OK;

@@ -552,7 +552,7 @@ void failed_buffers() {
                     expect(x.load() == CFLR_OK, "load");
                     g_overflow = OVF_CAND | OVF_GROUPS;
                 }
-                g_fail_alloc = nth(k);
+                g_fail_alloc = from(k);
                 // (100,000 edges: more initial pairs than the first buffers hold)
                 rc = solving ? cflr_solve(x.c, nullptr) : x.load(5000, 100000);
                 g_fail_alloc = nullptr;
@@ -675,7 +675,30 @@ void failed_growths() {
         expect(b.second.pinned || !b.second.live, "device memory left allocated");
 }
 
+// A device without room for roomy first pair sets, or for the rest of a load
+// beside them: the load takes small ones.
+void load_without_roomy_sets() {
+    const size_t sets = 3 * (512u << 10);         // of the three named non-terminals
+    for (int beside = 0; beside < 2; beside++) {
+        Context x;
+        int failed = 0, seen = 0;
+        g_fail_alloc = [&](size_t bytes) {
+            seen += bytes == sets;
+            bool fail = bytes == sets && !beside;
+            if (beside)
+                for (auto &b : g_blocks) fail |= b.second.n == sets && b.second.live;
+            failed += fail;
+            return fail;
+        };
+        expect(x.load() == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "small first sets");
+        g_fail_alloc = nullptr;
+        expect(seen == 1 && failed == 1, "one allocation failed");
+        expect(x.load() == CFLR_OK && cflr_solve(x.c, nullptr) == CFLR_OK, "with room again");
+    }
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"load_without_roomy_sets", load_without_roomy_sets},
     {"failed_growths", failed_growths},
     {"budget_after_failed_readouts", budget_after_failed_readouts},
     {"readout_without_map", readout_without_map},

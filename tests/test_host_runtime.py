@@ -34,7 +34,8 @@ def program(tmp_path_factory):
 @pytest.mark.parametrize("scenario", ["batch_across_streams", "failed_readouts",
                                       "failed_products", "failed_buffers",
                                       "failed_batch_tables", "readout_without_map",
-                                      "budget_after_failed_readouts", "failed_growths"])
+                                      "budget_after_failed_readouts", "failed_growths",
+                                      "load_without_roomy_sets"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout[-4000:] + r.stderr[-2000:]
