@@ -139,8 +139,9 @@ typedef struct {
  * products, or products alone when it probes the pair set instead of
  * loading the mask row, which it does when mask_len > probe_ratio *
  * products); bin 3 takes the rest with an n-bit bitmap, and also the groups of
- * bins 1 and 2 whose hash table would be no smaller than that bitmap (not
- * those with several output non-terminals).  Limits must
+ * bins 1 and 2 whose hash table would be no smaller than that bitmap is for
+ * the batch's graph of the most vertices (not those with several output
+ * non-terminals).  Limits must
  * increase and stay within 128, 1024 and 4096 (the bins' table sizes). */
 typedef struct {
     uint32_t probe_ratio;       /* >= 1                                             */

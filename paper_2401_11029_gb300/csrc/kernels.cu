@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
     // members write different non-terminals probe their pair sets (there is
     // no single mask row) and stay in the hash bins (force_probe).
     bool acct = true;   // whether this lane adds the group's work and bytes
-    auto classify = [&](uint32_t code, uint32_t part, uint32_t idx, uint32_t n, uint32_t d,
+    auto classify = [&](uint32_t code, uint32_t part, uint32_t idx, uint32_t d,
                         uint32_t mlen, unsigned long long mbytes, unsigned long long f,
                         unsigned long long fbytes, bool force_probe, uint2 &grp) -> int {
         const bool probe =
@@ -589,12 +589,18 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
         uint32_t lg = 5;
         while (b < 3 && (1ull << lg) < 2 * need) lg++;
         // A group of bins 1 and 2 whose table (8 bytes a slot) would be no
-        // smaller than the row's bitmap takes the bitmap: a tile then costs
-        // one shared-memory read instead of a probe sequence.  (Groups of
-        // bin 0 stay: a few tiles on one warp.)  With bin 1 on two warps a
-        // group, this took the 200k alias solve from 48.9 to 44.8 ms, the 100k
-        // one from 22.8 to 19.9 and the 20k one from 10.4 to 9.7.
-        if ((b == 1 || b == 2) && !force_probe && (n + 31) / 32 <= 2ull << lg) b = 3;
+        // smaller than a bitmap of the batch's widest row takes the bitmap: a
+        // tile then costs one shared-memory read instead of a probe sequence.
+        // (Groups of bin 0 stay: a few tiles on one warp.)  With bin 1 on two
+        // warps a group, this took the 200k alias solve from 48.9 to 44.8 ms,
+        // the 100k one from 22.8 to 19.9 and the 20k one from 10.4 to 9.7.
+        // The widest row, because bin 3's launch is laid out for it: going by
+        // its own instance's rows, a 20k-vertex group beside a 500k-vertex
+        // instance runs three to an SM, and beside a 2M-vertex one on a bitmap
+        // in global memory (8 20k alias graphs solved with the 500k points-to
+        // graph 151.5 ms, now 146.7; with a sparse 2M-vertex one 29.2, now
+        // 26.2; with the 200k alias graph 48.3, now 48.0).
+        if ((b == 1 || b == 2) && !force_probe && (uint32_t)W.bitmap_words <= 2u << lg) b = 3;
         grp = make_uint2(((code >> 2) << 8) | (lg << 3) | (probe ? MODE_PROBE : 0u) | part, idx);
         // algorithmic bytes: the delta entries (4 B each), the descriptor
         // (16 B) and tiles (8 B each) of every referenced row, and the mask
@@ -656,11 +662,11 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                     uint2 grp;
                     if (fm.z & FAM_CSHARED) {   // every member writes c: one mask row
                         const uint32_t mt = S.desc[pr0.x][r].y;
-                        emit(classify(code, PART_F, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false,
+                        emit(classify(code, PART_F, idx, d, mt, 8ull * mt, wk.f, wk.fb, false,
                                       grp),
                              grp);
                     } else if (wk.f <= T.limit[2]) {
-                        emit(classify(code, PART_F, idx, n, d, 0, 0, wk.f, wk.fb, true, grp), grp);
+                        emit(classify(code, PART_F, idx, d, 0, 0, wk.f, wk.fb, true, grp), grp);
                     } else {
                         // too large for a hash bin: one group per member,
                         // the threads taking the members
@@ -672,7 +678,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                             uint2 mg = make_uint2(0, 0);
                             if (i < fm.y && mf[i]) {
                                 const uint32_t mt = S.desc[P.prod[mp[i]].x][r].y;
-                                b = classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt,
+                                b = classify((mp[i] << 2) | fm.w, fm.w, idx, d, mt, 8ull * mt,
                                              mf[i], 16ull * mc[i] + 8ull * mf[i], false, mg);
                             }
                             if (cta) {
@@ -704,9 +710,9 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
             uint2 grp;
             if (fm.z & FAM_CSHARED) {   // every member writes c: one mask row
                 const uint32_t mt = S.desc[pr0.x][r].y;
-                emit(classify(code, PART_F, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
+                emit(classify(code, PART_F, idx, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
             } else if (wk.f <= T.limit[2]) {
-                emit(classify(code, PART_F, idx, n, d, 0, 0, wk.f, wk.fb, true, grp), grp);
+                emit(classify(code, PART_F, idx, d, 0, 0, wk.f, wk.fb, true, grp), grp);
             } else if (qstep == 32) {
                 // too large for a hash bin: one group per member; with a
                 // whole warp on the use, the lanes take the members (each
@@ -723,7 +729,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                         const Work wi = gathered_work(S, (fm.w == PART_A) ? pr.z : pr.y, o, n,
                                                       pool, dstart, d, 0, 1, &W.cnt->overflow);
                         if (wi.f)
-                            b = classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt, wi.f,
+                            b = classify((mp[i] << 2) | fm.w, fm.w, idx, d, mt, 8ull * mt, wi.f,
                                          wi.fb, false, mg);
                     }
                     stage_lanes(b, mg);
@@ -735,7 +741,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                                                       q0, qstep, &W.cnt->overflow));
                     if (wi.f == 0) continue;
                     const uint32_t mt = S.desc[P.prod[mp[i]].x][r].y;
-                    emit(classify((mp[i] << 2) | fm.w, fm.w, idx, n, d, mt, 8ull * mt, wi.f, wi.fb,
+                    emit(classify((mp[i] << 2) | fm.w, fm.w, idx, d, mt, 8ull * mt, wi.f, wi.fb,
                                   false, grp),
                          grp);
                 }
@@ -755,7 +761,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
         }
         if (wk.f == 0) return;
         uint2 grp;
-        emit(classify(code, part, idx, n, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
+        emit(classify(code, part, idx, d, mt, 8ull * mt, wk.f, wk.fb, false, grp), grp);
     };
 
     if constexpr (MODE == 1) {
@@ -875,7 +881,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
             // the group of a use with its sums: staged, or left to warp_use
             // (true) when a family splits into its members; lanes without a
             // use to finish pass lead = false
-            auto finish = [&](bool lead, uint4 rec, uint32_t idx, uint32_t n, uint32_t d,
+            auto finish = [&](bool lead, uint4 rec, uint32_t idx, uint32_t d,
                               uint32_t mtiles, unsigned long long f, uint32_t cnt) -> bool {
                 int b = -1;
                 uint2 grp = make_uint2(0, 0);
@@ -887,7 +893,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                         split = true;
                     } else {
                         acct = true;
-                        b = classify(rec.x, part, idx, n, d, mtiles, 8ull * mtiles, f,
+                        b = classify(rec.x, part, idx, d, mtiles, 8ull * mtiles, f,
                                      part == PART_U ? 4ull * d : 16ull * cnt + 8ull * f, tagged,
                                      grp);
                     }
@@ -1051,7 +1057,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                         }
                     }
                 }
-                slow |= finish(lead && !slow, rec, idx, n, d, mtiles, f, cnt);
+                slow |= finish(lead && !slow, rec, idx, d, mtiles, f, cnt);
                 for (unsigned sm = __ballot_sync(FULL_MASK, slow && lead); sm; sm &= sm - 1) {
                     const int q = __ffs(sm) - 1;
                     warp_use(__shfl_sync(FULL_MASK, rec.x, q), __shfl_sync(FULL_MASK, xo, q),

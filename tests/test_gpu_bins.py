@@ -48,3 +48,31 @@ def test_families_in_narrow_bins(limits):
         got = s.pairs_many(["PT", "FT"])
         for x in ("PT", "FT"):
             assert np.array_equal(got[x], want.pairs[x]), x
+
+
+@pytest.mark.parametrize("n_wide", [32 * 16384 + 1, 32 * 51200 + 1])
+def test_a_small_instance_beside_a_wide_one(n_wide):
+    """The bitmap bin's launch is laid out for the batch's widest rows (beyond
+    51200 words its bitmaps are in global memory): beside them the groups of a
+    small instance keep their hash tables."""
+    text = gen.grammar_text("fica")
+    small = gen.fica_like(n=3000, n_a=6000, n_d=2250, seed=7)
+    wide = gen.fica_like(n=300, n_a=600, n_d=225, seed=8)
+    wide = padded(wide, n_wide)
+    want = [oracle.solve(text, g) for g in (small, wide)]
+    solvers = [Solver(text, form=cflr.CFLR_FORM_GRAPH) for _ in want]
+    try:
+        for s, g in zip(solvers, (small, wide)):
+            s.load(g)
+        alone = solvers[0].solve()["groups"]
+        assert alone[1] == alone[2] == 0 and alone[3] > 0
+        for s in solvers:
+            cflr.cflr_reset(s.ctx)
+        beside = cflr.cflr_solve_batch([s.ctx for s in solvers])[0]["groups"]
+        assert beside[1] > 0
+        for s, w in zip(solvers, want):
+            for name in w.grammar.nts[:w.grammar.n_user]:
+                assert np.array_equal(s.pairs(name), w.pairs[name]), name
+    finally:
+        for s in solvers:
+            s.close()
