@@ -431,7 +431,7 @@ __device__ __forceinline__ void family_members(const SlotTab &S, uint32_t g0, ui
         for (int t = 0; t < 4; t++) {
             const uint32_t q = qb + nth * t + tid;
             k[t] = q < d ? pool[dstart + q] : 0u;
-            if (!CFLR_CHECK(k[t] < n, err)) k[t] = d;   // skipped below
+            if (!CFLR_CHECK(k[t] < n, err)) k[t] = EMPTY32;   // skipped below
         }
 #pragma unroll
         for (int t = 0; t < 4; t++) {
