@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                 const uint4 pr = P.prod[mp[i]];
                 return (fm.w == PART_A) ? pr.z : pr.y;
             };
-            if ((fm.z & FAM_CONSEC) && (qstep == 32 || qstep == 256) && fm.y <= 64) {
+            if (fm.y <= 64) {
                 // a whole warp (or CTA) on the use: per-member sums first,
                 // then the family's group, or one group per member
                 const bool cta = qstep == 256;
@@ -693,19 +693,8 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                 group_sync();
                 return;
             }
-            Work wk{0, 0};
-            if (fm.z & FAM_CONSEC) {
-                wk = family_work(S, g0, fm.y, o, n, pool, dstart, d, q0, qstep,
-                                 &W.cnt->overflow);
-            } else {
-                for (uint32_t i = 0; i < fm.y; i++) {
-                    const Work wi = gathered_work(S, member_slot(i), o, n, pool, dstart, d, q0,
-                                                  qstep, &W.cnt->overflow);
-                    wk.f += wi.f;
-                    wk.fb += wi.fb;
-                }
-            }
-            wk = sum(wk);
+            const Work wk = sum(family_work(S, g0, fm.y, o, n, pool, dstart, d, q0, qstep,
+                                            &W.cnt->overflow));
             if (wk.f == 0) return;
             uint2 grp;
             if (fm.z & FAM_CSHARED) {   // every member writes c: one mask row
@@ -831,7 +820,7 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
             }
             const int rows = __popc(__ballot_sync(FULL_MASK, has));   // the first lanes
             // a use of a row by the whole warp, which shares the entries:
-            // wide or scattered families, and families that split
+            // families of more than 64 members, and families that split
             auto warp_use = [&](uint32_t code, uint32_t xo, uint32_t idx, uint32_t dstart,
                                 uint32_t d) {
                 acct = lane == 0;
@@ -840,8 +829,8 @@ __global__ void __launch_bounds__(256, 3) k_symbolic(SlotTab S, ProdTab P, WorkB
                            [&](int bb, uint2 g) { stage_lanes(lane == 0 ? bb : -1, g); });
             };
             // product steps f and referenced rows cnt of entry k under `rec`
-            // (narrow: at most 64 members on consecutive slots; the slots of
-            // an instance follow one another, and so do their descriptors, 2n
+            // (at most 64 members, on consecutive slots; the slots of an
+            // instance follow one another, and so do their descriptors, 2n
             // each), the members' descriptors four at a time
             auto entry_work = [&](uint4 rec, uint32_t slot, uint32_t o, uint32_t n,
                                   const uint4 *db, uint32_t k, unsigned long long &f,
@@ -1086,9 +1075,8 @@ struct GroupInfo {
     bool probe;
     // family groups: member i is production P.fam_prod[first + i]; `tagged`
     // when the members write different non-terminals (accumulator keys
-    // carry the member); `consec` when the slots of their other operand are
-    // consecutive.  A plain group has first = its production.
-    bool fam, tagged, consec;
+    // carry the member).  A plain group has first = its production.
+    bool fam, tagged;
     uint32_t first, F;
 };
 
@@ -1102,7 +1090,6 @@ __device__ __forceinline__ GroupInfo decode_group(const ProdTab &P, const SlotTa
     gi.part = g.x & 3;
     gi.fam = gi.part == PART_F;
     gi.tagged = false;
-    gi.consec = false;
     gi.first = g.x >> 8;
     gi.F = 1;
     uint32_t p0 = gi.first;
@@ -1112,7 +1099,6 @@ __device__ __forceinline__ GroupInfo decode_group(const ProdTab &P, const SlotTa
         gi.first = fm.x;
         gi.F = fm.y;
         gi.tagged = (fm.z & FAM_CSHARED) == 0;
-        gi.consec = (fm.z & FAM_CONSEC) != 0;
         p0 = P.fam_prod[fm.x];
     }
     const uint4 pr = P.prod[p0];
@@ -1157,7 +1143,7 @@ __device__ __forceinline__ GroupMeta group_meta(const ProdTab &P, const SlotTab 
     const GroupInfo gi = decode_group(P, S, g);
     GroupMeta m;
     m.bits = gi.part | (gi.probe ? 4u : 0u) | (gi.fam ? 8u : 0u) | (gi.tagged ? 16u : 0u) |
-             (gi.consec ? 32u : 0u) | gi.lg << 8;
+             gi.lg << 8;
     m.idx = gi.idx;
     m.c = gi.c;
     m.a = gi.a;
@@ -1185,7 +1171,6 @@ __device__ __forceinline__ GroupInfo group_info(const GroupMeta &m) {
     gi.probe = m.bits & 4;
     gi.fam = m.bits & 8;
     gi.tagged = m.bits & 16;
-    gi.consec = m.bits & 32;
     gi.lg = m.bits >> 8;
     gi.o = gi.part == PART_B ? 1u : 0u;
     gi.idx = m.idx;
@@ -1220,12 +1205,11 @@ __device__ __forceinline__ unsigned long long group_key(const GroupInfo &gi, uin
 // last merge's (dn.y of them, at the end of the list).
 //   Plain groups: warp `warp_id` of `nwarps` takes an even share of the
 // entries, 32 consecutive ones at a time (lane l the l-th).
-//   Family groups (optimisation 4): when the members' gathered slots are
-// consecutive, the same shares of the entries, each entry's members found
-// from its occupancy bits; otherwise warp `warp_id` takes the (entry, member)
-// items warp_id*32 + l of every block of nwarps*32.  A member's row counts
-// only when its occupancy bit is set.  Tagged families key the accumulator
-// by member and word, and emit to each member's non-terminal.
+//   Family groups (optimisation 4): the same shares of the entries (of the
+// entries' occupancy words, for more than 64 members), each entry's members
+// found from its occupancy bits (the members' gathered slots are
+// consecutive).  Tagged families key the accumulator by member and word, and
+// emit to each member's non-terminal.
 // The 32 tile lists the lanes hold are walked together as one packed
 // sequence (see `walk_packed`) or list by list.  Returns the emitted count.
 
@@ -1505,7 +1489,7 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
         }
         return emitted;
     }
-    if (gi.fam && gi.consec && gi.F <= 64) {
+    if (gi.fam && gi.F <= 64) {
         // the (entry, member) pairs whose member has a row, packed 32 per
         // step: lane l takes entry l of a block of 32, its members' occupancy
         // bits become a 64-bit mask, and a warp scan numbers the pairs
@@ -1565,7 +1549,7 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
         }
         return emitted;
     }
-    if (gi.fam && gi.consec) {
+    if (gi.fam) {
         // more than 64 members: a lane per (entry, occupancy word) item, 32
         // at a time, numbered entry * words + word; the set bits of the words
         // are the (entry, member) pairs that have a row, packed 32 per step
@@ -1618,34 +1602,6 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
                 }
                 walk(toff, tn, tag, o_k);
             }
-        }
-        return emitted;
-    }
-    if (gi.fam) {
-        // members on scattered slots: the (entry, member) pairs numbered
-        // entry * F + member, 32 per warp step; a member's row counts when its occupancy bit is set
-        const unsigned long long items = (unsigned long long)d * gi.F;
-        for (unsigned long long ib = (unsigned long long)warp_id * 32; ib < items;
-             ib += (unsigned long long)nwarps * 32) {
-            const unsigned long long it = ib + lane;
-            uint32_t toff = 0, tn = 0, tag = 0, k = 0;
-            if (it < items) {
-                const uint32_t e = (uint32_t)(it / gi.F), i = (uint32_t)(it - (unsigned long long)e * gi.F);
-                k = pool[dstart + e];
-                const uint4 pr = P.prod[P.fam_prod[gi.first + i]];
-                const uint32_t gs = (gi.part == PART_A) ? pr.z : pr.y;
-                const uint32_t lx = S.local[gs];
-                if (CFLR_CHECK(k < gi.n, &W.cnt->overflow) &&
-                    ((S.occ[gs][(oo + k) * S.occ_w[gs] + (lx >> 5)] >> (lx & 31)) & 1u)) {
-                    const uint4 gd = S.desc[gs][oo + k];
-                    if (row_in_pool(S, gs, gd, &W.cnt->overflow)) {
-                        toff = gd.x;
-                        tn = gd.y - (gi.o ? (gd.w & DLAST_MASK) : 0u);
-                        tag = i;
-                    }
-                }
-            }
-            walk(toff, tn, tag, k);
         }
         return emitted;
     }

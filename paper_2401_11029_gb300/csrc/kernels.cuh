@@ -134,16 +134,16 @@ struct ProdTab {              // global production table of the batch
     // families run as one block product (optimisation 4):
     // {offset into fam_prod, members F, flags, part of the shared operand
     // (PART_A: a shared, PART_B: b shared)}; member i is production
-    // fam_prod[offset + i].  Flags: FAM_CSHARED when every member writes the
-    // same c, FAM_CONSEC when the slots of the members' other operand are
-    // consecutive (so are their occupancy bits)
+    // fam_prod[offset + i], and the slots of the members' other operand are
+    // consecutive (so are their occupancy bits).  Flag: FAM_CSHARED when every
+    // member writes the same c
     const uint4 *fam;
     const uint32_t *fam_prod;
 };
-constexpr uint32_t FAM_CSHARED = 1, FAM_CONSEC = 2;
+constexpr uint32_t FAM_CSHARED = 1;
 constexpr uint32_t USE_MEMBERS = 0xFFFFu;     // use_rec.w: members (1: one production)
 constexpr uint32_t USE_SHARED = 1u << 16;     // a family whose members write one c
-constexpr uint32_t USE_NARROW = 1u << 17;     // a family of at most 64 consecutive slots
+constexpr uint32_t USE_NARROW = 1u << 17;     // a family of at most 64 members
 
 struct Counters {
     unsigned long long groups[N_BINS];

@@ -581,20 +581,16 @@ struct Runner {
             std::vector<std::array<char, 2>> covered(g.bin_c.size(), {0, 0});
             // A family runs as one block product on the delta of the operand
             // its members share (one work-list use instead of F):
-            // {offset into fam_prod, F, 1 if every member writes one c | 2
-            // if the other operand's slots are consecutive, part}.
+            // {offset into fam_prod, F, FAM_CSHARED if every member writes one
+            // c, part}.
             auto add_family = [&](const std::vector<int> &m, int side, bool sc) {
                 const uint32_t F = (uint32_t)m.size(), off = (uint32_t)fam_prod.size();
-                bool consecutive = true;
                 for (uint32_t i = 0; i < F; i++) {
                     fam_prod.push_back(pid[m[i]]);
                     covered[m[i]][side] = 1;
-                    const uint32_t gi = side == 0 ? g.bin_b[m[i]] : g.bin_a[m[i]];
-                    const uint32_t g0 = side == 0 ? g.bin_b[m[0]] : g.bin_a[m[0]];
-                    consecutive &= gi == g0 + i;
                 }
                 const uint32_t fid = (uint32_t)fams.size();
-                fams.push_back(make_uint4(off, F, (sc ? 1u : 0u) | (consecutive ? 2u : 0u),
+                fams.push_back(make_uint4(off, F, sc ? FAM_CSHARED : 0u,
                                           side == 0 ? PART_A : PART_B));
                 const uint32_t x = side == 0 ? g.bin_a[m[0]] : g.bin_b[m[0]];
                 uses[(size_t)(b0 + x) * 2 + side].push_back(fid << 2 | PART_F);
@@ -654,7 +650,7 @@ struct Runner {
                 const uint4 pr = prods[fam ? fam_prod[fm.x] : code >> 2];
                 uint32_t w = fm.y;
                 if (fm.z & FAM_CSHARED) w |= USE_SHARED;
-                if ((fm.z & FAM_CONSEC) && fm.y <= 64) w |= USE_NARROW;
+                if (fam && fm.y <= 64) w |= USE_NARROW;
                 out.recs.push_back(make_uint4(code, pr.x, fm.w == PART_A ? pr.z : pr.y, w));
             }
             out.off.push_back((uint32_t)out.recs.size());
