@@ -1399,11 +1399,11 @@ __device__ __forceinline__ uint32_t expand_rows(const SlotTab &S, const ProdTab 
     // Segments start on 16-byte boundaries and a tile section holds an even
     // number of tiles, so a 16-byte half of a quad that holds a tile never
     // leaves its section; what a list does not fill of its last quad is zeroed.
-    // The accumulator is read for all of a lane's tiles before any is added: nearly every product is already present, so the reads overlap and
-    // one vote decides whether anything follows.  (Finding a list's owner for
-    // every 16-byte pair and testing a tile at a time, 38 instructions per
-    // warp and 32 tiles, bin 3 took 19.5 ms of the 200k alias solve; now
-    // 14.8.)
+    // The accumulator is read for all of a lane's tiles before any is added:
+    // nearly every product is already present, so the reads overlap and one
+    // vote decides whether anything follows.  (Finding a list's owner for every
+    // 16-byte pair and testing a tile at a time, 38 instructions per warp and
+    // 32 tiles, bin 3 took 19.5 ms of the 200k alias solve; now 14.8.)
     auto walk_packed = [&](uint32_t toff, uint32_t tn, uint32_t tag, uint32_t k) {
         constexpr int U = WALK_U / 2;
         const unsigned nz = __ballot_sync(FULL_MASK, tn != 0);
@@ -2732,9 +2732,10 @@ __global__ void k_fill_u64(unsigned long long *p, unsigned long long count,
 // for large sets and by the launch for small ones: a fill per set cost 4 us
 // each on the host (1539 sets of the 100k-vertex value-flow graph: with this
 // and k_clear_rows its reset-solve-read pass went from 14.7 to 8.6 ms, the
-// field-sensitive alias pass from 13.7 to 12.2 ms).  The sets are cut into chunks of CLEAR_CHUNK entries, numbered over
-// all sets; every block finds the sets of its chunks itself, from a scan of
-// CLEAR_SEG slots' chunk counts at a time, so the host prepares no table.
+// field-sensitive alias pass from 13.7 to 12.2 ms).  The sets are cut into
+// chunks of CLEAR_CHUNK entries, numbered over all sets; every block finds the
+// sets of its chunks itself, from a scan of CLEAR_SEG slots' chunk counts at a
+// time, so the host prepares no table.
 constexpr uint32_t CLEAR_SEG = 2048;     // slots scanned at a time, 8 a thread
 
 __global__ void __launch_bounds__(256) k_clear_sets(SlotTab S, uint32_t n_slots) {
@@ -3676,9 +3677,8 @@ void launch_capacity_big(const SlotTab &S, const InstTab &I, const WorkBufs &W, 
     set_smem_attrs();
     const size_t bm_bytes = (size_t)((max_n + 31) / 32) * 4;
     const bool sm = bm_bytes <= SMEM_BITMAP_MAX;
-    int per_sm = sm ? (int)((220 * 1024) / (bm_bytes + 3072)) : 8;
-    per_sm = per_sm < 1 ? 1 : (per_sm > 8 ? 8 : per_sm);
-    per_sm = per_sm > 2 ? 2 : per_sm;      // few rows are that long
+    int per_sm = sm ? (int)((220 * 1024) / (bm_bytes + 3072)) : 2;
+    per_sm = per_sm < 1 ? 1 : (per_sm > 2 ? 2 : per_sm);   // few rows are that long
     launch_after(k_capacity_big, sms * per_sm, sm ? bm_bytes : 0, st, S, I, W, sm ? 1 : 0);
 }
 

@@ -147,8 +147,9 @@ constexpr uint32_t USE_NARROW = 1u << 17;     // a family of at most 64 members
 
 struct Counters {
     unsigned long long groups[N_BINS];
-    unsigned long long claim[N_BINS + 1];   // next group of the bin to take (CTA-level bins);
-                                        // last: next batch of rows of k_symbolic
+    unsigned long long claim[N_BINS + 1];   // next group of the bin to take (bin 0: next
+                                        // batch of groups); last: next batch of rows of
+                                        // k_symbolic
     unsigned long long cand;
     unsigned long long delta;
     unsigned long long flops;

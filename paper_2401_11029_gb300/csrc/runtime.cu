@@ -806,8 +806,8 @@ struct Runner {
         std::memset(h + o_delta, 0, off_end - o_delta);
         fill_htabs();
         fill_pools();
-        // loop state, with every counter zero: parity 0, the pending delta rows (import_touched brings
-        // them), iteration count 0
+        // loop state, with every counter zero: parity 0, the pending delta rows
+        // (import_touched brings them), iteration count 0
         *h_ctl = LoopCtl{};
         h_ctl->limit = own->cfg.max_iterations ? own->cfg.max_iterations : 0xFFFFFFFFu;
         h_ctl->stop_on_converge = own->cfg.stop_on_first_converged ? 1u : 0u;
@@ -970,7 +970,7 @@ struct Runner {
         if (max_n > 200 * 1024 * 8) {   // bitmaps do not fit shared memory
             uint64_t words = (max_n + 31) / 32;
             d_bitmap.ensure(own, words * (uint64_t)sms * 8);
-            }
+        }
     }
 
     static constexpr uint64_t GROWN_TOGETHER = 1ull << 21;   // entries: 16 MB

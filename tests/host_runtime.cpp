@@ -289,7 +289,8 @@ void launch_symbolic(const SlotTab &, const ProdTab &P, const WorkBufs &W, int, 
     launch("symbolic", st);
     check_work("symbolic", W, st);
     arg("use_off", P.use_off, 1, st);
-    if (P.use_off && block_of(P.use_off)) expect(P.use_off[0] == 0, "production tables not written");
+    if (P.use_off && block_of(P.use_off))
+        expect(P.use_off[0] == 0, "production tables not written");
 }
 void launch_spgemm(int bin, const SlotTab &, const ProdTab &, const WorkBufs &W, uint32_t,
                    const Tuning &, int, cudaStream_t st) {
@@ -383,7 +384,8 @@ void launch_remap_touched(const uint2 *in, unsigned long long n, uint32_t slot_b
     launch("remap_touched", st);
     arg("remap: a context's delta rows", in, n, st);
     arg("remap: the batch's delta rows", out, n, st);
-    for (unsigned long long q = 0; q < n; q++) out[q] = make_uint2(in[q].x + 2 * slot_base, in[q].y);
+    for (unsigned long long q = 0; q < n; q++)
+        out[q] = make_uint2(in[q].x + 2 * slot_base, in[q].y);
 }
 void extract_plan(uint32_t count, uint32_t n, const uint64_t *, int, uint32_t *rows_per,
                   unsigned long long *first) {
