@@ -1457,7 +1457,9 @@ struct Runner {
             c->touched_n = n_in;
             ck(cudaMemcpyAsync(c->touched, d_touched[par].p, n_in * sizeof(uint2),
                                cudaMemcpyDeviceToDevice, st), "D2D touched");
-            if (c->stream != st) {
+            // (cudaStreamPerThread is one handle for a stream of every thread:
+            // what follows may come from another thread)
+            if (c->stream != st || st == cudaStreamPerThread) {
                 sync("export copy");
             } else {        // no wait here: what follows on this stream is ordered, and
                             // import_touched orders another stream's read

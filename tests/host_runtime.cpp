@@ -81,7 +81,17 @@ void merge(Clock &a, const Clock &b) {
 }
 bool covers(const Clock &c, Mark m) { return m.stream < c.size() && c[m.stream] >= m.seq; }
 
-Stream *of(cudaStream_t s) { return (Stream *)s; }
+Stream *of(cudaStream_t s) {
+    if (s != cudaStreamPerThread) return (Stream *)s;
+    // (the one of the only thread here)
+    static Stream *mine = nullptr;
+    if (!mine) {
+        if (g_streams.empty()) g_streams.push_back(nullptr);
+        mine = new Stream{g_streams.size(), {}};
+        g_streams.push_back(mine);
+    }
+    return mine;
+}
 Mark enqueue(cudaStream_t st) {
     Stream *s = of(st);
     merge(s->seen, g_host);
@@ -699,7 +709,17 @@ void load_without_roomy_sets() {
     }
 }
 
+// cudaStreamPerThread is another stream in every thread, though one handle: the
+// next call may come from another thread, so nothing may be pending.
+void per_thread_stream() {
+    Context x([](cflr_config &c) { c.stream = cudaStreamPerThread; });
+    expect(x.load() == CFLR_OK && idle(cudaStreamPerThread), "pending after a load");
+    expect(cflr_solve(x.c, nullptr) == CFLR_OK && idle(cudaStreamPerThread), "after a solve");
+    expect(cflr_reset(x.c) == CFLR_OK && idle(cudaStreamPerThread), "pending after a reset");
+}
+
 const std::map<std::string, void (*)()> SCENARIOS = {
+    {"per_thread_stream", per_thread_stream},
     {"load_without_roomy_sets", load_without_roomy_sets},
     {"failed_growths", failed_growths},
     {"budget_after_failed_readouts", budget_after_failed_readouts},

@@ -35,7 +35,7 @@ def program(tmp_path_factory):
                                       "failed_products", "failed_buffers",
                                       "failed_batch_tables", "readout_without_map",
                                       "budget_after_failed_readouts", "failed_growths",
-                                      "load_without_roomy_sets"])
+                                      "load_without_roomy_sets", "per_thread_stream"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout[-4000:] + r.stderr[-2000:]
